@@ -740,36 +740,37 @@ __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 
 
 // ---- pairwise form (Alg. 3) --------------------------------------------
 
-constexpr int kPairThreads = 128;
-constexpr int kPairPerThread = 2;  // receivers per thread: one packed FP32 pair
-constexpr int kPairTile = kPairThreads * kPairPerThread;
+// Every pair term is sin(x_j - x_i) = sin x_j cos x_i - cos x_j sin x_i, two
+// FMAs on the sines and cosines of the two phases (each within 7e-8, from the
+// fixed-point phases; the kernel that writes a phase writes its pair too).
+// Both products of a term enter the receiver's running sum one after the
+// other, so the sum stays as small as the sum of the sines and rounds like it.
+//
+// What bounds it: the FMA pipe, once the shared loads are kept below it.  Two
+// sources share a packed FP32 FMA (a receiver's sums over even and odd sources
+// are added at the end), so one 128-bit load (s0, s1, -c0, -c1), the same for
+// all lanes, brings two terms' operands already paired for RPT receivers per
+// lane: 2 RPT packed FMAs of 2 cycles on the scheduler's FMA pipe against 4
+// cycles of the SM's shared-memory return path, which four schedulers share.
+// N = 4096, 64 replicas: 76 us per stage launch to launch (54 us of packed FMAs)
+// against 342 us for a polynomial sine per term (9 packed instructions per two
+// terms); N = 1000, 3 replicas: 4.3 us against 23 us.
+//
+// RPT receivers per thread; S slices (warps) of a block take disjoint parts
+// of the sources and their partial sums are added in slice order.
+struct PairShape {
+  int rpt, s;
+  int receivers() const { return rpt * 32; }
+  int threads() const { return 32 * s; }
+};
 
-// acc += sin(phi_j - phi_i) for the thread's two receivers i0, i1 and one
-// source j, all three phases as 32-bit fixed-point turns.  The difference is
-// taken exactly in integers and wraps to [-1/2, 1/2) turn by itself, so no
-// range reduction of a float is needed and no receiver carries the rounding
-// of its own phase into every one of its terms.  With x = d 2^-32 turns and
-// t = 1/4 - ||x| - 1/4| in [0, 1/4] (sin(pi - y) = sin y folds the outer
-// quarters onto the inner ones), sin(2 pi x) = sign(x) sin(2 pi t), and
-// sin(2 pi t) = t (S0 + S1 t^2 + ... + S4 t^8) with S0 the FP32 value of 2 pi;
-// S1..S4 minimise the largest absolute error on a dense grid of [0, 1/4] (a
-// linear program, fitted for this library).  In FP32 the result is within
-// 2.2e-7 of sin(2 pi x) (RMS 6e-8, no bias).  The polynomial runs on packed
-// FP32 pairs, both receivers per instruction, and the special-function unit
-// is not used: its sine's error is systematic enough to move phases by ~1e-5
-// over 10^3 steps of a partly synchronised population.
-__device__ __forceinline__ void pair_terms2(uint32_t tj, uint32_t ti0, uint32_t ti1, float2 &acc) {
-  const float2 x = __fmul2_rn(make_float2((float)(int32_t)(tj - ti0), (float)(int32_t)(tj - ti1)),
-                              make_float2(2.3283064365386963e-10f, 2.3283064365386963e-10f));  // 2^-32
-  const float2 u = __fadd2_rn(make_float2(fabsf(x.x), fabsf(x.y)), make_float2(-0.25f, -0.25f));
-  const float2 t = __fadd2_rn(make_float2(0.25f, 0.25f), make_float2(-fabsf(u.x), -fabsf(u.y)));
-  const float2 t2 = __fmul2_rn(t, t);
-  float2 p = __ffma2_rn(t2, make_float2(3.903203201e+01f, 3.903203201e+01f),
-                        make_float2(-7.653708649e+01f, -7.653708649e+01f));
-  p = __ffma2_rn(p, t2, make_float2(8.160352325e+01f, 8.160352325e+01f));
-  p = __ffma2_rn(p, t2, make_float2(-4.134174728e+01f, -4.134174728e+01f));
-  p = __ffma2_rn(p, t2, make_float2(6.283185482e+00f, 6.283185482e+00f));
-  acc = __ffma2_rn(make_float2(copysignf(t.x, x.x), copysignf(t.y, x.y)), p, acc);
+template <int RPT>
+__device__ __forceinline__ void pair_terms(const float4 &src, const float (&si)[RPT], const float (&ci)[RPT],
+                                           float2 (&acc)[RPT]) {
+#pragma unroll
+  for (int k = 0; k < RPT; ++k) acc[k] = __ffma2_rn(make_float2(src.x, src.y), make_float2(ci[k], ci[k]), acc[k]);
+#pragma unroll
+  for (int k = 0; k < RPT; ++k) acc[k] = __ffma2_rn(make_float2(src.z, src.w), make_float2(si[k], si[k]), acc[k]);
 }
 
 // One SRK2 stage: receivers i of one replica in this CTA, all sources j
@@ -778,74 +779,128 @@ __device__ __forceinline__ void pair_terms2(uint32_t tj, uint32_t ti0, uint32_t 
 // (corrector) takes the sums over theta~ and writes the new theta.  STAGE 2
 // is PROG2's UpdateRHS: the sums over theta, stored in g1 for the
 // AdvanceSystem kernel of the Euler-Maruyama scheme.
-template <int STAGE>
-__global__ void __launch_bounds__(kPairThreads) kur_pairwise_stage(const KurPairArgs A) {
-  __shared__ uint4 src_s[kPairTile / 4];  // source phases (fixed-point turns), four per entry
+template <int STAGE, int RPT, int S>
+__global__ void __launch_bounds__(32 * S) kur_pairwise_stage(const KurPairArgs A) {
+  constexpr int THREADS = 32 * S, RPC = RPT * 32;
+  constexpr int TILE = 1024;  // sources
+  constexpr int NP = TILE / 2 / THREADS;
+  __shared__ float4 src_s[TILE / 2];
+  __shared__ float red[S * RPC];
   const int rep = blockIdx.y;
-  const int64_t N = A.N;
-  const int64_t base = (int64_t)rep * N;
-  const uint32_t *src = STAGE == 1 ? A.theta_t : A.theta;  // corrector: sums over theta~
-  uint32_t ti[kPairPerThread];
-  float acc[kPairPerThread];
-  int64_t idx[kPairPerThread];
+  const uint32_t N = (uint32_t)A.N;  // < 2^31
+  const int64_t base = (int64_t)rep * A.N;
+  const float2 *src = (STAGE == 1 ? A.sc_t : A.sc) + base;  // corrector: sums over theta~
+  const int t = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int64_t i0 = (int64_t)blockIdx.x * RPC;
+  float si[RPT], ci[RPT];
+  float2 acc[RPT];
 #pragma unroll
-  for (int k = 0; k < kPairPerThread; ++k) {
-    idx[k] = (int64_t)blockIdx.x * kPairTile + threadIdx.x + k * kPairThreads;
-    ti[k] = idx[k] < N ? src[base + idx[k]] : 0u;
-    acc[k] = 0.0f;
+  for (int k = 0; k < RPT; ++k) {
+    const int64_t i = i0 + t + 32 * k;
+    const float2 a = i < N ? src[i] : make_float2(0.0f, 0.0f);
+    si[k] = a.x;
+    ci[k] = a.y;
+    acc[k] = make_float2(0.0f, 0.0f);
   }
-  static_assert(kPairPerThread == 2, "the receivers of a thread form one packed pair");
-  uint32_t *src_w = reinterpret_cast<uint32_t *>(src_s);
-  float2 acc2 = make_float2(0.0f, 0.0f);
-  for (int64_t j0 = 0; j0 < N; j0 += kPairTile) {
-    const int cnt = (N - j0) < kPairTile ? (int)(N - j0) : kPairTile;
+  // the next tile's sources are in flight during the current tile's terms;
+  // sources beyond N are zero terms
+  float2 pa[NP], pb[NP];
+  auto load = [&](uint32_t j0) {
 #pragma unroll
-    for (int k = 0; k < kPairPerThread; ++k) {
-      const int jj = threadIdx.x + k * kPairThreads;
-      if (jj < cnt) src_w[jj] = src[base + j0 + jj];
+    for (int u = 0; u < NP; ++u) {
+      const uint32_t j = j0 + 2 * (threadIdx.x + u * THREADS);
+      pa[u] = j < N ? src[j] : make_float2(0.0f, 0.0f);
+      pb[u] = j + 1 < N ? src[j + 1] : make_float2(0.0f, 0.0f);
+    }
+  };
+  load(0);
+  for (uint32_t j0 = 0; j0 < N; j0 += TILE) {
+#pragma unroll
+    for (int u = 0; u < NP; ++u)
+      src_s[threadIdx.x + u * THREADS] = make_float4(pa[u].x, pb[u].x, -pa[u].y, -pb[u].y);
+    __syncthreads();
+    if (N - j0 > TILE) load(j0 + TILE);
+    const int cnt = N - j0 < TILE ? (int)(N - j0) : TILE;
+    const int pairs = ((cnt + 7) & ~7) >> 1;
+    const int per = ((pairs + S - 1) / S + 3) & ~3;
+    const int pe = min((q + 1) * per, pairs);
+    for (int p = q * per; p < pe; p += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) pair_terms<RPT>(src_s[p + u], si, ci, acc);
     }
     __syncthreads();
-    if (cnt == kPairTile) {
-#pragma unroll 2
-      for (int q = 0; q < kPairTile / 4; ++q) {
-        const uint4 t4 = src_s[q];
-        pair_terms2(t4.x, ti[0], ti[1], acc2);
-        pair_terms2(t4.y, ti[0], ti[1], acc2);
-        pair_terms2(t4.z, ti[0], ti[1], acc2);
-        pair_terms2(t4.w, ti[0], ti[1], acc2);
-      }
-    } else {
-      for (int jj = 0; jj < cnt; ++jj) pair_terms2(src_w[jj], ti[0], ti[1], acc2);
-    }
-    __syncthreads();
   }
-  acc[0] = acc2.x;
-  acc[1] = acc2.y;
-  if (STAGE == 2) {
 #pragma unroll
-    for (int k = 0; k < kPairPerThread; ++k)
-      if (idx[k] < N) A.g1[base + idx[k]] = acc[k];
-    return;
-  }
+  for (int k = 0; k < RPT; ++k) red[q * RPC + t + 32 * k] = acc[k].x + acc[k].y;
+  __syncthreads();
   const uint2 key = seed_to_key(A.seed);
   const int64_t n = A.n;
+  for (int rl = threadIdx.x; rl < RPC; rl += THREADS) {
+    const int64_t i = i0 + rl;
+    if (i >= N) break;
+    float g = red[rl];
 #pragma unroll
-  for (int k = 0; k < kPairPerThread; ++k) {
-    if (idx[k] >= N) continue;
-    const int64_t gi = base + idx[k];
+    for (int w = 1; w < S; ++w) g += red[w * RPC + rl];
+    const int64_t gi = base + i;
+    if (STAGE == 2) {
+      A.g1[gi] = g;
+      continue;
+    }
     float z[4];
-    gauss4((uint32_t)(n >> 2), (uint32_t)idx[k], (uint32_t)rep, kTagKuramoto, key, z);
+    gauss4((uint32_t)(n >> 2), (uint32_t)i, (uint32_t)rep, kTagKuramoto, key, z);
     const float psi = pick4(z, (int)(n & 3));
     const float wdt = A.omega[gi] * A.wscale;
+    uint32_t th = A.theta[gi];
+    float sn, cs;
     if (STAGE == 0) {
-      const float d1 = fmaf(A.sc, psi, fmaf(A.kc, acc[k], wdt));
-      A.theta_t[gi] = A.theta[gi] + (uint32_t)__float2int_rn(d1 * 4294967296.0f);
-      A.g1[gi] = acc[k];
+      const float d1 = fmaf(A.sc_noise, psi, fmaf(A.kc, g, wdt));
+      th += (uint32_t)__float2int_rn(d1 * 4294967296.0f);
+      A.theta_t[gi] = th;
+      A.g1[gi] = g;
+      sincos_turns(th, sn, cs);
+      A.sc_t[gi] = make_float2(sn, cs);
     } else {
-      const float d = fmaf(A.sc, psi, fmaf(A.kh, A.g1[gi] + acc[k], wdt));
-      A.theta[gi] += (uint32_t)__float2int_rn(d * 4294967296.0f);
+      const float d = fmaf(A.sc_noise, psi, fmaf(A.kh, A.g1[gi] + g, wdt));
+      th += (uint32_t)__float2int_rn(d * 4294967296.0f);
+      A.theta[gi] = th;
+      sincos_turns(th, sn, cs);
+      A.sc[gi] = make_float2(sn, cs);
     }
   }
+}
+
+// sin and cos of every phase, the sources of the first pairwise stage.
+__global__ void kur_sincos_kernel(const uint32_t *theta, float2 *sc, int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    float sn, cs;
+    sincos_turns(theta[i], sn, cs);
+    sc[i] = make_float2(sn, cs);
+  }
+}
+
+// The shape of the pairwise launches.  Eight receivers per thread keep the
+// shared loads well below the FMA pipe's time; four slices give each of an
+// SM's schedulers one warp of every block (with two, 1024 blocks on 152 SMs
+// left 3 warps on one scheduler and 4 on another: 92 us per stage at N = 4096,
+// 64 replicas, against 76 us).  Below about twelve warps per SM more slices
+// take the place of receivers per thread.
+PairShape pair_shape(int64_t N, int64_t R, int sm_count) {
+  const int64_t want = (int64_t)sm_count * 12;
+  if ((N + 255) / 256 * R * 4 >= want) return {8, 4};
+  if ((N + 127) / 128 * R * 8 >= want) return {4, 8};
+  return {2, 16};
+}
+
+template <int STAGE>
+cudaError_t launch_pairwise(const KurPairArgs &a, int64_t R, const PairShape &p, cudaStream_t s) {
+  const dim3 grid((unsigned)((a.N + p.receivers() - 1) / p.receivers()), (unsigned)R);
+  if (p.s == 4)
+    kur_pairwise_stage<STAGE, 8, 4><<<grid, p.threads(), 0, s>>>(a);
+  else if (p.s == 8)
+    kur_pairwise_stage<STAGE, 4, 8><<<grid, p.threads(), 0, s>>>(a);
+  else
+    kur_pairwise_stage<STAGE, 2, 16><<<grid, p.threads(), 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 // PROG2's AdvanceSystem with Euler-Maruyama: theta += wdt + kc g + sc psi
@@ -858,8 +913,12 @@ __global__ void kur_advance_euler_kernel(const KurPairArgs A, int64_t R) {
     const int64_t rep = gi / A.N, i = gi - rep * A.N;
     float z[4];
     gauss4((uint32_t)(A.n >> 2), (uint32_t)i, (uint32_t)rep, kTagKuramoto, key, z);
-    const float d = fmaf(A.sc, pick4(z, (int)(A.n & 3)), fmaf(A.kc, A.g1[gi], A.omega[gi] * A.wscale));
-    A.theta[gi] += (uint32_t)__float2int_rn(d * 4294967296.0f);
+    const float d = fmaf(A.sc_noise, pick4(z, (int)(A.n & 3)), fmaf(A.kc, A.g1[gi], A.omega[gi] * A.wscale));
+    const uint32_t th = A.theta[gi] + (uint32_t)__float2int_rn(d * 4294967296.0f);
+    A.theta[gi] = th;
+    float sn, cs;
+    sincos_turns(th, sn, cs);
+    A.sc[gi] = make_float2(sn, cs);
   }
 }
 
@@ -1283,6 +1342,7 @@ sde_status kuramoto_create(const sde_config *cfg, int sm_count, uint32_t *err, K
     alloc((void **)&k->theta_t, NR * 4);
     alloc((void **)&k->g1, NR * 4);
   }
+  if (cfg->model == SDE_KURAMOTO_PAIRWISE) alloc((void **)&k->pair_sc, NR * 2 * sizeof(float2));
   if (grid_possible) {
     mfg_grid_for(k->N, k->R, sm_count, k->mfg_grid);
     k->mfg_blocks = *std::max_element(k->mfg_grid, k->mfg_grid + 4);
@@ -1339,8 +1399,9 @@ sde_status kuramoto_create(const sde_config *cfg, int sm_count, uint32_t *err, K
     k->block = block;
     k->opt = opt;
   } else if (cfg->model == SDE_KURAMOTO_PAIRWISE) {
-    k->block = kPairThreads;
-    k->opt = kPairPerThread;
+    const PairShape p = pair_shape(k->N, k->R, sm_count);
+    k->block = p.threads();
+    k->opt = p.rpt;
   }
   *out = k;
   return SDE_OK;
@@ -1402,6 +1463,7 @@ void kuramoto_destroy(KuramotoCtx *k) {
   cudaFree(k->theta);
   cudaFree(k->theta_t);
   cudaFree(k->g1);
+  cudaFree(k->pair_sc);
   cudaFree(k->r_scratch);
   cudaFree(k->mfg_partials);
   cudaFree(k->mfg_tot);
@@ -1471,17 +1533,22 @@ sde_status kuramoto_run(KuramotoCtx *k, const sde_run_desc *r, cudaStream_t s, c
     a.theta = k->theta;
     a.theta_t = k->theta_t;
     a.g1 = k->g1;
+    a.sc = k->pair_sc;
+    a.sc_t = k->pair_sc + NR;
     a.omega = r->omega_dev;
     a.N = k->N;
     a.wscale = (float)(k->dt * inv2pi);
     a.kc = (float)(k->K / (double)k->N * k->dt * inv2pi);
     a.kh = (float)(0.5 * k->K / (double)k->N * k->dt * inv2pi);
-    a.sc = (float)(sqrt(2.0 * k->D * k->dt) * inv2pi);
+    a.sc_noise = (float)(sqrt(2.0 * k->D * k->dt) * inv2pi);
     a.seed = k->seed;
-    const dim3 grid((unsigned)((k->N + kPairTile - 1) / kPairTile), (unsigned)k->R);
+    const PairShape shape = pair_shape(k->N, k->R, k->sm_count);
+    if (r->n_end > r->n_begin) {
+      kur_sincos_kernel<<<cvt_grid, 256, 0, s>>>(k->theta, k->pair_sc, NR);
+      SDE_CUDA_TRY(cudaGetLastError());
+    }
     int64_t sample = 0;
     const bool euler = (k->flags & SDE_FLAG_EULER) != 0;
-    const int64_t NR = k->N * k->R;
     const unsigned adv_grid = (unsigned)std::min<int64_t>((NR + 255) / 256, (int64_t)k->sm_count * 8);
     for (int64_t n = r->n_begin; n < r->n_end; ++n) {
       if (k->M > 0 && (n - r->n_begin) % k->M == 0) {
@@ -1492,16 +1559,16 @@ sde_status kuramoto_run(KuramotoCtx *k, const sde_run_desc *r, cudaStream_t s, c
       if (euler) {
         // PROG2: UpdateRHS, then AdvanceSystem
         SDE_CUDA_TRY(ktime_begin(k, s));
-        kur_pairwise_stage<2><<<grid, kPairThreads, 0, s>>>(a);
+        SDE_CUDA_TRY(launch_pairwise<2>(a, k->R, shape, s));
         SDE_CUDA_TRY(ktime_end(k, s));
         kur_advance_euler_kernel<<<adv_grid, 256, 0, s>>>(a, k->R);
         continue;
       }
       SDE_CUDA_TRY(ktime_begin(k, s));
-      kur_pairwise_stage<0><<<grid, kPairThreads, 0, s>>>(a);
+      SDE_CUDA_TRY(launch_pairwise<0>(a, k->R, shape, s));
       SDE_CUDA_TRY(ktime_end(k, s));
       SDE_CUDA_TRY(ktime_begin(k, s));
-      kur_pairwise_stage<1><<<grid, kPairThreads, 0, s>>>(a);
+      SDE_CUDA_TRY(launch_pairwise<1>(a, k->R, shape, s));
       SDE_CUDA_TRY(ktime_end(k, s));
     }
     SDE_CUDA_TRY(cudaGetLastError());

@@ -36,6 +36,7 @@ struct KuramotoCtx {
   uint32_t *theta_t = nullptr;  // predictor phases (pairwise, general, grid-wide mean field)
   float *g1 = nullptr;          // first-stage coupling sums (pairwise, general); grid-wide
                                 // mean field: the first-stage part of the step increment
+  float2 *pair_sc = nullptr;    // pairwise: [2][R][N] (sin, cos) of theta, then of theta~
   double *r_scratch = nullptr;  // r samples when the caller passes none
   int64_t r_scratch_rows = 0;
   // general coupling
@@ -81,10 +82,11 @@ struct KurPairArgs {
   uint32_t *theta;
   uint32_t *theta_t;
   float *g1;
+  float2 *sc, *sc_t;  // (sin, cos) of theta and of theta~
   const float *omega;
   int64_t N;
   int64_t n;
-  float wscale, kc, kh, sc;
+  float wscale, kc, kh, sc_noise;
   uint64_t seed;
 };
 
