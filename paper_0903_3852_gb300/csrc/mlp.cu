@@ -12,10 +12,11 @@
 // layers runs the fused tensor-core kernel of mlp_tc.cuh: the square hidden
 // layers as tcgen05 MMAs (M = 128 points, N = 256, K = 256) with the bias,
 // SiLU and the output layer in their epilogues.  The training path (forward
-// with stored pre-activations, backward, Adam) uses one tiled CUDA-core kernel
-// with 64 x 64 output tiles for all three GEMM shapes (forward, weight
-// gradient, input gradient) through layout flags, with the bias / activation /
-// derivative fused into its epilogue.
+// with stored pre-activations, backward, Adam) runs on the CUDA cores, every
+// sum over k in ascending order with one FMA per term: about a dozen launches
+// per step for all members together (members are a grid dimension):
+// 180 us for 4 members of 1024 points, 1.70 ms when each member's layers were
+// launched by themselves.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -23,6 +24,7 @@
 #include <algorithm>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -38,105 +40,502 @@ namespace {
 
 constexpr uint32_t kTagInit = 6u;  // Philox stream tag of the initial weights
 
-enum Epi { EPI_FWD_HIDDEN = 0, EPI_FWD_OUT = 1, EPI_STORE = 2, EPI_DSILU = 3 };
-
-__device__ __forceinline__ float ld(const float *p) { return *p; }
-__device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-
 __device__ __forceinline__ float sigmoidf_(float z) { return 1.0f / (1.0f + expf(-z)); }
 
-struct EpiArgs {
-  const float *bias;      // FWD_*: bias[n]
-  float *zout;            // FWD_HIDDEN: pre-activation [M][N]; FWD_OUT / STORE: output [M][N]
-  __nv_bfloat16 *hout;    // FWD_HIDDEN: SiLU(z) [M][N]; DSILU: dZ [M][N]
-  const float *zin;       // DSILU: pre-activation [M][N]
+__device__ __forceinline__ float silu_grad(float acc, float z) {
+  const float s = sigmoidf_(z);
+  return acc * (s * (1.0f + z * (1.0f - s)));
+}
+
+__device__ __forceinline__ float bf16_round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
+// ---- square layers: C[m][n] = sum_k A(m, k) B(n, k), members along z -------
+//
+// 64 x 64 outputs per CTA of 128 threads, 8 x 4 per thread as packed FP32
+// pairs along m (a packed FMA rounds each half like fmaf, so every output is
+// the same chain of FMAs over ascending k as a scalar loop).  K slices of 32
+// are staged as FP32 in shared memory, the next slice's global loads (16
+// bytes each) in flight during the current slice's FMAs.
+// What bounds it: shared memory returns 128 bytes per cycle to the SM's four
+// schedulers, 48 cycles per k against 32 of packed FMAs, and its latency with
+// one or two warps per scheduler, so the fragments of kF k's are read ahead.
+// The members and, for the weight gradients, the layers share a launch
+// (grid.z): one member's GEMM fills a tenth of the GPU.  4 members, 1024 points
+// each, 256 wide: 22 us a layer forward, 26 us backward, 34 us for the weight
+// gradients of both square layers (one member's layer at a time: 17, 27 and 84
+// us each).  Measured beside it: 4 x 4 outputs in 256 threads (23, 26, 37 us);
+// 8 x 8 (gradients 8 x 4) in 64 threads from BF16 in shared memory, half the
+// shared traffic but one warp per scheduler (28, 32, 59 us).
+enum Epi { EPI_FWD = 0, EPI_DSILU = 1, EPI_DW = 2 };
+
+constexpr int TM = 64, TN = 64, TK = 32, GT = 128, TPAD = 4, kF = 2;
+constexpr int kMaxLayers = 9;  // n_hidden <= 8
+
+struct GemmArgs {
+  int64_t B;        // rows of a member's batch
+  int32_t H;        // width of the square layers
+  int32_t n_layers; // EPI_DW: layers along z (member-major)
+  int64_t rows;     // row stride between members in the activation buffers (= B)
+  const void *a[kMaxLayers];             // FWD: h_l; DSILU, DW: dZ_l (FP32 holding BF16 values)
+  const __nv_bfloat16 *b[kMaxLayers];    // FWD, DSILU: W_l of the first member; DW: h_l
+  int64_t b_member;                      // member stride of b
+  const float *bias;                     // FWD, first member
+  int64_t p_member;                      // member stride of bias / gradients (parameters per member)
+  float *z;                              // FWD: pre-activation out; DSILU: in, overwritten by dZ_{l-1}
+  __nv_bfloat16 *h;                      // FWD: SiLU(z) out
+  float *grad[kMaxLayers];               // DW: gradient of W_l, first member
 };
 
-// C[m][n] = sum_k A(m, k) B(n, k);
-// A(m, k) = A_T ? A[k * M + m] : A[m * K + k];  B(n, k) = B_T ? B[k * N + n] : B[n * K + k].
-template <typename TA, typename TB, bool A_T, bool B_T, int EPI>
-__global__ void __launch_bounds__(256) mlp_gemm_kernel(const TA *__restrict__ A, const TB *__restrict__ Bm,
-                                                       int M, int N, int K, EpiArgs e) {
-  constexpr int TM = 64, TN = 64, TK = 16;
-  __shared__ float As[TK][TM + 4];
-  __shared__ float Bs[TK][TN + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += TK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int el = tid * 4 + q;  // 1024 elements of each tile
-      int m, k;
-      if (A_T) {
-        k = el / TM;
-        m = el % TM;
-      } else {
-        m = el / TK;
-        k = el % TK;
-      }
-      const int gm = m0 + m, gk = k0 + k;
-      float a = 0.0f;
-      if (gm < M && gk < K) a = A_T ? ld(A + (size_t)gk * M + gm) : ld(A + (size_t)gm * K + gk);
-      As[k][m] = a;
-      int n, kb;
-      if (B_T) {
-        kb = el / TN;
-        n = el % TN;
-      } else {
-        n = el / TK;
-        kb = el % TK;
-      }
-      const int gn = n0 + n, gkb = k0 + kb;
-      float b = 0.0f;
-      if (gn < N && gkb < K) b = B_T ? ld(Bm + (size_t)gkb * N + gn) : ld(Bm + (size_t)gn * K + gkb);
-      Bs[kb][n] = b;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = As[kk][ty * 4 + i];
-        b[i] = Bs[kk][tx * 4 + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
+__device__ __forceinline__ void unpack(const uint4 &v, float (&f)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= M) continue;
+    f[2 * i] = __uint_as_float(w[i] << 16);
+    f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+  }
+}
+__device__ __forceinline__ void unpack(const uint4 &v, float (&f)[4]) {
+  f[0] = __uint_as_float(v.x);
+  f[1] = __uint_as_float(v.y);
+  f[2] = __uint_as_float(v.z);
+  f[3] = __uint_as_float(v.w);
+}
+
+// One operand's 64 x 32 slice: TRANS false: rows of `ld` elements with k
+// contiguous; true: rows of k with the 64 outputs contiguous.  `limit` bounds
+// the row index of the source (batch rows), zero beyond it.
+template <typename T, bool TRANS>
+struct Slice {
+  static constexpr int EV = 16 / (int)sizeof(T);            // elements per 16-byte load
+  static constexpr int NV = TM * TK / EV / GT;              // loads per thread
+  uint4 v[NV];
+  __device__ __forceinline__ void load(const T *src, int64_t ld, int64_t o0, int64_t k0, int64_t limit) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      const size_t o = (size_t)m * N + n;
-      if (EPI == EPI_FWD_HIDDEN) {
-        const float z = acc[i][j] + e.bias[n];
-        e.zout[o] = z;
-        e.hout[o] = __float2bfloat16_rn(z * sigmoidf_(z));
-      } else if (EPI == EPI_FWD_OUT) {
-        e.zout[o] = acc[i][j] + e.bias[n];
-      } else if (EPI == EPI_STORE) {
-        e.zout[o] = acc[i][j];
+    for (int i = 0; i < NV; ++i) {
+      const int c = threadIdx.x + i * GT;
+      const int64_t row = TRANS ? k0 + c / (TM / EV) : o0 + (c & (TM - 1));
+      const int64_t col = TRANS ? o0 + (c % (TM / EV)) * EV : k0 + (c / TM) * EV;
+      v[i] = row < limit ? *reinterpret_cast<const uint4 *>(src + row * ld + col) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  __device__ __forceinline__ void store(float (*S)[TM + TPAD]) const {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = threadIdx.x + i * GT;
+      float f[EV];
+      unpack(v[i], f);
+      if (TRANS) {
+        float *d = &S[c / (TM / EV)][(c % (TM / EV)) * EV];
+#pragma unroll
+        for (int e = 0; e < EV; e += 4) *reinterpret_cast<float4 *>(d + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
       } else {
-        const float z = e.zin[o];
-        const float s = sigmoidf_(z);
-        e.hout[o] = __float2bfloat16_rn(acc[i][j] * (s * (1.0f + z * (1.0f - s))));
+#pragma unroll
+        for (int e = 0; e < EV; ++e) S[(c / TM) * EV + e][c & (TM - 1)] = f[e];
+      }
+    }
+  }
+};
+
+template <int EPI>
+__global__ void __launch_bounds__(GT) mlp_gemm_kernel(const GemmArgs g) {
+  using TA = typename std::conditional<EPI == EPI_FWD, __nv_bfloat16, float>::type;
+  constexpr bool A_T = EPI == EPI_DW, B_T = EPI != EPI_FWD;
+  __shared__ __align__(16) float As[2][TK][TM + TPAD];
+  __shared__ __align__(16) float Bs[2][TK][TN + TPAD];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int layer = EPI == EPI_DW ? (int)(blockIdx.z % g.n_layers) : 0;
+  const int64_t member = EPI == EPI_DW ? blockIdx.z / g.n_layers : blockIdx.z;
+  const int64_t m0 = (int64_t)blockIdx.x * TM;
+  const int n0 = blockIdx.y * TN;
+  const int64_t H = g.H, B = g.B;
+  const TA *A = (const TA *)g.a[layer] + member * g.rows * H;
+  const __nv_bfloat16 *Bm = g.b[layer] + member * g.b_member;
+  const int64_t K = EPI == EPI_DW ? B : H;
+  const int64_t a_limit = B, b_limit = EPI == EPI_DW ? B : H;  // both operands of DW run over batch rows
+  Slice<TA, A_T> sa;
+  Slice<__nv_bfloat16, B_T> sb;
+  sa.load(A, H, m0, 0, a_limit);
+  sb.load(Bm, H, n0, 0, b_limit);
+  sa.store(As[0]);
+  sb.store(Bs[0]);
+  __syncthreads();
+  float2 acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+  int buf = 0;
+  for (int64_t k0 = 0; k0 < K; k0 += TK) {
+    const bool more = k0 + TK < K;
+    if (more) {
+      sa.load(A, H, m0, k0 + TK, a_limit);
+      sb.load(Bm, H, n0, k0 + TK, b_limit);
+    }
+    // kF k's fragments at a time, read while the previous ones are multiplied
+    float4 a0[2][kF], a1[2][kF], b[2][kF];
+    auto frag = [&](int q, int k) {
+#pragma unroll
+      for (int u = 0; u < kF; ++u) {
+        a0[q][u] = *reinterpret_cast<const float4 *>(&As[buf][k + u][ty * 4]);
+        a1[q][u] = *reinterpret_cast<const float4 *>(&As[buf][k + u][32 + ty * 4]);
+        b[q][u] = *reinterpret_cast<const float4 *>(&Bs[buf][k + u][tx * 4]);
+      }
+    };
+    frag(0, 0);
+#pragma unroll
+    for (int kg = 0; kg < TK / kF; ++kg) {
+      const int q = kg & 1;
+      if (kg + 1 < TK / kF) frag(q ^ 1, (kg + 1) * kF);
+#pragma unroll
+      for (int u = 0; u < kF; ++u) {
+        const float2 ap[4] = {make_float2(a0[q][u].x, a0[q][u].y), make_float2(a0[q][u].z, a0[q][u].w),
+                              make_float2(a1[q][u].x, a1[q][u].y), make_float2(a1[q][u].z, a1[q][u].w)};
+        const float bv[4] = {b[q][u].x, b[q][u].y, b[q][u].z, b[q][u].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[i][j] = __ffma2_rn(ap[i], make_float2(bv[j], bv[j]), acc[i][j]);
+      }
+    }
+    if (more) {
+      buf ^= 1;
+      sa.store(As[buf]);
+      sb.store(Bs[buf]);
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int64_t m = m0 + (i < 4 ? 0 : 32) + ty * 4 + (i & 3);
+    const int n = n0 + tx * 4;
+    float c[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[j] = (i & 1) ? acc[i / 2][j].y : acc[i / 2][j].x;
+    if (EPI == EPI_DW) {
+      float *o = g.grad[layer] + member * g.p_member + m * H + n;  // FP32 parameters: 4-byte aligned only
+#pragma unroll
+      for (int j = 0; j < 4; ++j) o[j] = c[j];
+    } else if (m < B) {
+      const int64_t o = (member * g.rows + m) * H + n;
+      if (EPI == EPI_FWD) {
+        const float *bias = g.bias + member * g.p_member + n;
+        __nv_bfloat16 hv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          c[j] += bias[j];
+          hv[j] = __float2bfloat16_rn(c[j] * sigmoidf_(c[j]));
+        }
+        *reinterpret_cast<float4 *>(g.z + o) = make_float4(c[0], c[1], c[2], c[3]);
+        *reinterpret_cast<uint2 *>(g.h + o) = *reinterpret_cast<const uint2 *>(hv);
+      } else {
+        const float4 z = *reinterpret_cast<const float4 *>(g.z + o);
+        *reinterpret_cast<float4 *>(g.z + o) =
+            make_float4(bf16_round(silu_grad(c[0], z.x)), bf16_round(silu_grad(c[1], z.y)),
+                        bf16_round(silu_grad(c[2], z.z)), bf16_round(silu_grad(c[3], z.w)));
       }
     }
   }
 }
 
-__global__ void to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = __float2bfloat16_rn(src[i]);
+// ---- layer 0, and the BF16 copies of the parameters ------------------------
+//
+// The first blocks of each member compute layer 0 (n_in <= 8 inputs: one
+// thread per column, kRows0 batch rows per block), the others round the
+// member's FP32 parameters to the BF16 operands of the square layers; the two
+// do not depend on each other.
+constexpr int kRows0 = 16;
+
+struct Layer0Args {
+  const float *X;        // [members or 1][B][n_in]
+  int64_t x_member;      // member stride of X (0: one batch for all members)
+  const float *params;   // first member
+  int64_t P, P_bf16;     // parameters per member and the member stride of wbf (a multiple of 8)
+  int64_t w0, b0;        // offsets of W_0, b_0
+  int64_t B, rows;
+  int32_t n_in, H, blocks0;
+  float *z;
+  __nv_bfloat16 *h, *wbf;
+};
+
+__global__ void __launch_bounds__(256) mlp_layer0_kernel(const Layer0Args a) {
+  __shared__ float xs[kRows0][8];
+  const int64_t member = blockIdx.y;
+  const float *pm = a.params + member * a.P;
+  if ((int)blockIdx.x >= a.blocks0) {
+    const int64_t stride = (int64_t)(gridDim.x - a.blocks0) * 256;
+    for (int64_t i = (int64_t)(blockIdx.x - a.blocks0) * 256 + threadIdx.x; i < a.P; i += stride)
+      a.wbf[member * a.P_bf16 + i] = __float2bfloat16_rn(pm[i]);
+    return;
+  }
+  const int64_t r0 = (int64_t)blockIdx.x * kRows0;
+  const int nr = (int)(a.B - r0 < kRows0 ? a.B - r0 : kRows0);
+  for (int i = threadIdx.x; i < nr * a.n_in; i += 256)
+    xs[i / a.n_in][i % a.n_in] = bf16_round(a.X[member * a.x_member + r0 * a.n_in + i]);
+  __syncthreads();
+  for (int n = threadIdx.x; n < a.H; n += 256) {
+    float w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = k < a.n_in ? bf16_round(pm[a.w0 + (int64_t)n * a.n_in + k]) : 0.0f;
+    const float bias = pm[a.b0 + n];
+    for (int r = 0; r < nr; ++r) {
+      float acc = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < a.n_in) acc = fmaf(xs[r][k], w[k], acc);
+      const float z = acc + bias;
+      const int64_t o = (member * a.rows + r0 + r) * a.H + n;
+      a.z[o] = z;
+      a.h[o] = __float2bfloat16_rn(z * sigmoidf_(z));
+    }
+  }
+}
+
+// ---- output layer, its gradient and the last hidden layer's dZ -------------
+//
+// 32 batch rows per block: each row's dot product with w_out is one lane's
+// chain over ascending k (rows staged in shared memory); training goes on to
+// g = 2/B (pred - y) and dZ = g w_out SiLU'(z), which overwrites z.
+constexpr int kRowsOut = 32, kOutChunk = 256;
+
+struct OutArgs {
+  const __nv_bfloat16 *h;  // last hidden activations
+  float *z;                // last hidden pre-activations, replaced by dZ
+  const float *params;     // first member
+  int64_t P, wo, bo;
+  int64_t B, rows;
+  int32_t H;
+  const float *y;          // [members or 1][B]; NULL: forward only
+  int64_t y_member;
+  float *pred;             // first member
+  int64_t pred_member;
+  float *g;                // [members][rows]
+};
+
+__global__ void __launch_bounds__(256) mlp_out_kernel(const OutArgs a) {
+  __shared__ __align__(16) __nv_bfloat16 hs[kRowsOut][kOutChunk + 8];
+  __shared__ float ws[kOutChunk];
+  __shared__ float gs[kRowsOut];
+  const int64_t member = blockIdx.y;
+  const int64_t r0 = (int64_t)blockIdx.x * kRowsOut;
+  const int nr = (int)(a.B - r0 < kRowsOut ? a.B - r0 : kRowsOut);
+  const float *pm = a.params + member * a.P;
+  const __nv_bfloat16 *h = a.h + (member * a.rows + r0) * a.H;
+  float acc = 0.0f;
+  for (int c0 = 0; c0 < a.H; c0 += kOutChunk) {
+    const int cn = a.H - c0 < kOutChunk ? a.H - c0 : kOutChunk;  // a multiple of 64
+    for (int i = threadIdx.x; i < nr * (cn / 8); i += 256) {
+      const int r = i / (cn / 8), c = (i % (cn / 8)) * 8;
+      *reinterpret_cast<uint4 *>(&hs[r][c]) = *reinterpret_cast<const uint4 *>(h + (int64_t)r * a.H + c0 + c);
+    }
+    for (int i = threadIdx.x; i < cn; i += 256) ws[i] = bf16_round(pm[a.wo + c0 + i]);
+    __syncthreads();
+    if ((int)threadIdx.x < nr) {
+      for (int c = 0; c < cn; c += 8) {
+        float f[8];
+        unpack(*reinterpret_cast<const uint4 *>(&hs[threadIdx.x][c]), f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc = fmaf(f[e], ws[c + e], acc);
+      }
+    }
+    __syncthreads();
+  }
+  if ((int)threadIdx.x < nr) {
+    const int64_t b = r0 + threadIdx.x;
+    const float pred = acc + pm[a.bo];
+    a.pred[member * a.pred_member + b] = pred;
+    if (a.y) {
+      const float d = pred - a.y[member * a.y_member + b];
+      const float gv = 2.0f * d / (float)a.B;
+      a.g[member * a.rows + b] = gv;
+      gs[threadIdx.x] = gv;
+    }
+  }
+  if (!a.y) return;
+  __syncthreads();
+  // eight float4 of z per thread at a time, loaded before any of them is replaced
+  float4 *z = reinterpret_cast<float4 *>(a.z + (member * a.rows + r0) * a.H);
+  const int q4 = a.H / 4, total = nr * q4;
+  for (int i0 = threadIdx.x; i0 < total; i0 += 8 * 256) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * 256 < total) v[u] = z[i0 + u * 256];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * 256;
+      if (i >= total) break;
+      const float gv = gs[i / q4];
+      const float *w = pm + a.wo + (i % q4) * 4;
+      v[u].x = bf16_round(silu_grad(gv * bf16_round(w[0]), v[u].x));
+      v[u].y = bf16_round(silu_grad(gv * bf16_round(w[1]), v[u].y));
+      v[u].z = bf16_round(silu_grad(gv * bf16_round(w[2]), v[u].z));
+      v[u].w = bf16_round(silu_grad(gv * bf16_round(w[3]), v[u].w));
+      z[i] = v[u];
+    }
+  }
+}
+
+// ---- the small gradients and the loss --------------------------------------
+//
+// One launch, the blocks of a member in four roles: (0) W_out and (1) W_0, 64
+// columns per block, each output one chain of FMAs over the batch; (2) bias
+// gradients, eight columns per block; (3) the output bias and the loss.  A
+// chain over the batch is serial, so the rows are staged 128 at a time in
+// shared memory by all threads, the next rows' loads in flight meanwhile.
+struct SmallArgs {
+  const __nv_bfloat16 *h_last;
+  const float *dz[kMaxLayers];  // hidden layers' dZ
+  const float *X;
+  int64_t x_member;
+  const float *g, *pred, *y;
+  int64_t pred_member, y_member;
+  int64_t B, rows, P;
+  int32_t H, n_in, n_hidden;
+  int64_t w0, wo, bo;
+  int64_t b[kMaxLayers];        // hidden layers' bias offsets
+  float *grad;                  // first member
+  float *loss;                  // [members] or NULL
+};
+
+__device__ __forceinline__ float block_sum(float s, float *red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = threadIdx.x < 8 ? red[threadIdx.x] : 0.0f;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  __syncthreads();
+  return s;  // valid in thread 0
+}
+
+constexpr int kChainRows = 128;
+
+// out[n * nk + k] = sum_b D[b][n] F[b][k], n0 .. n0 + 63, k < nk <= 8: 64
+// threads per pair of k's, a column each, two chains side by side (one warp's
+// instructions per row are what a tile waits for: all eight k's in one thread
+// took 27 us for the launch instead of 24).  NK = 1: one k, g in FP32;
+// NK = 8: X, a BF16 operand.
+template <typename T, int NK>
+__device__ __forceinline__ void chain_grad(const T *D, int64_t ldd, const float *F, int nk, int64_t B, int n0,
+                                           float *out, float (*Ds)[64], float (*Fs)[8]) {
+  constexpr int EV = 16 / (int)sizeof(T), NV = kChainRows * 64 / EV / 256;
+  uint4 v[NV];
+  float f[4];
+  auto load = [&](int64_t b0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = threadIdx.x + i * 256;
+      const int64_t b = b0 + c / (64 / EV);
+      v[i] = b < B ? *reinterpret_cast<const uint4 *>(D + b * ldd + n0 + (c % (64 / EV)) * EV)
+                   : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = threadIdx.x + i * 256;  // row e / 8, k = e % 8
+      const int64_t b = b0 + e / 8;
+      f[i] = (b < B && e % 8 < nk) ? F[b * nk + e % 8] : 0.0f;
+    }
+  };
+  load(0);
+  constexpr int KT = NK == 1 ? 1 : 2;  // chains per thread
+  const int col = threadIdx.x & 63, kq = (threadIdx.x >> 6) * KT;
+  const bool active = kq < nk;
+  float acc[KT] = {};
+  for (int64_t b0 = 0; b0 < B; b0 += kChainRows) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = threadIdx.x + i * 256;
+      float e[EV];
+      unpack(v[i], e);
+      float *d = &Ds[c / (64 / EV)][(c % (64 / EV)) * EV];
+#pragma unroll
+      for (int q = 0; q < EV; q += 4) *reinterpret_cast<float4 *>(d + q) = make_float4(e[q], e[q + 1], e[q + 2], e[q + 3]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = threadIdx.x + i * 256;
+      Fs[e / 8][e % 8] = NK > 1 ? bf16_round(f[i]) : f[i];
+    }
+    __syncthreads();
+    if (b0 + kChainRows < B) load(b0 + kChainRows);
+    if (active) {
+      // eight rows' values are read before their FMAs: a chain waits for its
+      // FMAs only, not for shared memory row by row
+#pragma unroll 2
+      for (int r0 = 0; r0 < kChainRows; r0 += 8) {
+        float d[8], fr[8][KT];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          d[r] = Ds[r0 + r][col];
+#pragma unroll
+          for (int k = 0; k < KT; ++k) fr[r][k] = Fs[r0 + r][kq + k];
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int k = 0; k < KT; ++k) acc[k] = fmaf(d[r], fr[r][k], acc[k]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < KT; ++k)
+    if (kq + k < nk) out[(int64_t)(n0 + col) * nk + kq + k] = acc[k];
+}
+
+__global__ void __launch_bounds__(256) mlp_small_grad_kernel(const SmallArgs a) {
+  __shared__ __align__(16) float Ds[kChainRows][64];
+  __shared__ __align__(16) float Fs[kChainRows][8];
+  __shared__ float red[32];
+  const int64_t member = blockIdx.y;
+  float *grad = a.grad + member * a.P;
+  const float *g = a.g + member * a.rows;
+  const int nc = a.H / 64;
+  int j = blockIdx.x;
+  if (j < nc) {
+    chain_grad<__nv_bfloat16, 1>(a.h_last + member * a.rows * a.H, a.H, g, 1, a.B, j * 64, grad + a.wo, Ds, Fs);
+    return;
+  }
+  j -= nc;
+  if (j < nc) {
+    chain_grad<float, 8>(a.dz[0] + member * a.rows * a.H, a.H, a.X + member * a.x_member, a.n_in, a.B, j * 64,
+                            grad + a.w0, Ds, Fs);
+    return;
+  }
+  j -= nc;
+  if (j < a.n_hidden * (a.H / 8)) {
+    const int l = j / (a.H / 8), n0 = (j % (a.H / 8)) * 8;
+    const float *dz = a.dz[l] + member * a.rows * a.H + n0;
+    float s[8] = {};
+    for (int64_t b = threadIdx.x; b < a.B; b += 256) {
+      const float4 u = *reinterpret_cast<const float4 *>(dz + b * a.H);
+      const float4 w = *reinterpret_cast<const float4 *>(dz + b * a.H + 4);
+      const float e[8] = {u.x, u.y, u.z, u.w, w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s[q] += e[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float t = block_sum(s[q], red);
+      if (threadIdx.x == 0) grad[a.b[l] + n0 + q] = t;
+    }
+    return;
+  }
+  float s = 0.0f, sq = 0.0f;
+  for (int64_t b = threadIdx.x; b < a.B; b += 256) {
+    s += g[b];
+    const float d = a.pred[member * a.pred_member + b] - a.y[member * a.y_member + b];
+    sq += d * d;
+  }
+  s = block_sum(s, red);
+  sq = block_sum(sq, red);
+  if (threadIdx.x == 0) {
+    grad[a.bo] = s;
+    if (a.loss) a.loss[member] = sq / (float)a.B;
+  }
 }
 
 // Uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) for weights and biases.
@@ -149,46 +548,6 @@ __global__ void init_kernel(float *params, const int64_t *off, const int *fin, i
     const float bound = rsqrtf((float)fin[l]);
     const uint4 r = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)(i >> 32), (uint32_t)member, kTagInit), key);
     params[(int64_t)member * P + i] = (2.0f * uniform24(r.x) - 1.0f) * bound;
-  }
-}
-
-// out = 2/B (y_pred - y), loss = mean (y_pred - y)^2 (one block, fixed order).
-__global__ void loss_kernel(const float *pred, const float *y, int64_t B, float *g, float *loss) {
-  __shared__ float red[32];
-  float s = 0.0f;
-  for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
-    const float d = pred[b] - y[b];
-    g[b] = 2.0f * d / (float)B;
-    s += d * d;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0 && loss) *loss = s / (float)B;
-  }
-}
-
-// db[n] = sum_b dZ[b][n]: one block per column, fixed order.
-template <typename T>
-__global__ void colsum_kernel(const T *dz, int64_t B, int N, float *db) {
-  __shared__ float red[32];
-  const int n = blockIdx.x;
-  float s = 0.0f;
-  for (int64_t b = threadIdx.x; b < B; b += blockDim.x) s += ld(dz + b * N + n);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) db[n] = s;
   }
 }
 
@@ -260,12 +619,13 @@ struct sde_mlp {
   std::vector<int64_t> woff, boff;
   int64_t P = 0;                // parameters per member
   float *params = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;  // [members][P]
-  __nv_bfloat16 *wbf = nullptr;                                         // [P]
-  std::vector<__nv_bfloat16 *> h;  // L entries: layer inputs (bf16), h[0] = X
-  std::vector<float *> z;          // L - 1 hidden pre-activations
-  __nv_bfloat16 *dz[2] = {nullptr, nullptr};
-  float *out = nullptr;            // [members][B]
-  float *gout = nullptr;           // [B] output-layer gradient
+  int64_t P_bf16 = 0;              // P rounded up to 8: the BF16 copies' rows stay 16-byte aligned
+  int64_t rows = 0;                // batch rows of the activation buffers (members share them)
+  __nv_bfloat16 *wbf = nullptr;    // [members][P_bf16]
+  std::vector<__nv_bfloat16 *> h;  // L entries: layer inputs (bf16), h[0] unused (layer 0 reads X)
+  std::vector<float *> z;          // L - 1 hidden pre-activations; the backward leaves dZ in their place
+  float *out = nullptr;            // [members][max_batch]
+  float *gout = nullptr;           // [rows] output-layer gradient
   float *lo_hi = nullptr;          // [10]
   int64_t *off_dev = nullptr;
   int *fin_dev = nullptr;
@@ -282,74 +642,135 @@ namespace {
 
 using namespace sde;
 
-template <typename TA, typename TB, bool A_T, bool B_T, int EPI>
-cudaError_t gemm(const TA *A, const TB *B, int M, int N, int K, EpiArgs e, cudaStream_t s) {
-  dim3 grid((M + 63) / 64, (N + 63) / 64);
-  mlp_gemm_kernel<TA, TB, A_T, B_T, EPI><<<grid, 256, 0, s>>>(A, B, M, N, K, e);
-  return cudaGetLastError();
+// Members whose batches of B rows fit in the activation buffers together.
+int64_t member_group(const sde_mlp *q, int64_t B) {
+  return std::max<int64_t>(1, std::min<int64_t>(q->cfg.n_members, q->rows / B));
 }
 
-// Forward pass of one member over X (FP32 [B][n_in]); output -> out_row[B].
-sde_status mlp_forward_member(sde_mlp *q, int member, const float *X, int64_t B, float *out_row, cudaStream_t s) {
+// Forward pass of members m0 .. m0 + G - 1, each over its own B rows of X
+// (x_member apart; 0: the same rows); with y also the output gradient and the
+// last hidden layer's dZ.  Predictions -> q->out.
+sde_status mlp_forward_members(sde_mlp *q, int64_t m0, int64_t G, const float *X, int64_t x_member, int64_t B,
+                               const float *y, int64_t y_member, cudaStream_t s) {
   SDE_CUDA_TRY(cudaGetLastError());
-  to_bf16_kernel<<<grid1(q->P), 256, 0, s>>>(q->params + (int64_t)member * q->P, q->wbf, q->P);
-  to_bf16_kernel<<<grid1(B * q->cfg.n_in), 256, 0, s>>>(X, q->h[0], B * q->cfg.n_in);
+  const int H = q->cfg.hidden;
+  const float *pm = q->params + m0 * q->P;
+  Layer0Args a0{};
+  a0.X = X;
+  a0.x_member = x_member;
+  a0.params = pm;
+  a0.P = q->P;
+  a0.P_bf16 = q->P_bf16;
+  a0.w0 = q->woff[0];
+  a0.b0 = q->boff[0];
+  a0.B = B;
+  a0.rows = B;
+  a0.n_in = q->cfg.n_in;
+  a0.H = H;
+  a0.blocks0 = (int)((B + kRows0 - 1) / kRows0);
+  a0.z = q->z[0];
+  a0.h = q->h[1];
+  a0.wbf = q->wbf;
+  mlp_layer0_kernel<<<dim3((unsigned)(a0.blocks0 + 128), (unsigned)G), 256, 0, s>>>(a0);
   SDE_CUDA_TRY(cudaGetLastError());
-  const float *pm = q->params + (int64_t)member * q->P;
-  for (int l = 0; l < q->L; ++l) {
-    EpiArgs e{};
-    e.bias = pm + q->boff[l];
-    if (l < q->L - 1) {
-      e.zout = q->z[l];
-      e.hout = q->h[l + 1];
-      SDE_CUDA_TRY((gemm<__nv_bfloat16, __nv_bfloat16, false, false, EPI_FWD_HIDDEN>(
-          q->h[l], q->wbf + q->woff[l], (int)B, q->fout[l], q->fin[l], e, s)));
-    } else {
-      e.zout = out_row;
-      SDE_CUDA_TRY((gemm<__nv_bfloat16, __nv_bfloat16, false, false, EPI_FWD_OUT>(
-          q->h[l], q->wbf + q->woff[l], (int)B, q->fout[l], q->fin[l], e, s)));
-    }
+  for (int l = 1; l < q->L - 1; ++l) {
+    GemmArgs g{};
+    g.B = B;
+    g.H = H;
+    g.n_layers = 1;
+    g.rows = B;
+    g.a[0] = q->h[l];
+    g.b[0] = q->wbf + q->woff[l];
+    g.b_member = q->P_bf16;
+    g.bias = pm + q->boff[l];
+    g.p_member = q->P;
+    g.z = q->z[l];
+    g.h = q->h[l + 1];
+    mlp_gemm_kernel<EPI_FWD><<<dim3((unsigned)((B + TM - 1) / TM), H / TN, (unsigned)G), GT, 0, s>>>(g);
+    SDE_CUDA_TRY(cudaGetLastError());
   }
+  OutArgs o{};
+  o.h = q->h[q->L - 1];
+  o.z = q->z[q->L - 2];
+  o.params = pm;
+  o.P = q->P;
+  o.wo = q->woff[q->L - 1];
+  o.bo = q->boff[q->L - 1];
+  o.B = B;
+  o.rows = B;
+  o.H = H;
+  o.y = y;
+  o.y_member = y_member;
+  o.pred = q->out + m0 * q->cfg.max_batch;
+  o.pred_member = q->cfg.max_batch;
+  o.g = q->gout;
+  mlp_out_kernel<<<dim3((unsigned)((B + kRowsOut - 1) / kRowsOut), (unsigned)G), 256, 0, s>>>(o);
+  SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }
 
-// Gradient of the MSE of one member into grad_out[P]; loss -> loss_out.
-sde_status mlp_grad_member(sde_mlp *q, int member, const float *X, const float *y, int64_t B, float *grad_out,
-                           float *loss_out, cudaStream_t s) {
-  float *pred = q->out + (int64_t)member * q->cfg.max_batch;
-  sde_status st = mlp_forward_member(q, member, X, B, pred, s);
+// Gradients of the MSE of members m0 .. m0 + G - 1 -> grad (q->P apart), their
+// losses -> loss (NULL allowed).
+sde_status mlp_grad_members(sde_mlp *q, int64_t m0, int64_t G, const float *X, int64_t x_member, const float *y,
+                            int64_t y_member, int64_t B, float *grad, float *loss, cudaStream_t s) {
+  sde_status st = mlp_forward_members(q, m0, G, X, x_member, B, y, y_member, s);
   if (st != SDE_OK) return st;
-  loss_kernel<<<1, 1024, 0, s>>>(pred, y, B, q->gout, loss_out);
-  SDE_CUDA_TRY(cudaGetLastError());
-  int cur = 0;
-  for (int l = q->L - 1; l >= 0; --l) {
-    EpiArgs e{};
-    // weight gradient dW_l = dZ_l^T h_l  ([fout][fin], K = batch)
-    e.zout = grad_out + q->woff[l];
-    if (l == q->L - 1) {
-      SDE_CUDA_TRY((gemm<float, __nv_bfloat16, true, true, EPI_STORE>(q->gout, q->h[l], q->fout[l], q->fin[l],
-                                                                       (int)B, e, s)));
-      colsum_kernel<float><<<q->fout[l], 256, 0, s>>>(q->gout, B, q->fout[l], grad_out + q->boff[l]);
-    } else {
-      SDE_CUDA_TRY((gemm<__nv_bfloat16, __nv_bfloat16, true, true, EPI_STORE>(q->dz[cur], q->h[l], q->fout[l],
-                                                                               q->fin[l], (int)B, e, s)));
-      colsum_kernel<__nv_bfloat16><<<q->fout[l], 256, 0, s>>>(q->dz[cur], B, q->fout[l], grad_out + q->boff[l]);
-    }
+  const int H = q->cfg.hidden, nh = q->cfg.n_hidden;
+  for (int l = nh - 1; l >= 1; --l) {  // dZ_{l-1} = (dZ_l W_l) SiLU'(z_{l-1})
+    GemmArgs g{};
+    g.B = B;
+    g.H = H;
+    g.n_layers = 1;
+    g.rows = B;
+    g.a[0] = q->z[l];
+    g.b[0] = q->wbf + q->woff[l];
+    g.b_member = q->P_bf16;
+    g.z = q->z[l - 1];
+    mlp_gemm_kernel<EPI_DSILU><<<dim3((unsigned)((B + TM - 1) / TM), H / TN, (unsigned)G), GT, 0, s>>>(g);
     SDE_CUDA_TRY(cudaGetLastError());
-    if (l > 0) {
-      // dZ_{l-1} = (dZ_l W_l) * SiLU'(z_{l-1})   ([B][fin])
-      EpiArgs d{};
-      d.zin = q->z[l - 1];
-      d.hout = q->dz[cur ^ 1];
-      if (l == q->L - 1)
-        SDE_CUDA_TRY((gemm<float, __nv_bfloat16, false, true, EPI_DSILU>(q->gout, q->wbf + q->woff[l], (int)B,
-                                                                         q->fin[l], q->fout[l], d, s)));
-      else
-        SDE_CUDA_TRY((gemm<__nv_bfloat16, __nv_bfloat16, false, true, EPI_DSILU>(
-            q->dz[cur], q->wbf + q->woff[l], (int)B, q->fin[l], q->fout[l], d, s)));
-      cur ^= 1;
-    }
   }
+  if (nh > 1) {  // dW_l = dZ_l^T h_l of every square layer
+    GemmArgs g{};
+    g.B = B;
+    g.H = H;
+    g.n_layers = nh - 1;
+    g.rows = B;
+    g.b_member = B * H;
+    g.p_member = q->P;
+    for (int l = 1; l < nh; ++l) {
+      g.a[l - 1] = q->z[l];
+      g.b[l - 1] = q->h[l];
+      g.grad[l - 1] = grad + q->woff[l];
+    }
+    mlp_gemm_kernel<EPI_DW><<<dim3(H / TM, H / TN, (unsigned)(G * (nh - 1))), GT, 0, s>>>(g);
+    SDE_CUDA_TRY(cudaGetLastError());
+  }
+  SmallArgs a{};
+  a.h_last = q->h[nh];
+  for (int l = 0; l < nh; ++l) {
+    a.dz[l] = q->z[l];
+    a.b[l] = q->boff[l];
+  }
+  a.X = X;
+  a.x_member = x_member;
+  a.g = q->gout;
+  a.pred = q->out + m0 * q->cfg.max_batch;
+  a.pred_member = q->cfg.max_batch;
+  a.y = y;
+  a.y_member = y_member;
+  a.B = B;
+  a.rows = B;
+  a.P = q->P;
+  a.H = H;
+  a.n_in = q->cfg.n_in;
+  a.n_hidden = nh;
+  a.w0 = q->woff[0];
+  a.wo = q->woff[nh];
+  a.bo = q->boff[nh];
+  a.grad = grad;
+  a.loss = loss;
+  mlp_small_grad_kernel<<<dim3((unsigned)(2 * (H / 64) + nh * (H / 8) + 1), (unsigned)G), 256, 0, s>>>(a);
+  SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }
 
@@ -363,8 +784,6 @@ void mlp_free(sde_mlp *q) {
   cudaFree(q->wbf);
   for (auto p : q->h) cudaFree(p);
   for (auto p : q->z) cudaFree(p);
-  cudaFree(q->dz[0]);
-  cudaFree(q->dz[1]);
   cudaFree(q->out);
   cudaFree(q->gout);
   cudaFree(q->lo_hi);
@@ -426,16 +845,19 @@ sde_status sde_mlp_create(const sde_mlp_config *cfg, sde_mlp **out) {
   alloc((void **)&q->m, sizeof(float) * M * q->P);
   alloc((void **)&q->v, sizeof(float) * M * q->P);
   alloc((void **)&q->grad, sizeof(float) * M * q->P);
-  alloc((void **)&q->wbf, sizeof(__nv_bfloat16) * q->P);
+  // the members' batches share the activation rows: at least one member's
+  // largest batch, and up to 32 MB more of pre-activations per layer so that
+  // small networks' members train together at their largest batch too
+  q->rows = std::max<int64_t>(B, std::min<int64_t>(M * B, (32ll << 20) / (4 * H)));
+  q->P_bf16 = (q->P + 7) & ~7ll;
+  const int64_t rows = q->rows;
+  alloc((void **)&q->wbf, sizeof(__nv_bfloat16) * M * q->P_bf16);
   q->h.assign(q->L, nullptr);
   q->z.assign(q->L - 1, nullptr);
-  alloc((void **)&q->h[0], sizeof(__nv_bfloat16) * B * cfg->n_in);
-  for (int l = 1; l < q->L; ++l) alloc((void **)&q->h[l], sizeof(__nv_bfloat16) * B * H);
-  for (int l = 0; l < q->L - 1; ++l) alloc((void **)&q->z[l], sizeof(float) * B * H);
-  alloc((void **)&q->dz[0], sizeof(__nv_bfloat16) * B * H);
-  alloc((void **)&q->dz[1], sizeof(__nv_bfloat16) * B * H);
+  for (int l = 1; l < q->L; ++l) alloc((void **)&q->h[l], sizeof(__nv_bfloat16) * rows * H);
+  for (int l = 0; l < q->L - 1; ++l) alloc((void **)&q->z[l], sizeof(float) * rows * H);
   alloc((void **)&q->out, sizeof(float) * M * B);
-  alloc((void **)&q->gout, sizeof(float) * B);
+  alloc((void **)&q->gout, sizeof(float) * rows);
   alloc((void **)&q->lo_hi, sizeof(float) * 10);
   alloc((void **)&q->off_dev, sizeof(int64_t) * (q->L + 1));
   alloc((void **)&q->fin_dev, sizeof(int) * q->L);
@@ -551,8 +973,10 @@ sde_status sde_mlp_forward(sde_mlp *q, const float *X, int64_t B, float *mean, f
     mlptc::mlp_fwd_tc_kernel<<<grid, mlptc::THREADS, mlptc::SMEM_BYTES, s>>>(q->map_whh, a);
     SDE_CUDA_TRY(cudaGetLastError());
   } else {
-    for (int mm = 0; mm < q->cfg.n_members; ++mm) {
-      sde_status st = mlp_forward_member(q, mm, X, B, q->out + (int64_t)mm * q->cfg.max_batch, s);
+    const int64_t G = member_group(q, B);
+    for (int64_t mm = 0; mm < q->cfg.n_members; mm += G) {
+      sde_status st =
+          mlp_forward_members(q, mm, std::min<int64_t>(G, q->cfg.n_members - mm), X, 0, B, nullptr, 0, s);
       if (st != SDE_OK) return st;
     }
   }
@@ -568,7 +992,7 @@ sde_status sde_mlp_grad(sde_mlp *q, int32_t member, const float *X, const float 
   SDE_CHECK_ARG(member >= 0 && member < q->cfg.n_members, "member out of range");
   SDE_CHECK_ARG(B >= 1 && B <= q->cfg.max_batch, "batch must be in [1, max_batch]");
   SDE_CHECK_ARG(X && y && grad, "X, y and grad must be non-NULL");
-  return mlp_grad_member(q, member, X, y, B, grad, loss, (cudaStream_t)stream);
+  return mlp_grad_members(q, member, 1, X, 0, y, 0, B, grad, loss, (cudaStream_t)stream);
 }
 
 sde_status sde_mlp_use_tensor_cores(sde_mlp *q, int32_t enable) {
@@ -610,11 +1034,10 @@ static sde_status mlp_train(sde_mlp *q, const float *X, const float *y, int64_t 
   SDE_CHECK_ARG(B >= 1 && B <= q->cfg.max_batch, "batch must be in [1, max_batch]");
   SDE_CHECK_ARG(X && y, "X and y must be non-NULL");
   cudaStream_t s = (cudaStream_t)stream;
-  for (int mm = 0; mm < q->cfg.n_members; ++mm) {
-    const int64_t xo = per_member ? (int64_t)mm * B * q->cfg.n_in : 0;
-    const int64_t yo = per_member ? (int64_t)mm * B : 0;
-    sde_status st = mlp_grad_member(q, mm, X + xo, y + yo, B, q->grad + (int64_t)mm * q->P,
-                                    loss ? loss + mm : nullptr, s);
+  const int64_t G = member_group(q, B), x_member = per_member ? B * q->cfg.n_in : 0, y_member = per_member ? B : 0;
+  for (int64_t mm = 0; mm < q->cfg.n_members; mm += G) {
+    sde_status st = mlp_grad_members(q, mm, std::min<int64_t>(G, q->cfg.n_members - mm), X + mm * x_member, x_member,
+                                     y + mm * y_member, y_member, B, q->grad + mm * q->P, loss ? loss + mm : nullptr, s);
     if (st != SDE_OK) return st;
   }
   q->step += 1;

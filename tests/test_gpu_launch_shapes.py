@@ -1,5 +1,7 @@
 """Launch shapes at the edges of their ranges: tiles with remainders, the
 smallest sizes, every branch of a size rule."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -34,3 +36,31 @@ def test_pairwise_shapes_match_mean_field(N, R, euler):
     phi_mf, r_mf, _ = kur_run(mf, w["phi0"], w["omega"], 0, 5)
     assert np.abs(angle_diff(phi, phi_mf)).max() <= 1e-6
     assert np.abs(r - r_mf).max() <= 2e-5
+
+
+@pytest.mark.parametrize("hidden,n_hidden,n_in,B,max_batch", [
+    (64, 1, 1, 1, 1), (256, 3, 5, 63, 64), (256, 3, 5, 65, 4096), (320, 2, 8, 129, 129), (256, 2, 7, 20000, 20000)])
+def test_members_train_together_as_alone(hidden, n_hidden, n_in, B, max_batch):
+    """Members share launches (in groups where their batches fill the activation
+    rows: the last case): each ends bit for bit where it ends alone."""
+    ensure_built()
+    rng = np.random.default_rng(B)
+    M = 3
+    X = torch.from_numpy(rng.uniform(-1, 1, (M, B, n_in)).astype(np.float32)).cuda()
+    y = torch.sin(2 * X[..., 0]).contiguous()
+    kw = dict(n_in=n_in, hidden=hidden, n_hidden=n_hidden, max_batch=max_batch)
+    both = sde.Mlp(members=M, seed=5, **kw)
+    alone = []
+    for q in range(M):
+        m = sde.Mlp(members=1, seed=1, **kw)
+        m.set_params(0, both.get_params(q))
+        alone.append(m)
+    loss = torch.zeros(M, device="cuda")
+    for _ in range(2):
+        both.train_step_members(X, y, loss)
+        for q, m in enumerate(alone):
+            l1 = torch.zeros(1, device="cuda")
+            m.train_step(X[q].contiguous(), y[q].contiguous(), l1)
+            assert l1.item() == loss[q].item() and math.isfinite(l1.item())
+    for q, m in enumerate(alone):
+        assert torch.equal(both.get_params(q), m.get_params(0))
