@@ -66,9 +66,17 @@ __global__ void kg_operand_kernel(const uint32_t *theta, T *op, int64_t N) {
 // loaded before any arithmetic, so each thread keeps several loads in flight.
 constexpr int kStageIlp = 4;
 
+// The GEMM output at idx: the sum of its `planes` partial sums, plane stride
+// `stride` (one plane unless the FP32 GEMM split K).
+__device__ __forceinline__ float plane_sum(const float *__restrict__ Dt, int64_t idx, int planes, int64_t stride) {
+  float s = Dt[idx];
+  for (int p = 1; p < planes; ++p) s += Dt[p * stride + idx];
+  return s;
+}
+
 template <int STAGE, typename T>
-__global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__ Dt, const tc::StageArgs a,
-                                                       T *op_next) {
+__global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__ Dt, int planes,
+                                                       const tc::StageArgs a, T *op_next) {
   const int64_t r = blockIdx.y;
   const int64_t N = a.N;
   const int64_t i0 = (int64_t)blockIdx.x * (256 * kStageIlp) + threadIdx.x;
@@ -82,8 +90,8 @@ __global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__
     ok[u] = i < N;
     const int64_t ii = ok[u] ? i : 0;
     const int64_t idx = r * N + ii;
-    ps[u] = Dt[(2 * r) * N + ii];
-    pc[u] = Dt[(2 * r + 1) * N + ii];
+    ps[u] = plane_sum(Dt, (2 * r) * N + ii, planes, 2 * a.NR);
+    pc[u] = plane_sum(Dt, (2 * r + 1) * N + ii, planes, 2 * a.NR);
     th[u] = a.theta[idx];
     th_s[u] = STAGE == 0 ? th[u] : a.theta_t[idx];
     om[u] = a.omega[idx];
@@ -102,13 +110,16 @@ __global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__
 }
 
 // Coupling sums alone: out[r][i] = cos x_i Dt[2r][i] - sin x_i Dt[2r+1][i].
-__global__ void kg_coupling_kernel(const float *__restrict__ Dt, const uint32_t *theta, float *out, int64_t N) {
+__global__ void kg_coupling_kernel(const float *__restrict__ Dt, int planes, const uint32_t *theta, float *out,
+                                   int64_t N) {
   const int64_t r = blockIdx.y;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   float s, c;
   sincos_turns(theta[r * N + i], s, c);
-  out[r * N + i] = c * Dt[(2 * r) * N + i] - s * Dt[(2 * r + 1) * N + i];
+  const int64_t stride = 2 * N * gridDim.y;
+  out[r * N + i] = c * plane_sum(Dt, (2 * r) * N + i, planes, stride) -
+                   s * plane_sum(Dt, (2 * r + 1) * N + i, planes, stride);
 }
 
 __global__ void kg_to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t n) {
@@ -117,84 +128,178 @@ __global__ void kg_to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t 
 }
 
 // ---- FP32 CUDA-core GEMM (baseline): Dt[c][i] = sum_j K[i][j] B[c][j] ----
-// 128 x 128 tile per block of 256 threads, 8 x 8 outputs per thread, K
-// slices of 8 staged (transposed) in shared memory, double buffered.
-constexpr int SG_BM = 128, SG_BN = 128, SG_BK = 8;
+//
+// One CTA of 128 threads: 256 rows x 8 TN columns of D over a share of K, 16 x
+// TN outputs per thread as packed FP32 pairs along the rows.  K slices of 8
+// are staged transposed in shared memory, double buffered, the next slice's
+// global loads in flight during the current slice's FMAs and each k's
+// fragments read while the previous k is multiplied.  Partial sums of a K
+// split go to planes of Dt and are added by the kernel that reads them.
+// What bounds it: shared memory returns 128 bytes per cycle to the SM's four
+// schedulers, 4 (16 + TN) cycles per k against 16 TN cycles of packed FMAs, so
+// the FMA pipe is the limit from TN = 6 up; and how evenly the tiles fill the
+// GPU (sgemm_shape).  3000 x 200 x 3000: 109 us (33 TFLOP/s; 42 % of the FMA
+// pipe, waiting for the global loads of a slice) against 538 us for 128 x 128
+// tiles of scalar FMAs, which gave 48 CTAs; with the columns stored as (b, b)
+// pairs in shared memory 232 us (its return path at 130 % of the FMA time).
+constexpr int SG_BM = 256, SG_BK = 8, SG_THREADS = 128, SG_TM = 16;
 
-__global__ void __launch_bounds__(256) sgemm_nt_kernel(const float *__restrict__ A, const float *__restrict__ B,
-                                                       float *__restrict__ Dt, int M, int Ncols, int Kdim) {
-  __shared__ float As[2][SG_BK][SG_BM];
-  __shared__ float Bs[2][SG_BK][SG_BN];
+struct SgemmShape {
+  int tn = 0;     // columns per thread
+  int split = 1;  // K shares (planes of Dt)
+  int kshare = 0; // K per share, a multiple of SG_BK
+};
+
+template <int TN>
+__global__ void __launch_bounds__(SG_THREADS, TN <= 7 ? 2 : 1)
+    sgemm_nt_kernel(const float *__restrict__ A, const float *__restrict__ B, float *__restrict__ Dt, int M, int Ncols,
+                    int Kdim, int kshare) {
+  constexpr int BN = 8 * TN;
+  constexpr int NB = (BN * SG_BK / 4 + SG_THREADS - 1) / SG_THREADS;  // float4 loads of B per thread
+  __shared__ __align__(16) float As[2][SG_BK][SG_BM + 4];
+  __shared__ float Bs[2][SG_BK][BN + 4];
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;  // 16 x 16 threads
-  const int m0 = blockIdx.x * SG_BM, n0 = blockIdx.y * SG_BN;
-  // loader mapping: 128 rows x 8 k = 256 float4: row = tid >> 1, k4 = (tid & 1) * 4
-  const int lr = tid >> 1, lk = (tid & 1) * 4;
-  const float *Ap = A + (size_t)(m0 + lr) * Kdim + lk;
-  const float *Bp = B + (size_t)(n0 + lr) * Kdim + lk;
-  const bool a_ok = (m0 + lr) < M, b_ok = (n0 + lr) < Ncols;
-  float acc[8][8];
+  const int tx = tid & 7, ty = tid >> 3;  // columns tx + 8 j; rows 64 i + 4 ty .. + 3, i = 0 .. 3
+  const int m0 = blockIdx.x * SG_BM, n0 = blockIdx.y * BN;
+  const int kb = blockIdx.z * kshare, ke = min(kb + kshare, Kdim);
+  const bool ok0 = m0 + tid < M, ok1 = m0 + 128 + tid < M;
+  const float *A0 = A + (size_t)(ok0 ? m0 + tid : 0) * Kdim, *A1 = A + (size_t)(ok1 ? m0 + 128 + tid : 0) * Kdim;
+  float4 ra[4], rb[NB];
+  // Kdim and kshare are multiples of 8: a slice lies wholly inside or outside
+  auto load = [&](int k0) {
+    const float4 zero = make_float4(0, 0, 0, 0);
+    ra[0] = ok0 ? *(const float4 *)(A0 + k0) : zero;
+    ra[1] = ok0 ? *(const float4 *)(A0 + k0 + 4) : zero;
+    ra[2] = ok1 ? *(const float4 *)(A1 + k0) : zero;
+    ra[3] = ok1 ? *(const float4 *)(A1 + k0 + 4) : zero;
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+    for (int q = 0; q < NB; ++q) {
+      const int c = tid + q * SG_THREADS, n = c >> 1;
+      rb[q] = (n < BN && n0 + n < Ncols) ? *(const float4 *)(B + (size_t)(n0 + n) * Kdim + k0 + 4 * (c & 1)) : zero;
+    }
+  };
+  auto store = [&](int buf) {
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
-  float4 ra = a_ok ? *(const float4 *)Ap : make_float4(0, 0, 0, 0);
-  float4 rb = b_ok ? *(const float4 *)Bp : make_float4(0, 0, 0, 0);
-  int buf = 0;
-  As[0][lk + 0][lr] = ra.x;
-  As[0][lk + 1][lr] = ra.y;
-  As[0][lk + 2][lr] = ra.z;
-  As[0][lk + 3][lr] = ra.w;
-  Bs[0][lk + 0][lr] = rb.x;
-  Bs[0][lk + 1][lr] = rb.y;
-  Bs[0][lk + 2][lr] = rb.z;
-  Bs[0][lk + 3][lr] = rb.w;
-  __syncthreads();
-  for (int k0 = 0; k0 < Kdim; k0 += SG_BK) {
-    const bool more = k0 + SG_BK < Kdim;
-    if (more) {
-      ra = a_ok ? *(const float4 *)(Ap + k0 + SG_BK) : make_float4(0, 0, 0, 0);
-      rb = b_ok ? *(const float4 *)(Bp + k0 + SG_BK) : make_float4(0, 0, 0, 0);
+    for (int q = 0; q < 4; ++q) {
+      const int m = tid + 128 * (q >> 1), k = 4 * (q & 1);
+      As[buf][k + 0][m] = ra[q].x;
+      As[buf][k + 1][m] = ra[q].y;
+      As[buf][k + 2][m] = ra[q].z;
+      As[buf][k + 3][m] = ra[q].w;
     }
 #pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int c = tid + q * SG_THREADS, n = c >> 1, k = 4 * (c & 1);
+      if (n < BN) {
+        Bs[buf][k + 0][n] = rb[q].x;
+        Bs[buf][k + 1][n] = rb[q].y;
+        Bs[buf][k + 2][n] = rb[q].z;
+        Bs[buf][k + 3][n] = rb[q].w;
+      }
+    }
+  };
+  float2 acc[SG_TM / 2][TN];
+#pragma unroll
+  for (int i = 0; i < SG_TM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+  load(kb);
+  store(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = kb; k0 < ke; k0 += SG_BK) {
+    const bool more = k0 + SG_BK < ke;
+    if (more) load(k0 + SG_BK);
+    float4 fa[2][4];
+    float fb[2][TN];
+    auto frag = [&](int q, int kk) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) fa[q][i] = *(const float4 *)&As[buf][kk][64 * i + 4 * ty];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) fb[q][j] = Bs[buf][kk][tx + 8 * j];
+    };
+    frag(0, 0);
+#pragma unroll
     for (int kk = 0; kk < SG_BK; ++kk) {
-      float a[8], b[8];
-      const float4 a0 = *(const float4 *)&As[buf][kk][ty * 4];
-      const float4 a1 = *(const float4 *)&As[buf][kk][64 + ty * 4];
-      const float4 b0 = *(const float4 *)&Bs[buf][kk][tx * 4];
-      const float4 b1 = *(const float4 *)&Bs[buf][kk][64 + tx * 4];
-      a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-      a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-      b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
-      b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+      if (kk + 1 < SG_BK) frag((kk + 1) & 1, kk + 1);
+      const float4 (&a)[4] = fa[kk & 1];
 #pragma unroll
-      for (int x = 0; x < 8; ++x)
+      for (int j = 0; j < TN; ++j) {
+        const float2 b = make_float2(fb[kk & 1][j], fb[kk & 1][j]);
 #pragma unroll
-        for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(a[x], b[y], acc[x][y]);
+        for (int i = 0; i < 4; ++i) {
+          acc[2 * i][j] = __ffma2_rn(make_float2(a[i].x, a[i].y), b, acc[2 * i][j]);
+          acc[2 * i + 1][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), b, acc[2 * i + 1][j]);
+        }
+      }
     }
     if (more) {
       buf ^= 1;
-      As[buf][lk + 0][lr] = ra.x;
-      As[buf][lk + 1][lr] = ra.y;
-      As[buf][lk + 2][lr] = ra.z;
-      As[buf][lk + 3][lr] = ra.w;
-      Bs[buf][lk + 0][lr] = rb.x;
-      Bs[buf][lk + 1][lr] = rb.y;
-      Bs[buf][lk + 2][lr] = rb.z;
-      Bs[buf][lk + 3][lr] = rb.w;
+      store(buf);
       __syncthreads();
     }
   }
-  // rows of this thread: m0 + {ty*4 .. ty*4+3, 64+ty*4 .. 64+ty*4+3}; columns likewise with tx
+  float *D = Dt + (size_t)blockIdx.z * Ncols * M;
 #pragma unroll
-  for (int y = 0; y < 8; ++y) {
-    const int col = n0 + (y < 4 ? tx * 4 + y : 64 + tx * 4 + (y - 4));
+  for (int j = 0; j < TN; ++j) {
+    const int col = n0 + tx + 8 * j;
     if (col >= Ncols) continue;
-    float *dst = Dt + (size_t)col * M;
-    const int r0 = m0 + ty * 4, r1 = m0 + 64 + ty * 4;
-    if (r0 + 3 < M) *(float4 *)(dst + r0) = make_float4(acc[0][y], acc[1][y], acc[2][y], acc[3][y]);
-    if (r1 + 3 < M) *(float4 *)(dst + r1) = make_float4(acc[4][y], acc[5][y], acc[6][y], acc[7][y]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + 64 * i + 4 * ty;  // M is a multiple of 8
+      if (m < M)
+        *(float4 *)(D + (size_t)col * M + m) =
+            make_float4(acc[2 * i][j].x, acc[2 * i][j].y, acc[2 * i + 1][j].x, acc[2 * i + 1][j].y);
+    }
   }
+}
+
+constexpr int kSgemmTn[] = {1, 2, 3, 5, 7, 8};
+constexpr int kSgemmMaxSplit = 16;
+
+// Columns per thread and K shares of the FP32 GEMM for M x Ncols outputs, by
+// the cycles of the busiest SM: its tile shares times the cycles per k (the
+// larger of 16 TN of packed FMAs and 4 (16 + TN) of shared-memory return, and
+// a sixth more where a single share leaves one warp per scheduler); a share
+// costs about 24 more k's for its prologue and epilogue, and every plane of
+// partial sums its write and read (8 bytes per output at 24 bytes per cycle
+// and SM).
+SgemmShape sgemm_shape(int64_t M, int64_t Ncols, int64_t Kdim, int sm_count) {
+  SgemmShape best;
+  double t_best = 0.0;
+  for (int tn : kSgemmTn) {
+    const int64_t tiles = ((M + SG_BM - 1) / SG_BM) * ((Ncols + 8 * tn - 1) / (8 * tn));
+    for (int s = 1; s <= kSgemmMaxSplit; ++s) {
+      const int64_t share = ((Kdim + s - 1) / s + SG_BK - 1) / SG_BK * SG_BK;
+      if (s > 1 && (share < 64 || share * (s - 1) >= Kdim || (s - 1) * M * Ncols * 4 > (256ll << 20))) break;
+      const double per_sm = (double)((tiles * s + sm_count - 1) / sm_count);
+      const double cyc = std::max(16.0 * tn, 4.0 * (SG_TM + tn)) * (tiles * s <= sm_count ? 1.17 : 1.0);
+      const double t = per_sm * cyc * (double)(share + 24) +
+                       (double)s * (double)M * (double)Ncols * 8.0 / (24.0 * sm_count);
+      if (best.tn == 0 || t < t_best) {
+        best.tn = tn;
+        best.split = s;
+        best.kshare = (int)share;
+        t_best = t;
+      }
+    }
+  }
+  return best;
+}
+
+cudaError_t launch_sgemm(const SgemmShape &p, const float *A, const float *B, float *Dt, int M, int Ncols, int Kdim,
+                         cudaStream_t s) {
+  const dim3 grid((M + SG_BM - 1) / SG_BM, (Ncols + 8 * p.tn - 1) / (8 * p.tn), p.split);
+  switch (p.tn) {
+    case 1: sgemm_nt_kernel<1><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 2: sgemm_nt_kernel<2><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 3: sgemm_nt_kernel<3><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 5: sgemm_nt_kernel<5><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 7: sgemm_nt_kernel<7><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 8: sgemm_nt_kernel<8><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
 }
 
 constexpr int64_t kTimedStepStride = 8;
@@ -213,6 +318,7 @@ struct GemmPlan {
   CUtensorMap mapK;
   CUtensorMap mapOp[2];  // box of bn rows (one CTA's tile)
   CUtensorMap mapOpHalf[2];  // box of 128 rows (one CTA's half of a pair tile)
+  SgemmShape sg;      // FP32 GEMM
   int bn = 0;
   bool pair = false;  // CTA-pair GEMM (tc_gemm2_bf16_kernel)
   tc::EpiMaps em;     // pair GEMM: the SRK2 state its fused epilogue loads by TMA
@@ -339,10 +445,9 @@ cudaError_t launch_gemm(KuramotoCtx *k, int which, cudaStream_t s, int epi = tc:
     if (epi == tc::EPI_STAGE1) return launch_tc<128, tc::EPI_STAGE1>(k, which, sa, s);
     return launch_tc<128, tc::EPI_STORE_D>(k, which, sa, s);
   } else {
-    dim3 grid((M + SG_BM - 1) / SG_BM, (Ncols + SG_BN - 1) / SG_BN);
-    sgemm_nt_kernel<<<grid, 256, 0, s>>>(k->Kf32, (const float *)op_buf(k, which), k->P, M, Ncols, Kdim);
+    return launch_sgemm(((GemmPlan *)k->gemm_plan)->sg, k->Kf32, (const float *)op_buf(k, which), k->P, M, Ncols, Kdim,
+                        s);
   }
-  return cudaGetLastError();
 }
 
 dim3 grid_nr(const KuramotoCtx *k) { return dim3((unsigned)((k->N + 255) / 256), (unsigned)k->R); }
@@ -364,9 +469,11 @@ cudaError_t launch_stage(KuramotoCtx *k, int next, const float *omega, int64_t n
                          cudaStream_t s) {
   const tc::StageArgs a = stage_args(k, next, omega, n, run_begin);
   if (is_tc(k))
-    kg_stage_kernel<STAGE, __nv_bfloat16><<<grid_stage(k), 256, 0, s>>>(k->P, a, (__nv_bfloat16 *)op_buf(k, next));
+    kg_stage_kernel<STAGE, __nv_bfloat16>
+        <<<grid_stage(k), 256, 0, s>>>(k->P, 1, a, (__nv_bfloat16 *)op_buf(k, next));
   else
-    kg_stage_kernel<STAGE, float><<<grid_stage(k), 256, 0, s>>>(k->P, a, (float *)op_buf(k, next));
+    kg_stage_kernel<STAGE, float><<<grid_stage(k), 256, 0, s>>>(k->P, ((GemmPlan *)k->gemm_plan)->sg.split, a,
+                                                               (float *)op_buf(k, next));
   return cudaGetLastError();
 }
 
@@ -389,13 +496,14 @@ sde_status kuramoto_general_alloc(KuramotoCtx *k) {
   cudaError_t e;
   if ((e = device_alloc((void **)&k->theta_t, NR * 4)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   if ((e = device_alloc((void **)&k->g1, NR * 4)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-  if ((e = device_alloc((void **)&k->P, NR * 2 * 4)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+  GemmPlan *g = new GemmPlan();
+  k->gemm_plan = g;
+  if (!is_tc(k)) g->sg = sgemm_shape(k->N, 2 * k->R, k->N, k->sm_count);
+  if ((e = device_alloc((void **)&k->P, NR * 2 * 4 * g->sg.split)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   if ((e = device_alloc((void **)&k->psi4, NR * 8 * sizeof(float))) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   if (is_tc(k)) {
     if ((e = device_alloc((void **)&k->Kbf16, NN * 2)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = device_alloc((void **)&k->Bt, NR * 2 * 2 * 2)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    GemmPlan *g = new GemmPlan();
-    k->gemm_plan = g;
     g->bn = (2 * k->R) % 256 == 0 ? 256 : 128;
     g->pair = k->N % 256 == 0 && (2 * k->R) % tc::BN2 == 0 && !(k->flags & SDE_FLAG_GEMM_SINGLE_CTA);
     sde_status st = make_map(&g->mapK, k->Kbf16, k->N, k->N, tc::BM);
@@ -473,8 +581,8 @@ sde_status kuramoto_general_alloc(KuramotoCtx *k) {
     if ((e = device_alloc((void **)&k->Kf32, NN * 4)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = device_alloc((void **)&k->Bt32, NR * 2 * 4 * 2)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   }
-  k->block = is_tc(k) ? tc::THREADS : 256;
-  k->opt = is_tc(k) ? ((GemmPlan *)k->gemm_plan)->bn : SG_BN;
+  k->block = is_tc(k) ? tc::THREADS : SG_THREADS;
+  k->opt = is_tc(k) ? g->bn : 8 * g->sg.tn;
   if (is_tc(k)) {
     const GemmPlan *g = (const GemmPlan *)k->gemm_plan;
     // CTAs per GEMM tile (0: stream-K, the split grid's CTA count in opt)
@@ -569,7 +677,7 @@ sde_status kuramoto_general_coupling(KuramotoCtx *k, float *out, cudaStream_t s)
   }
   SDE_CUDA_TRY(launch_operand(k, 0, s));
   SDE_CUDA_TRY(launch_gemm(k, 0, s));
-  kg_coupling_kernel<<<grid_nr(k), 256, 0, s>>>(k->P, k->theta, out, k->N);
+  kg_coupling_kernel<<<grid_nr(k), 256, 0, s>>>(k->P, ((GemmPlan *)k->gemm_plan)->sg.split, k->theta, out, k->N);
   SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }

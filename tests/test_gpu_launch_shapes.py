@@ -38,6 +38,24 @@ def test_pairwise_shapes_match_mean_field(N, R, euler):
     assert np.abs(r - r_mf).max() <= 2e-5
 
 
+@pytest.mark.parametrize("N,R", [(8, 1), (16, 3), (136, 13), (264, 25), (512, 100), (1000, 7), (3000, 28)])
+def test_fp32_gemm_shapes(N, R):
+    """Coupling sums of the FP32 form against FP64: every chain of N FMAs errs by
+    at most N 2^-24 sum|K_ij| (the sines by 2^-23 each)."""
+    ensure_built()
+    w = inputs.kuramoto_general(n_osc=N, replicas=R, seed=N)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_GENERAL_FP32, N, R, 0.0, 0.02, 0.005, 1)
+    K = torch.from_numpy(w["Kmat"]).cuda()
+    ens.set_coupling(K)
+    phi = torch.from_numpy(w["phi0"]).cuda()
+    got = ens.coupling(phi).double()
+    x, Kt = phi.double(), K.double().t()
+    s, c = torch.sin(x), torch.cos(x)
+    ref = c * (s @ Kt) - s * (c @ Kt)
+    bound = 2.0 * (N + 8) * 2.0 ** -24 * K.double().abs().sum(1)
+    assert torch.all((got - ref).abs() <= bound)
+
+
 @pytest.mark.parametrize("hidden,n_hidden,n_in,B,max_batch", [
     (64, 1, 1, 1, 1), (256, 3, 5, 63, 64), (256, 3, 5, 65, 4096), (320, 2, 8, 129, 129), (256, 2, 7, 20000, 20000)])
 def test_members_train_together_as_alone(hidden, n_hidden, n_in, B, max_batch):
