@@ -268,7 +268,9 @@ void sde_debug_fail_allocation(int32_t nth);
 const char *sde_last_error(void);
 
 /* Launch shape chosen at create (after autotuning): threads per block, paths
-   (Josephson; values 11 and 12 mean 1 and 2 with registers capped at 64) or
+   (Josephson; values 11 and 12 mean 1 and 2 with registers capped at 64, 21
+   one path per thread with its noise drawn by a second warp, the shape of
+   small ensembles) or
    oscillators (Kuramoto) per thread, and CTAs per replica (the thread-block
    cluster of the mean-field kernel; 0 for the grid-wide mean field, whose
    per-thread count is then the oscillators each thread strides over; for the

@@ -49,6 +49,7 @@ struct sde_ctx {
   Moments *partials = nullptr;
   uint32_t *queue = nullptr;
   int block = 0, ilp = 0;
+  bool ws_ok = false;  // the points suit the warp-pair kernel
   // ---- Kuramoto ----
   KuramotoCtx *kur = nullptr;
   // ---- common ----
@@ -56,6 +57,8 @@ struct sde_ctx {
   int64_t n_obs_rows = 0;
   int64_t max_obs_rows = 0;
   uint32_t *err = nullptr;
+  void *stage = nullptr;  // pinned host memory: the error word, then observable rows
+  size_t stage_bytes = 0;
   cudaStream_t last_stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool timed = false;
@@ -117,6 +120,7 @@ void free_ctx(sde_ctx *c) {
   cudaFree(c->queue);
   cudaFree(c->obs);
   cudaFree(c->err);
+  cudaFreeHost(c->stage);
   kuramoto_destroy(c->kur);
   delete c;
 }
@@ -145,6 +149,7 @@ sde_status build_units(sde_ctx *c, int ilp) {
       units.push_back(u);
     }
     L.point_range_h[p] = make_int2(first, (int)units.size());
+    L.max_units = std::max(L.max_units, (int32_t)units.size() - first);
   }
   L.n_units = (int32_t)units.size();
   SDE_CUDA_TRY(dmalloc(&L.units, units.size()));
@@ -204,9 +209,13 @@ sde_status jj_enqueue(sde_ctx *c, const sde_run_desc *r, cudaStream_t s, int ilp
   if (time_it) SDE_CUDA_TRY(record(c->ev0, s, capturing));
   if (c->cfg.schedule == SDE_SCHED_PERSISTENT) {
     if (L.n_units > 0) {
-      SDE_CUDA_TRY(cudaMemsetAsync(c->queue, 0, sizeof(uint32_t), s));
-      a.queue = c->queue;
-      SDE_CUDA_TRY(jj_launch(a, ilp, block, persistent_grid(c, ilp, block), s));
+      if (ilp % 100 == kJJWarpPairs) {
+        SDE_CUDA_TRY(jj_launch(a, ilp, block, jj_ws_grid(L.n_units), s));
+      } else {
+        SDE_CUDA_TRY(cudaMemsetAsync(c->queue, 0, sizeof(uint32_t), s));
+        a.queue = c->queue;
+        SDE_CUDA_TRY(jj_launch(a, ilp, block, persistent_grid(c, ilp, block), s));
+      }
     }
   } else {
     const int warps = block / 32;
@@ -220,7 +229,7 @@ sde_status jj_enqueue(sde_ctx *c, const sde_run_desc *r, cudaStream_t s, int ilp
     }
   }
   if (time_it) SDE_CUDA_TRY(record(c->ev1, s, capturing));
-  SDE_CUDA_TRY(jj_finalize(c->consts, L.point_range, c->n_points, c->partials, r->n_end, c->obs, s));
+  SDE_CUDA_TRY(jj_finalize(c->consts, L.point_range, c->n_points, L.max_units, c->partials, r->n_end, c->obs, s));
   return SDE_OK;
 }
 
@@ -248,6 +257,12 @@ sde_status jj_autotune(sde_ctx *c) {
   else
     il = {2, 4, 12, 14};  // one path per thread never wins; it stays selectable
   // Euler-Maruyama kernels carry the variant code + 100
+  if (!fixed_block && !fixed_ilp && c->cfg.schedule == SDE_SCHED_PERSISTENT && c->ws_ok &&
+      c->units[1].n_units <= kWsUnitsPerSm * c->sm_count) {
+    c->block = jj_ws_block();
+    c->ilp = kJJWarpPairs + ((c->cfg.flags & SDE_FLAG_EULER) ? 100 : 0);
+    return SDE_OK;
+  }
   const int scheme = (c->cfg.flags & SDE_FLAG_EULER) ? 100 : 0;
   for (int b : bl)
     for (int i : il) cand.push_back({b, i + scheme});
@@ -370,6 +385,7 @@ sde_status create_josephson(sde_ctx *c, const sde_config *cfg) {
     off += cfg->paths[p];
   }
   c->total_paths = off;
+  c->ws_ok = jj_ws_eligible(cfg->points, cfg->n_points, cfg->steps_per_period);
   SDE_CUDA_TRY(jj_configure());
 
   // the point and step tables are needed only by the prepare kernel: freed
@@ -552,16 +568,38 @@ sde_status sde_run_ensemble(sde_ctx *c, const sde_run_desc *r, void *stream) {
   return SDE_OK;
 }
 
+constexpr int64_t kStageRows = 4096;
+constexpr size_t kStageHead = 16;  // the error word, padded
+
 sde_status sde_observables(sde_ctx *c, sde_obs_row *rows, int64_t capacity, int64_t *n_rows) {
   clear_error();
   SDE_CHECK_ARG(c != nullptr, "ctx is NULL");
   SDE_CHECK_ARG(capacity >= 0 && (rows != nullptr || capacity == 0), "rows/capacity");
-  SDE_CUDA_TRY(cudaStreamSynchronize(c->last_stream));
   const int64_t n = std::min<int64_t>(capacity, c->n_obs_rows);
-  if (n > 0) SDE_CUDA_TRY(cudaMemcpy(rows, c->obs, sizeof(sde_obs_row) * n, cudaMemcpyDeviceToHost));
+  // The error word and the rows come back behind the run in one wait, through
+  // pinned memory kept with the context (up to kStageRows rows; more rows than
+  // that are copied by themselves).
+  const int64_t staged = std::min<int64_t>(n, kStageRows);
+  const size_t need = kStageHead + sizeof(sde_obs_row) * (size_t)staged;
+  if (c->stage_bytes < need) {
+    cudaFreeHost(c->stage);
+    c->stage = nullptr;
+    c->stage_bytes = 0;
+    SDE_CUDA_TRY(cudaHostAlloc(&c->stage, need, cudaHostAllocDefault));
+    c->stage_bytes = need;
+  }
+  char *stage = (char *)c->stage;
+  SDE_CUDA_TRY(cudaMemcpyAsync(stage, c->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->last_stream));
+  if (staged > 0)
+    SDE_CUDA_TRY(cudaMemcpyAsync(stage + kStageHead, c->obs, sizeof(sde_obs_row) * staged, cudaMemcpyDeviceToHost,
+                                 c->last_stream));
+  SDE_CUDA_TRY(cudaStreamSynchronize(c->last_stream));
+  if (staged > 0) memcpy(rows, stage + kStageHead, sizeof(sde_obs_row) * staged);
+  if (n > staged)
+    SDE_CUDA_TRY(cudaMemcpy(rows + staged, c->obs + staged, sizeof(sde_obs_row) * (n - staged), cudaMemcpyDeviceToHost));
   if (n_rows) *n_rows = c->n_obs_rows;
   uint32_t err = 0;
-  SDE_CUDA_TRY(cudaMemcpy(&err, c->err, sizeof(uint32_t), cudaMemcpyDeviceToHost));
+  memcpy(&err, stage, sizeof(uint32_t));
   // a latched device status is reported once, then cleared for later runs
   if (err) SDE_CUDA_TRY(cudaMemset(c->err, 0, sizeof(uint32_t)));
   if (err & kErrTimeout) {

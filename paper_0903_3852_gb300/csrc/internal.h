@@ -46,6 +46,7 @@ struct Moments {
 struct JJUnitList {
   int ilp = 0;
   int32_t n_units = 0;
+  int32_t max_units = 0;  // of one point
   JJUnit *units = nullptr;          // device, ordered longest-first
   int2 *point_range = nullptr;      // device, [n_points]: unit range of each point
   std::vector<int2> point_range_h;  // host copy
@@ -76,14 +77,25 @@ struct JJLaunchArgs {
   PhiloxKeys keys;  // round keys of seed
 };
 
+// Launch variant of the small-ensemble kernel (one path per thread, its noise
+// drawn by a second warp).
+constexpr int kJJWarpPairs = 21;
+// Up to this many units of 32 paths per SM that kernel is taken.  Fig. 2's
+// point, 4000 steps, against the fastest other kernel: 166 vs 430 us at 2 units
+// per SM and below, 214 vs 431 at 4, 370 vs 432 at 8, 615 vs 592 at 12.
+constexpr int kWsUnitsPerSm = 8;
+
 // Kernel launchers (josephson.cu).
+bool jj_ws_eligible(const sde_jj_point *pts, int n_points, int P);
+int jj_ws_grid(int n_units);
+int jj_ws_block();
 cudaError_t jj_prepare(const sde_jj_point *points_dev, int n_points, int P, const int64_t *steps_dev,
                        const int64_t *offsets_dev, const int64_t *paths_dev, JJConsts *consts_dev,
                        float *drive_dev, cudaStream_t s);
 cudaError_t jj_launch(const JJLaunchArgs &a, int ilp, int block, int grid, cudaStream_t s);
 int jj_max_blocks_per_sm(int ilp, int block, int P);
 cudaError_t jj_configure();  // once per process, before the first launch (not under capture)
-cudaError_t jj_finalize(const JJConsts *consts, const int2 *point_range, int n_points,
+cudaError_t jj_finalize(const JJConsts *consts, const int2 *point_range, int n_points, int max_units,
                         const Moments *partials, int64_t n_end, sde_obs_row *obs, cudaStream_t s);
 
 // Histograms (histogram.cu).

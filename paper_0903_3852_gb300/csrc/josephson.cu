@@ -33,6 +33,7 @@
 #include <mutex>
 #include <string>
 
+#include "cos2pi64.cuh"
 #include "internal.h"
 #include "philox.cuh"
 
@@ -327,6 +328,37 @@ __device__ __forceinline__ double warp_sum(double a) {
   return a;
 }
 
+// Moments of the per-path window averages of a unit, after step n_end.
+template <int ILP>
+__device__ __forceinline__ void jj_unit_moments(Moments *out, int64_t n_end, const JJConsts &c,
+                                                const double (&vs)[ILP], const bool (&valid)[ILP], int lane) {
+  const int64_t reach = n_end < c.steps ? n_end : c.steps;
+  const int64_t wcount = reach > c.wstart ? reach - c.wstart : 0;
+  double cnt = 0.0, sum = 0.0;
+  if (wcount > 0) {
+#pragma unroll
+    for (int i = 0; i < ILP; ++i)
+      if (valid[i]) {
+        cnt += 1.0;
+        sum += vs[i] / (double)wcount;
+      }
+  }
+  cnt = warp_sum(cnt);
+  sum = warp_sum(sum);
+  const double mean = cnt > 0.0 ? sum / cnt : 0.0;
+  double m2 = 0.0;
+  if (wcount > 0) {
+#pragma unroll
+    for (int i = 0; i < ILP; ++i)
+      if (valid[i]) {
+        const double d = vs[i] / (double)wcount - mean;
+        m2 += d * d;
+      }
+  }
+  m2 = warp_sum(m2);
+  if (lane == 0) *out = Moments{cnt, mean, m2};
+}
+
 template <int ILP, bool EM, bool ONEBB = false>
 __device__ __forceinline__ void jj_unit(const JJLaunchArgs &A, int u, const float *drive, float *wtab,
                                         const float *bm_tab, int lane) {
@@ -394,32 +426,7 @@ __device__ __forceinline__ void jj_unit(const JJLaunchArgs &A, int u, const floa
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(A.err, kErrNonFinite);
 
-  // Moments of the per-path window averages of this unit.
-  const int64_t reach = A.n_end < c.steps ? A.n_end : c.steps;
-  const int64_t wcount = reach > c.wstart ? reach - c.wstart : 0;
-  double cnt = 0.0, sum = 0.0;
-  if (wcount > 0) {
-#pragma unroll
-    for (int i = 0; i < ILP; ++i)
-      if (valid[i]) {
-        cnt += 1.0;
-        sum += vs[i] / (double)wcount;
-      }
-  }
-  cnt = warp_sum(cnt);
-  sum = warp_sum(sum);
-  const double mean = cnt > 0.0 ? sum / cnt : 0.0;
-  double m2 = 0.0;
-  if (wcount > 0) {
-#pragma unroll
-    for (int i = 0; i < ILP; ++i)
-      if (valid[i]) {
-        const double d = vs[i] / (double)wcount - mean;
-        m2 += d * d;
-      }
-  }
-  m2 = warp_sum(m2);
-  if (lane == 0) A.partials[u] = Moments{cnt, mean, m2};
+  jj_unit_moments<ILP>(A.partials + u, A.n_end, c, vs, valid, lane);
 }
 
 template <int ILP, bool EM, bool ONEBB = false>
@@ -482,6 +489,274 @@ __global__ void __maxnreg__(96) jj_kernel_packed4_cap96(const JJLaunchArgs A) {
   jj_kernel_body<4, EM, true>(A);
 }
 
+// ---- small ensembles: steps and noise in different warps -------------------
+//
+// With fewer warps than schedulers a launch lasts as long as one path's chain
+// of dependent operations, and there the noise, which depends on no state, is
+// better drawn elsewhere: a CTA holds kPairs pairs of warps, one stepping 32
+// paths, the other drawing their Gaussians ahead into a ring of two blocks of
+// 64 steps (named barriers hand the blocks over; blocks of 32 steps: 197 us
+// where 64 take 164).  Four warps per CTA, so that
+// each has a scheduler to itself.  The chain of a step is 13 FP32 operations
+// (x -> force -> v~ -> x'), 52 cycles; rint(x) on it is taken as (x + 1.5
+// 2^23) - 1.5 2^23, the same value for |x| < 2^22 in two additions where the
+// conversion unit takes longer, and a group's floor(x) from two comparisons.  The steps' values and roundings are those of
+// the one-path kernel: bit-identical.
+// 1024 paths, 20,000 steps: 0.82 ms (85 cycles per step, 73 of them the chain)
+// against 2.19 ms for the fastest kernel that draws and steps in one warp.
+constexpr int kPairs = 2;               // stepping warps per CTA
+constexpr int kWsBlock = 64 * kPairs;
+constexpr uint32_t kRingGroups = 16;    // groups of 4 steps per ring block (aligned to 64 steps)
+constexpr float kRoundMagic = 12582912.0f;
+// Largest |v| at a group's start for which x moves by less than one period in
+// the group's steps and predictors, so that floor(x) is -1, 0 or 1 (and |x|
+// far below 2^22): over four steps |v| grows to at most q^4 (|v| + 4 kick), q =
+// 1 + 2 gamma dt, kick = twice a step's largest force and noise (a 24-bit
+// uniform's Gaussian is below 5.8).
+__host__ __device__ inline double jj_ws_vmax(double gamma, double a, double f, double dt, double s) {
+  const double q = 1.0 + 2.0 * gamma * dt, q4 = q * q * q * q;
+  const double kick = 2.0 * (dt * (6.2832 + fabs(a) + fabs(f)) + 5.8 * s);
+  return 0.98 / (5.0 * dt * q4) - 4.0 * kick;
+}
+
+__device__ __forceinline__ float jj_force_lat(float x, float A) {
+  const float b = 0.25f - fabsf(x - __fsub_rn(__fadd_rn(x, kRoundMagic), kRoundMagic));
+  const float s = b * b;
+  float p = -2.484164429e+02f;  // as in jj_force
+  p = fmaf(p, s, 4.809764709e+02f);
+  p = fmaf(p, s, -5.127142334e+02f);
+  p = fmaf(p, s, 2.597572937e+02f);
+  p = fmaf(p, s, -3.947841644e+01f);
+  return fmaf(b, p, A);
+}
+
+template <bool ACC, bool EM>
+__device__ __forceinline__ void jj_step_lat(float &x, float &v, float &acc, float z, const JJConsts &c, float e0,
+                                            float e1) {
+  const float vn = fmaf(c.s, z, v);
+  const float F1 = jj_force_lat(x, fmaf(-c.gamma, v, e0));
+  if (EM) {
+    x = fmaf(c.dt, v, x);
+    v = fmaf(c.dt, F1, vn);
+    if (ACC) acc += v;
+    return;
+  }
+  const float xt = fmaf(c.dt, v, x);
+  const float vt = fmaf(c.dt, F1, vn);
+  const float F2 = jj_force_lat(xt, fmaf(-c.gamma, vt, e1));
+  x = fmaf(c.h, v + vt, x);
+  v = fmaf(c.h, F1 + F2, vn);
+  if (ACC) acc += v;
+}
+
+__device__ __forceinline__ void pair_bar_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+
+// A whole group: four steps, then x back into [0, 1) knowing that it moved by
+// less than one period (the same x and w as jj_wrap).
+template <bool ACC, bool EM>
+__device__ __forceinline__ void jj_ws_group(float &x, int &w, float &v, float &acc, const float4 &z, const JJConsts &c,
+                                            const float4 &d, float d4) {
+  jj_step_lat<ACC, EM>(x, v, acc, z.x, c, d.x, d.y);
+  jj_step_lat<ACC, EM>(x, v, acc, z.y, c, d.y, d.z);
+  jj_step_lat<ACC, EM>(x, v, acc, z.z, c, d.z, d.w);
+  jj_step_lat<ACC, EM>(x, v, acc, z.w, c, d.w, d4);
+  const float up = __fsub_rn(x, 1.0f), dn = __fadd_rn(x, 1.0f);
+  const bool hi = x >= 1.0f, lo = x < 0.0f;
+  w += (hi ? 1 : 0) - (lo ? 1 : 0);
+  x = hi ? up : (lo ? dn : x);
+}
+
+// A whole ring block on one side of the window's start.  Returns
+// whether every group started with |v| <= vmax (warp-uniform); if not the
+// caller repeats the block group by group.
+template <bool ACC, bool EM>
+__device__ __forceinline__ bool jj_ws_block_steps(float &x, int &w, float &v, float &acc, const float4 *zr,
+                                                  const JJConsts &c, const float *tab, int P, int &k, float vmax) {
+  bool bad = false;
+  float4 z = zr[0], d = *reinterpret_cast<const float4 *>(tab + k);
+  float d4 = tab[k + 4];
+#pragma unroll 4
+  for (uint32_t g = 0; g < kRingGroups; ++g) {
+    // the next group's noise and drive, read during this group's steps
+    k = k + 4 == P ? 0 : k + 4;
+    const float4 zn = zr[((g + 1) & (kRingGroups - 1)) * 32], dn = *reinterpret_cast<const float4 *>(tab + k);
+    const float d4n = tab[k + 4];
+    bad |= !(fabsf(v) <= vmax);
+    jj_ws_group<ACC, EM>(x, w, v, acc, z, c, d, d4);
+    z = zn;
+    d = dn;
+    d4 = d4n;
+  }
+  return !__any_sync(0xffffffffu, bad);
+}
+
+// The steps of one group at its ends: those in [n0, n1), then those in [m0,
+// m1) with the window sum, x folded after each part (as two jj_segment calls
+// meeting inside the group do).
+template <bool EM>
+__device__ __forceinline__ void jj_ws_partial(float &x, int &w, float &v, float &acc, const float4 &z4,
+                                              const JJConsts &c, const float *drive, int P, int &k, int64_t base,
+                                              int64_t n0, int64_t n1, int64_t m0, int64_t m1) {
+  const float z[4] = {z4.x, z4.y, z4.z, z4.w};
+  bool any0 = false, any1 = false;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int64_t n = base + s;
+    if (n >= n0 && n < n1) {
+      const int kn = k + 1 == P ? 0 : k + 1;
+      jj_step<false, EM>(x, v, acc, z[s], c, drive[k], drive[kn]);
+      k = kn;
+      any0 = true;
+    }
+  }
+  if (any0) jj_wrap(x, w);
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int64_t n = base + s;
+    if (n >= m0 && n < m1) {
+      const int kn = k + 1 == P ? 0 : k + 1;
+      jj_step<true, EM>(x, v, acc, z[s], c, drive[k], drive[kn]);
+      k = kn;
+      any1 = true;
+    }
+  }
+  if (any1) jj_wrap(x, w);
+}
+
+// The unit of a pair of warps and the run's steps.
+struct JJWsUnit {
+  int32_t path_begin, n_paths;  // within the point
+  uint32_t point;
+  int64_t offset;               // of its first path in the state arrays
+  int64_t n_begin, n_end;
+};
+
+// One warp of a pair (`steps`: the stepping one) over its unit; tab holds the
+// point's drive table, ring the pair's Gaussians.
+template <bool EM>
+__device__ __forceinline__ void jj_ws_pair(const JJWsUnit &r, const JJConsts &c, const JJState &st,
+                                           const PhiloxKeys &keys, int P, const float *tab, const float *bm_tab,
+                                           float4 (*ring)[kRingGroups][32], int pair, bool steps, uint32_t *err,
+                                           Moments *out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nb = r.n_begin, ne = r.n_end < c.steps ? r.n_end : c.steps;
+  const uint32_t g0 = (uint32_t)(nb >> 2), g1 = ne > nb ? (uint32_t)((ne - 1) >> 2) : g0;
+  const uint32_t nblk = ne > nb ? g1 / kRingGroups - g0 / kRingGroups + 1u : 0u;
+  const int bar_full = 1 + 4 * pair, bar_empty = 3 + 4 * pair;
+  if (!steps) {
+    // ---- noise ----
+    const uint32_t pid = (uint32_t)(r.path_begin + lane);
+    for (uint32_t i = 0; i < nblk; ++i) {
+      const int b = (int)(i & 1u);
+      const uint32_t lo = i == 0 ? g0 : (g0 / kRingGroups + i) * kRingGroups;
+      const uint32_t hi = i + 1 == nblk ? g1 : (lo | (kRingGroups - 1u));
+      if (i >= 2) pair_bar_sync(bar_empty + b);
+#pragma unroll 2
+      for (uint32_t g = lo; g <= hi; ++g) {
+        const uint4 wd = philox4x32_10(make_uint4(g, pid, r.point, kTagJosephson), keys);
+        float2 z02, z13;
+        box_muller_tab2(wd.x, wd.y, wd.z, wd.w, bm_tab, z02, z13);
+        ring[b][g % kRingGroups][lane] = make_float4(z02.x, z13.x, z02.y, z13.y);
+      }
+      pair_bar_arrive(bar_full + b);
+    }
+    return;
+  }
+  // ---- steps ----
+  const bool valid[1] = {lane < r.n_paths};
+  const int64_t gi = r.offset + lane;
+  float x = 0.0f, v = 0.0f;
+  int w = 0;
+  double vs[1] = {0.0};
+  if (valid[0]) {
+    x = st.x_in[gi];
+    v = st.v_in[gi];
+    if (st.w_in) w = st.w_in[gi];
+    if (st.vsum_in) vs[0] = st.vsum_in[gi];
+  }
+  jj_wrap(x, w);
+  float acc = 0.0f;
+  int k = (int)(nb % P);
+  const int64_t ws = c.wstart;
+  const float vmax = (float)jj_ws_vmax(c.gamma, c.a, c.f, c.dt64, c.s);
+  for (uint32_t i = 0; i < nblk; ++i) {
+    const int b = (int)(i & 1u);
+    const uint32_t lo = i == 0 ? g0 : (g0 / kRingGroups + i) * kRingGroups;
+    const uint32_t hi = i + 1 == nblk ? g1 : (lo | (kRingGroups - 1u));
+    const float4 *zr = &ring[b][0][lane];
+    pair_bar_sync(bar_full + b);
+    const int64_t n0 = (int64_t)lo << 2, n1 = ((int64_t)hi + 1) << 2;
+    bool done = false;
+    if (n0 >= nb && n1 <= ne && lo % kRingGroups == 0u && hi % kRingGroups == kRingGroups - 1u && (ws <= n0 || ws >= n1)) {
+      const float x0 = x, v0 = v, acc0 = acc;
+      const int w0 = w, k0 = k;
+      done = ws <= n0 ? jj_ws_block_steps<true, EM>(x, w, v, acc, zr, c, tab, P, k, vmax)
+                      : jj_ws_block_steps<false, EM>(x, w, v, acc, zr, c, tab, P, k, vmax);
+      if (!done) {
+        x = x0;
+        v = v0;
+        acc = acc0;
+        w = w0;
+        k = k0;
+      }
+    }
+    if (!done) {
+      for (uint32_t g = lo; g <= hi; ++g) {
+        const int64_t m0 = (int64_t)g << 2, m1 = m0 + 4;
+        const float4 z = zr[(g % kRingGroups) * 32];
+        if (m0 >= nb && m1 <= ne && (ws <= m0 || ws >= m1) && !__any_sync(0xffffffffu, !(fabsf(v) <= vmax))) {
+          const float4 d = *reinterpret_cast<const float4 *>(tab + k);
+          if (ws <= m0)
+            jj_ws_group<true, EM>(x, w, v, acc, z, c, d, tab[k + 4]);
+          else
+            jj_ws_group<false, EM>(x, w, v, acc, z, c, d, tab[k + 4]);
+          k = k + 4 == P ? 0 : k + 4;
+        } else {
+          jj_ws_partial<EM>(x, w, v, acc, z, c, tab, P, k, m0, nb, ne < ws ? ne : ws, nb > ws ? nb : ws, ne);
+        }
+      }
+    }
+    if (i + 2 < nblk) pair_bar_arrive(bar_empty + b);
+    if (((hi + 1u) & 15u) == 0u) {  // flush at absolute 64-step boundaries, as jj_segment
+      vs[0] += (double)acc;
+      acc = 0.0f;
+    }
+  }
+  vs[0] += (double)acc;
+  if (valid[0]) {
+    st.x_out[gi] = x;
+    st.v_out[gi] = v;
+    st.w_out[gi] = w;
+    st.vsum_out[gi] = vs[0];
+  }
+  if (err && __any_sync(0xffffffffu, valid[0] && !(isfinite(x) && isfinite(v))) && lane == 0)
+    atomicOr(err, kErrNonFinite);
+  jj_unit_moments<1>(out, r.n_end, c, vs, valid, lane);
+}
+
+template <bool EM>
+__global__ void __launch_bounds__(kWsBlock) jj_ws_kernel(const JJLaunchArgs A) {
+  extern __shared__ float4 drive_s4[];  // per pair: a cos(2 pi k / P) + f, k = 0 .. P + 3
+  __shared__ float bm_tab[2 * kBmTable];
+  __shared__ float4 ring[kPairs][2][kRingGroups][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int pair = warp % kPairs;
+  const bool steps = warp < kPairs;
+  const int u = A.unit_begin + (int)blockIdx.x * kPairs + pair;
+  const bool have = u < A.unit_end;
+  const JJUnit un = A.units[have ? u : A.unit_begin];
+  const JJConsts c = A.consts[un.point];
+  float *tab = reinterpret_cast<float *>(drive_s4) + jj_table_stride(A.P) * pair;
+  if (steps)
+    for (int q = lane; q < A.P + 4; q += 32) tab[q] = fmaf(c.a, A.drive[q < A.P ? q : q % A.P], c.f);
+  fill_bm_table(bm_tab);
+  __syncthreads();
+  if (!have) return;
+  const JJWsUnit r{un.path_begin, un.n_paths, (uint32_t)un.point, c.path_offset + un.path_begin, A.n_begin, A.n_end};
+  jj_ws_pair<EM>(r, c, A.st, A.keys, A.P, tab, bm_tab, ring[pair], pair, steps, A.err, A.partials + u);
+}
+
 __global__ void jj_prepare_kernel(const sde_jj_point *pts, int n_points, int P,
                                   const int64_t *steps, const int64_t *offsets,
                                   const int64_t *paths, JJConsts *out, float *drive) {
@@ -507,43 +782,62 @@ __global__ void jj_prepare_kernel(const sde_jj_point *pts, int n_points, int P,
   if (t < P) drive[t] = (float)cospi(2.0 * (double)t / (double)P);
 }
 
-// Merge of two (n, mean, M2) triples (Chan, Golub & LeVeque 1979).
-__device__ __forceinline__ Moments merge(const Moments &a, const Moments &b) {
-  const double n = a.n + b.n;
-  if (n == 0.0) return Moments{0.0, 0.0, 0.0};
-  const double d = b.mean - a.mean;
-  return Moments{n, a.mean + d * (b.n / n), a.m2 + b.m2 + d * d * (a.n * b.n / n)};
+// FP64 sum over the block in a fixed order; every thread receives it.
+__device__ __forceinline__ double block_sum64(double a, double *red) {
+  a = warp_sum(a);
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  if (warps == 1) return a;
+  __syncthreads();
+  if (lane == 0) red[threadIdx.x >> 5] = a;
+  __syncthreads();
+  return warp_sum(lane < warps ? red[lane] : 0.0);
 }
 
-// One warp per point: lane-strided merge over the point's units in a fixed
-// order, then a fixed shuffle tree (deterministic result).
-__global__ void jj_finalize_kernel(const JJConsts *consts, const int2 *range, int n_points,
-                                   const Moments *partials, int64_t n_end, sde_obs_row *obs) {
-  const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (p >= n_points) return;
-  const int2 r = range[p];
-  Moments m{0.0, 0.0, 0.0};
-  for (int u = r.x + lane; u < r.y; u += 32) m = merge(m, partials[u]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Moments q;
-    q.n = __shfl_down_sync(0xffffffffu, m.n, o);
-    q.mean = __shfl_down_sync(0xffffffffu, m.mean, o);
-    q.m2 = __shfl_down_sync(0xffffffffu, m.m2, o);
-    if (lane + o < 32) m = merge(m, q);
+// The observables of one point from the moments of its units [u0, u1), by one
+// block: mean = sum n_i mean_i / n, then M2 = sum m2_i + n_i (mean_i - mean)^2
+// (deterministic: fixed strides and tree).  Two passes with one division
+// instead of a pairwise merge per unit, whose two FP64 divisions took ~1.2 us
+// each on one lane's chain: 1,000,000 paths through the allocation-free entry
+// point, 1000 steps, 2.99 -> 1.59 ms together with its packed kernels.
+__device__ __forceinline__ void jj_point_row(const Moments *partials, int u0, int u1, int64_t steps, double dt,
+                                             int64_t n_end, sde_obs_row *out, double *red) {
+  double n = 0.0, sum = 0.0;
+  for (int u = u0 + (int)threadIdx.x; u < u1; u += blockDim.x) {
+    const Moments m = partials[u];
+    n += m.n;
+    sum = fma(m.n, m.mean, sum);
   }
-  if (lane == 0) {
-    const JJConsts c = consts[p];
-    const int64_t reach = n_end < c.steps ? n_end : c.steps;
+  n = block_sum64(n, red);
+  sum = block_sum64(sum, red);
+  const double mean = n > 0.0 ? sum / n : 0.0;
+  double m2 = 0.0;
+  for (int u = u0 + (int)threadIdx.x; u < u1; u += blockDim.x) {
+    const Moments m = partials[u];
+    const double d = m.mean - mean;
+    m2 += fma(m.n * d, d, m.m2);
+  }
+  m2 = block_sum64(m2, red);
+  if (threadIdx.x == 0) {
+    const int64_t reach = n_end < steps ? n_end : steps;
     sde_obs_row row;
-    row.count = m.n;
-    row.mean = m.n > 0.0 ? m.mean : 0.0;
-    row.var = m.n > 1.0 ? m.m2 / (m.n - 1.0) : 0.0;
-    row.se = m.n > 0.0 ? sqrt(row.var / m.n) : 0.0;
-    row.t = (double)reach * c.dt64;
-    obs[p] = row;
+    row.count = n;
+    row.mean = mean;
+    row.var = n > 1.0 ? m2 / (n - 1.0) : 0.0;
+    row.se = n > 0.0 ? sqrt(row.var / n) : 0.0;
+    row.t = (double)reach * dt;
+    *out = row;
   }
+}
+
+// Threads of a block over n_units units: a warp for a few, more where the
+// strided loop would be long.
+int jj_row_threads(int n_units) { return n_units <= 64 ? 32 : (n_units <= 1024 ? 256 : 1024); }
+
+__global__ void jj_finalize_kernel(const JJConsts *consts, const int2 *range, const Moments *partials, int64_t n_end,
+                                   sde_obs_row *obs) {
+  __shared__ double red[32];
+  const int p = blockIdx.x;
+  jj_point_row(partials, range[p].x, range[p].y, consts[p].steps, consts[p].dt64, n_end, obs + p, red);
 }
 
 __global__ void philox_fill_kernel(const uint4 *ctr, uint2 key, uint4 *out, int64_t n) {
@@ -582,6 +876,8 @@ __global__ void box_muller_words_kernel(const uint2 *w, int64_t n, int variant, 
   }
 }
 
+size_t jj_ws_smem(int P) { return sizeof(float) * (size_t)jj_table_stride(P) * kPairs; }
+
 void *jj_kernel_ptr(int variant) {
   switch (variant) {
     case 1: return (void *)jj_kernel<1>;
@@ -596,6 +892,8 @@ void *jj_kernel_ptr(int variant) {
     case 111: return (void *)jj_kernel_cap64<1, true>;
     case 112: return (void *)jj_kernel_cap64<2, true>;
     case 114: return (void *)jj_kernel_packed4_cap96<true>;
+    case kJJWarpPairs: return (void *)jj_ws_kernel<false>;
+    case 100 + kJJWarpPairs: return (void *)jj_ws_kernel<true>;
   }
   return nullptr;
 }
@@ -611,8 +909,27 @@ cudaError_t jj_prepare(const sde_jj_point *points_dev, int n_points, int P, cons
   return cudaGetLastError();
 }
 
+int jj_ws_grid(int n_units) { return (n_units + kPairs - 1) / kPairs; }
+int jj_ws_block() { return kWsBlock; }
+
+// The warp-pair kernel takes drive tables of whole groups that fit a warp's
+// table, and points whose velocities leave the block path (jj_ws_vmax) rarely:
+// the driven velocity is of the order of a / omega + f / gamma and the noise's
+// sqrt(D), a few of each.
+bool jj_ws_eligible(const sde_jj_point *pts, int n_points, int P) {
+  if (P % 4 != 0 || P > kWarpTableMaxP) return false;
+  for (int i = 0; i < n_points; ++i) {
+    const sde_jj_point &p = pts[i];
+    const double dt = 2.0 * 3.14159265358979323846 / (p.omega * (double)P);
+    const double vmax = jj_ws_vmax(p.gamma, p.a, p.f, dt, sqrt(2.0 * p.gamma * p.D * dt));
+    if (!(vmax >= 2.0 * (fabs(p.a) / p.omega + fabs(p.f) / p.gamma + 6.0 * sqrt(p.D)) + 3.0)) return false;
+  }
+  return true;
+}
+
 // `ilp` encodes the variant: 1, 2, 4 = paths per thread; +10 = fewer registers
-// (64 for 1 and 2 paths per thread, 96 for 4); +100 = Euler-Maruyama.
+// (64 for 1 and 2 paths per thread, 96 for 4); kJJWarpPairs = one path per
+// thread, the noise drawn by a second warp; +100 = Euler-Maruyama.
 cudaError_t jj_launch(const JJLaunchArgs &a, int ilp, int block, int grid, cudaStream_t s) {
   const size_t smem = jj_smem_bytes(a.P, block);
   switch (ilp) {
@@ -629,6 +946,8 @@ cudaError_t jj_launch(const JJLaunchArgs &a, int ilp, int block, int grid, cudaS
     case 111: jj_kernel_cap64<1, true><<<grid, block, smem, s>>>(a); break;
     case 112: jj_kernel_cap64<2, true><<<grid, block, smem, s>>>(a); break;
     case 114: jj_kernel_packed4_cap96<true><<<grid, block, smem, s>>>(a); break;
+    case kJJWarpPairs: jj_ws_kernel<false><<<grid, kWsBlock, jj_ws_smem(a.P), s>>>(a); break;
+    case 100 + kJJWarpPairs: jj_ws_kernel<true><<<grid, kWsBlock, jj_ws_smem(a.P), s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -659,11 +978,9 @@ cudaError_t jj_configure() {
   return status;
 }
 
-cudaError_t jj_finalize(const JJConsts *consts, const int2 *point_range, int n_points,
+cudaError_t jj_finalize(const JJConsts *consts, const int2 *point_range, int n_points, int max_units,
                         const Moments *partials, int64_t n_end, sde_obs_row *obs, cudaStream_t s) {
-  const int wpb = 8;
-  jj_finalize_kernel<<<(n_points + wpb - 1) / wpb, 32 * wpb, 0, s>>>(consts, point_range, n_points,
-                                                                    partials, n_end, obs);
+  jj_finalize_kernel<<<n_points, jj_row_threads(max_units), 0, s>>>(consts, point_range, partials, n_end, obs);
   return cudaGetLastError();
 }
 
@@ -715,107 +1032,115 @@ namespace {
 static __device__ __align__(256) Moments g_noalloc_partials[SDE_NOALLOC_UNITS];
 
 struct NoallocArgs {
-  sde_jj_point p;
+  JJConsts c;
+  double inv4P;  // 1 / (4 P)
   int32_t P;
   int32_t n_paths;
-  int64_t steps;
   int64_t n_begin, n_end;
-  uint64_t seed;
   PhiloxKeys keys;
   JJState st;
   Moments *partials;  // device address of g_noalloc_partials
 };
 
-// One warp per 32 paths, one path per thread: the same arithmetic and the same
-// unit decomposition as the plain schedule with one path per thread.
-__global__ void __launch_bounds__(256) jj_noalloc_kernel(const NoallocArgs A) {
-  extern __shared__ float4 drive_s4[];
+// cos(2 pi k / P) rounded to FP32, k in [0, P]: sin(2 pi b) with b = 1/4 - min(k, P
+// - k) / P, whose numerator is an exact integer.
+__device__ __forceinline__ float drive_entry(int k, int P, double inv4P) {
+  const int kk = k <= P - k ? k : P - k;
+  const double b = (double)(P - 4 * kk) * inv4P;
+  return (float)(b * sin2pi64_poly(b * b));
+}
+
+// ILP paths per thread (2 or 4, packed pairs as in the persistent kernels), the moments taken per 32 paths as with one path per thread: the
+// same arithmetic and unit decomposition as the plain schedule with one path
+// per thread whatever ILP.
+template <int ILP>
+__device__ __forceinline__ void jj_noalloc_body(const NoallocArgs &A) {
+  extern __shared__ float4 drive_s4[];  // a cos(2 pi k / P) + f, k = 0 .. P + 3
   __shared__ float bm_tab[2 * kBmTable];
   float *drive_s = reinterpret_cast<float *>(drive_s4);
-  const double dt = 2.0 * 3.14159265358979323846 / (A.p.omega * (double)A.P);
+  const JJConsts &c = A.c;
   for (int i = threadIdx.x; i < A.P + 4; i += blockDim.x)
-    drive_s[i] = (float)cospi(2.0 * (double)(i % A.P) / (double)A.P);
+    drive_s[i] = fmaf(c.a, drive_entry(i % A.P, A.P, A.inv4P), c.f);
   fill_bm_table(bm_tab);
   __syncthreads();
-  JJConsts c;
-  c.gamma = (float)A.p.gamma;
-  c.a = (float)A.p.a;
-  c.f = (float)A.p.f;
-  c.dt = (float)dt;
-  c.h = (float)(0.5 * dt);
-  c.s = (float)sqrt(2.0 * A.p.gamma * A.p.D * dt);
-  c.paths = A.n_paths;
-  c.pad = 0;
-  c.steps = A.steps;
-  c.wstart = A.steps - A.steps / 2;
-  c.path_offset = 0;
-  c.dt64 = dt;
-  const int u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int u = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * ILP;  // first unit of 32 paths
   const int n_units = (A.n_paths + 31) / 32;
   if (u >= n_units) return;
   const int lane = threadIdx.x & 31;
-  const PhiloxKeys &key = A.keys;
-  const int j = u * 32 + lane;
-  const bool valid = j < A.n_paths;
-  float x[1] = {0.0f}, v[1] = {0.0f};
-  int w[1] = {0};
-  double vs[1] = {0.0};
-  const uint32_t pid[1] = {(uint32_t)j};
-  if (valid) {
-    x[0] = A.st.x_in[j];
-    v[0] = A.st.v_in[j];
-    if (A.st.w_in) w[0] = A.st.w_in[j];
-    if (A.st.vsum_in) vs[0] = A.st.vsum_in[j];
+  float x[ILP], v[ILP];
+  int w[ILP];
+  double vs[ILP];
+  uint32_t pid[ILP];
+  bool valid[ILP];
+#pragma unroll
+  for (int i = 0; i < ILP; ++i) {
+    const int j = (u + i) * 32 + lane;
+    valid[i] = j < A.n_paths;
+    pid[i] = (uint32_t)j;
+    x[i] = v[i] = 0.0f;
+    w[i] = 0;
+    vs[i] = 0.0;
+    if (valid[i]) {
+      x[i] = A.st.x_in[j];
+      v[i] = A.st.v_in[j];
+      if (A.st.w_in) w[i] = A.st.w_in[j];
+      if (A.st.vsum_in) vs[i] = A.st.vsum_in[j];
+    }
+    jj_wrap(x[i], w[i]);
   }
-  const float fl = floorf(x[0]);
-  x[0] -= fl;
-  w[0] += (int)fl;
   const int64_t ne = A.n_end < c.steps ? A.n_end : c.steps;
   if (A.n_begin < ne) {
     int k = (int)(A.n_begin % A.P);
     const int64_t split = ne < c.wstart ? ne : c.wstart;
-    jj_segment<1, false>(x, w, v, vs, c, drive_s, A.P, k, A.n_begin, split, key, pid, 0u, bm_tab);
-    jj_segment<1, true>(x, w, v, vs, c, drive_s, A.P, k, A.n_begin > c.wstart ? A.n_begin : c.wstart, ne,
-                        key, pid, 0u, bm_tab);
+    jj_segment<ILP, false, false, true, ILP >= 4>(x, w, v, vs, c, drive_s, A.P, k, A.n_begin, split, A.keys, pid, 0u,
+                                                  bm_tab);
+    jj_segment<ILP, true, false, true, ILP >= 4>(x, w, v, vs, c, drive_s, A.P, k,
+                                                 A.n_begin > c.wstart ? A.n_begin : c.wstart, ne, A.keys, pid, 0u,
+                                                 bm_tab);
   }
-  if (valid) {
-    A.st.x_out[j] = x[0];
-    A.st.v_out[j] = v[0];
-    A.st.w_out[j] = w[0];
-    A.st.vsum_out[j] = vs[0];
+#pragma unroll
+  for (int i = 0; i < ILP; ++i) {
+    if (valid[i]) {
+      const int j = (u + i) * 32 + lane;
+      A.st.x_out[j] = x[i];
+      A.st.v_out[j] = v[i];
+      A.st.w_out[j] = w[i];
+      A.st.vsum_out[j] = vs[i];
+    }
+    if (u + i < n_units) {
+      const double vsi[1] = {vs[i]};
+      const bool vi[1] = {valid[i]};
+      jj_unit_moments<1>(A.partials + u + i, A.n_end, c, vsi, vi, lane);
+    }
   }
-  const int64_t wcount = ne > c.wstart ? ne - c.wstart : 0;
-  const double m = (valid && wcount > 0) ? vs[0] / (double)wcount : 0.0;
-  const double cnt = warp_sum((valid && wcount > 0) ? 1.0 : 0.0);
-  const double mean = cnt > 0.0 ? warp_sum(m) / cnt : 0.0;
-  const double d = (valid && wcount > 0) ? m - mean : 0.0;
-  const double m2 = warp_sum(d * d);
-  if (lane == 0) A.partials[u] = Moments{cnt, mean, m2};
+}
+
+__global__ void __maxnreg__(72) jj_noalloc_packed2_kernel(const NoallocArgs A) { jj_noalloc_body<2>(A); }
+__global__ void __maxnreg__(96) jj_noalloc_packed4_kernel(const NoallocArgs A) { jj_noalloc_body<4>(A); }
+
+// Small ensembles: a pair of warps per 32 paths (jj_ws_pair).
+__global__ void __launch_bounds__(kWsBlock) jj_noalloc_ws_kernel(const NoallocArgs A) {
+  extern __shared__ float4 drive_s4[];
+  __shared__ float bm_tab[2 * kBmTable];
+  __shared__ float4 ring[kPairs][2][kRingGroups][32];
+  float *tab = reinterpret_cast<float *>(drive_s4);
+  const int pair = (threadIdx.x >> 5) % kPairs;
+  const bool steps = threadIdx.x < 32 * kPairs;
+  const JJConsts &c = A.c;
+  for (int i = threadIdx.x; i < A.P + 4; i += kWsBlock)
+    tab[i] = fmaf(c.a, drive_entry(i % A.P, A.P, A.inv4P), c.f);
+  fill_bm_table(bm_tab);
+  __syncthreads();
+  const int u = (int)blockIdx.x * kPairs + pair;
+  if (u >= (A.n_paths + 31) / 32) return;
+  const JJWsUnit r{u * 32, A.n_paths - u * 32 < 32 ? A.n_paths - u * 32 : 32, 0u, (int64_t)u * 32, A.n_begin, A.n_end};
+  jj_ws_pair<false>(r, c, A.st, A.keys, A.P, tab, bm_tab, ring[pair], pair, steps, nullptr, A.partials + u);
 }
 
 __global__ void jj_noalloc_finalize(const Moments *partials, int n_units, int64_t steps, double dt,
                                     int64_t n_end, sde_obs_row *obs) {
-  const int lane = threadIdx.x & 31;
-  Moments m{0.0, 0.0, 0.0};
-  for (int u = lane; u < n_units; u += 32) m = merge(m, partials[u]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Moments q;
-    q.n = __shfl_down_sync(0xffffffffu, m.n, o);
-    q.mean = __shfl_down_sync(0xffffffffu, m.mean, o);
-    q.m2 = __shfl_down_sync(0xffffffffu, m.m2, o);
-    if (lane + o < 32) m = merge(m, q);
-  }
-  if (lane == 0) {
-    const int64_t reach = n_end < steps ? n_end : steps;
-    sde_obs_row row;
-    row.count = m.n;
-    row.mean = m.n > 0.0 ? m.mean : 0.0;
-    row.var = m.n > 1.0 ? m.m2 / (m.n - 1.0) : 0.0;
-    row.se = m.n > 0.0 ? sqrt(row.var / m.n) : 0.0;
-    row.t = (double)reach * dt;
-    *obs = row;
-  }
+  __shared__ double red[32];
+  jj_point_row(partials, 0, n_units, steps, dt, n_end, obs, red);
 }
 
 }  // namespace
@@ -875,23 +1200,45 @@ extern "C" sde_status sde_josephson_run_noalloc(const sde_jj_point *point, int32
   }
   cudaStream_t s = (cudaStream_t)stream;
   NoallocArgs a{};
-  a.p = *point;
+  // the same FP64 expressions, rounded once, as jj_prepare_kernel
+  const double dt = 2.0 * 3.14159265358979323846 / (point->omega * (double)steps_per_period);
+  a.c.gamma = (float)point->gamma;
+  a.c.a = (float)point->a;
+  a.c.f = (float)point->f;
+  a.c.dt = (float)dt;
+  a.c.h = (float)(0.5 * dt);
+  a.c.s = (float)sqrt(2.0 * point->gamma * point->D * dt);
+  a.c.paths = (int32_t)n_paths;
+  a.c.steps = total_steps;
+  a.c.wstart = total_steps - total_steps / 2;
+  a.c.dt64 = dt;
+  a.inv4P = 1.0 / (4.0 * (double)steps_per_period);
   a.P = steps_per_period;
   a.n_paths = (int32_t)n_paths;
-  a.steps = total_steps;
   a.n_begin = n_begin;
   a.n_end = n_end;
-  a.seed = seed;
   a.keys = philox_round_keys(seed);
   a.st = JJState{x_in_dev, v_in_dev, w_in_dev, vsum_in_dev, x_out_dev, v_out_dev, w_out_dev, vsum_out_dev};
   a.partials = partials;
   const int n_units = (int)((n_paths + 31) / 32);
   if (n_units > 0) {
-    jj_noalloc_kernel<<<(n_units + 7) / 8, 256, sizeof(float) * (steps_per_period + 4), s>>>(a);
+    // Pairs of warps up to kWsUnitsPerSm units per SM as in the persistent
+    // schedule; then two paths per thread, and four where they still give each
+    // SM 20 warps (what 96 registers allow).  1000 steps against the scalar
+    // one-path kernel (both with the same reduction): 1000 paths 62 vs 101 us,
+    // 38,000 122 vs 150, 50,000 171 vs 210, 500,000 0.88 vs 1.15 ms.
+    int sms = 0;
+    SDE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const size_t smem = sizeof(float) * (size_t)(steps_per_period + 4);
+    if (n_units <= kWsUnitsPerSm * sms && jj_ws_eligible(point, 1, steps_per_period))
+      jj_noalloc_ws_kernel<<<jj_ws_grid(n_units), kWsBlock, smem, s>>>(a);
+    else if (n_units >= 4 * 20 * sms)
+      jj_noalloc_packed4_kernel<<<(n_units + 15) / 16, 128, smem, s>>>(a);
+    else
+      jj_noalloc_packed2_kernel<<<(n_units + 7) / 8, 128, smem, s>>>(a);
     SDE_CUDA_TRY(cudaGetLastError());
   }
-  const double dt = 2.0 * 3.14159265358979323846 / (point->omega * (double)steps_per_period);
-  jj_noalloc_finalize<<<1, 32, 0, s>>>(partials, n_units, total_steps, dt, n_end, obs_dev);
+  jj_noalloc_finalize<<<1, jj_row_threads(n_units), 0, s>>>(partials, n_units, total_steps, dt, n_end, obs_dev);
   SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }

@@ -82,3 +82,103 @@ def test_members_train_together_as_alone(hidden, n_hidden, n_in, B, max_batch):
             assert l1.item() == loss[q].item() and math.isfinite(l1.item())
     for q, m in enumerate(alone):
         assert torch.equal(both.get_params(q), m.get_params(0))
+
+
+FIG2 = dict(gamma=0.9, a=4.2, omega=4.9, f=0.1, D=1e-3)
+
+
+def _josephson(points, paths, steps, P, windows, x0, v0, flags=0, **kw):
+    n = int(np.sum(paths))
+    ens = sde.Ensemble.josephson(points, paths, steps, 7, steps_per_period=P, flags=flags, **kw)
+    x, v = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+    w = torch.empty(n, dtype=torch.int32, device="cuda")
+    vs = torch.empty(n, dtype=torch.float64, device="cuda")
+    xin, vin, more, n0 = x0, v0, {}, 0
+    for n1 in windows:
+        ens.run_josephson(n0, n1, xin, vin, x, v, w, vs, **more)
+        xin, vin, more, n0 = x, v, dict(w_in=w, vsum_in=vs), n1
+    return ens.tuning()[1], (x, v, w, vs), ens.observables()
+
+
+@pytest.mark.parametrize("paths,steps,P,windows,flags,v_scale", [
+    ([1024], [1000], 200, [1000], 0, 2.0),
+    ([1], [5], 200, [1, 3, 5], 0, 2.0),  # inside one group of four steps
+    ([100, 33, 64], [997, 1501, 64], 100, [63, 64, 65, 502, 1600], 0, 2.0),  # windows and their starts inside groups
+    ([70, 31], [400, 258], 200, [399, 400], sde.SDE_FLAG_EULER, 2.0),
+    ([96], [300], 1020, [300], 0, 2.0),  # the longest per-warp drive table
+    ([64], [200], 200, [200], 0, 60.0)])  # velocities beyond the block path's bound
+def test_small_ensembles_equal_the_one_warp_kernels(paths, steps, P, windows, flags, v_scale):
+    """The kernel of small ensembles (steps and noise in different warps) against
+    two paths per thread: states and window sums bit for bit, through the
+    allocation-free entry point as well; observables to rounding."""
+    ensure_built()
+    n = int(np.sum(paths))
+    rng = np.random.default_rng(n)
+    x0 = torch.from_numpy(rng.uniform(-1, 2, n).astype(np.float32)).cuda()
+    v0 = torch.from_numpy(rng.uniform(-v_scale, v_scale, n).astype(np.float32)).cuda()
+    points = [dict(FIG2, f=0.05 * i, D=1e-4 * 5 ** i) for i in range(len(paths))]
+    variant, a, obs_a = _josephson(points, paths, steps, P, windows, x0, v0, flags)
+    assert variant == 21
+    _, b, obs_b = _josephson(points, paths, steps, P, windows, x0, v0, flags, block_threads=128, paths_per_thread=2)
+    assert all(torch.equal(p, q) for p, q in zip(a, b))
+    assert np.allclose(obs_a["mean"], obs_b["mean"], rtol=1e-12, atol=1e-14)
+    assert np.allclose(obs_a["var"], obs_b["var"], rtol=1e-10, atol=1e-14)
+
+
+@pytest.mark.parametrize("n,P,steps", [(1, 200, 10), (333, 100, 130), (40000, 200, 66), (45000, 7, 33),
+                                       (400000, 200, 21)])
+def test_noalloc_kernels_equal_the_plain_schedule(n, P, steps):
+    """Every kernel of the allocation-free entry point (pairs of warps, two and
+    four paths per thread) against one path per thread, bit for bit."""
+    ensure_built()
+    rng = np.random.default_rng(n)
+    x0 = torch.from_numpy(rng.random(n).astype(np.float32)).cuda()
+    v0 = torch.from_numpy(rng.uniform(-2, 2, n).astype(np.float32)).cuda()
+    _, a, obs = _josephson([FIG2], [n], [steps], P, [steps], x0, v0, schedule=sde.SDE_SCHED_PLAIN, block_threads=256,
+                           paths_per_thread=1)
+    x, v, w, vs = (torch.empty_like(t) for t in a)
+    row = torch.empty(5, dtype=torch.float64, device="cuda")
+    sde.josephson_run_noalloc(FIG2, P, n, steps, 7, 0, steps, x0, v0, x, v, w, vs, row)
+    assert all(torch.equal(p, q) for p, q in zip(a, (x, v, w, vs)))
+    got = row.cpu().numpy()
+    assert np.allclose(got, [obs[k][0] for k in ("mean", "var", "se", "count", "t")], rtol=1e-10, atol=1e-14)
+
+
+@pytest.mark.parametrize("n,steps", [(1, 3), (65, 9), (5000, 40), (80000, 10)])
+def test_fp64_block_sizes(n, steps):
+    """Every block size of the FP64 kernel and windows inside a group of four
+    steps, against torch in FP64 (same Philox words through the library):
+    rounding of ~30 operations per step on values below ~10, 40 steps."""
+    ensure_built()
+    P, pt = 100, dict(FIG2, gamma=3.0)
+    rng = np.random.default_rng(n)
+    x = torch.from_numpy(rng.random(n)).cuda()
+    v = torch.from_numpy(rng.uniform(-2, 2, n)).cuda()
+    xo, vo, so = torch.empty_like(x), torch.empty_like(v), torch.empty_like(v)
+    sde.josephson_run_fp64(pt, P, steps, 5, 0, steps, x, v, xo, vo, vsum_out=so, point_index=2)
+    dt = 2 * math.pi / (pt["omega"] * P)
+    s, vsum = math.sqrt(2 * pt["gamma"] * pt["D"] * dt), torch.zeros_like(v)
+    ctr = torch.zeros((n, 4), dtype=torch.int32, device="cuda")
+    ctr[:, 1], ctr[:, 2], ctr[:, 3] = torch.arange(n, device="cuda"), 2, 1
+
+    def force(x, v, k):
+        return -pt["gamma"] * v - 2 * math.pi * torch.cos(2 * math.pi * x) + pt["a"] * math.cos(
+            2 * math.pi * (k % P) / P) + pt["f"]
+
+    for k in range(steps):
+        if k % 4 == 0:
+            ctr[:, 0] = k // 4
+            u = (((sde.philox4x32_10(ctr, 5).long() & 0xFFFFFFFF) >> 8) + 1).double() * 2.0 ** -24
+            z = []
+            for a, b in ((u[:, 0], u[:, 1]), (u[:, 2], u[:, 3])):
+                rho = torch.sqrt(-2 * torch.log(a))
+                z += [rho * torch.cos(2 * math.pi * b), rho * torch.sin(2 * math.pi * b)]
+        noise = s * z[k % 4]
+        F1 = force(x, v, k)
+        vt = v + dt * F1 + noise
+        F2 = force(x + dt * v, vt, k + 1)
+        x, v = x + 0.5 * dt * (v + vt), v + 0.5 * dt * (F1 + F2) + noise
+        if k + 1 > steps - steps // 2:
+            vsum = vsum + v
+    for got, ref in ((xo, x), (vo, v), (so, vsum)):
+        assert (got - ref).abs().max().item() <= 1e-12
