@@ -425,6 +425,10 @@ sde_status create_josephson(sde_ctx *c, const sde_config *cfg) {
   return jj_autotune(c);
 }
 
+// A run's launches: enqueued directly when its arguments differ from the last
+// run's, as a graph replay from the second identical run on.  Capturing and
+// instantiating a graph takes ~50 us of host time, which a call that is not
+// repeated (successive windows of one run) never earns back.
 sde_status run_graph(sde_ctx *c, const sde_run_desc *r, cudaStream_t s) {
   const bool same = c->gvalid && memcmp(&c->gdesc, r, sizeof(sde_run_desc)) == 0;
   if (!same) {
@@ -433,6 +437,15 @@ sde_status run_graph(sde_ctx *c, const sde_run_desc *r, cudaStream_t s) {
       c->gexec = nullptr;
     }
     c->gvalid = false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    SDE_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    const sde_status st = jj_enqueue(c, r, s, c->ilp, c->block, true, cap == cudaStreamCaptureStatusActive);
+    if (st != SDE_OK) return st;
+    c->gdesc = *r;
+    c->gvalid = true;
+    return SDE_OK;
+  }
+  if (!c->gexec) {
     cudaGraph_t g = nullptr;
     SDE_CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     sde_status st = jj_enqueue(c, r, c->cap_stream, c->ilp, c->block, true, true);
@@ -444,9 +457,10 @@ sde_status run_graph(sde_ctx *c, const sde_run_desc *r, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
     e = cudaGraphInstantiate(&c->gexec, g, 0);
     cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-    c->gdesc = *r;
-    c->gvalid = true;
+    if (e != cudaSuccess) {
+      c->gexec = nullptr;
+      return cuda_fail(e, "cudaGraphInstantiate");
+    }
   }
   SDE_CUDA_TRY(cudaGraphLaunch(c->gexec, s));
   return SDE_OK;

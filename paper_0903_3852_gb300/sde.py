@@ -74,6 +74,9 @@ class ObsRow(ctypes.Structure):
                 ("count", ctypes.c_double), ("t", ctypes.c_double)]
 
 
+_OBS_DTYPE = np.dtype([(name, "f8") for name, _ in ObsRow._fields_])
+
+
 class MlpConfig(ctypes.Structure):
     _fields_ = [("n_in", ctypes.c_int32), ("hidden", ctypes.c_int32), ("n_hidden", ctypes.c_int32),
                 ("n_members", ctypes.c_int32), ("max_batch", ctypes.c_int64), ("lr", ctypes.c_float),
@@ -195,6 +198,7 @@ class Ensemble:
         _check(lib().sde_create(ctypes.byref(cfg), ctypes.byref(h)))
         self._h = h
         self.cfg = cfg
+        self._rows = 0  # observable rows of the last run
 
     @classmethod
     def josephson(cls, points, paths, steps, seed, steps_per_period=200,
@@ -251,6 +255,7 @@ class Ensemble:
         r.x_out_dev, r.v_out_dev = _ptr(x_out), _ptr(v_out)
         r.w_out_dev, r.vsum_out_dev = _ptr(w_out), _ptr(vsum_out)
         _check(lib().sde_run_ensemble(self._h, ctypes.byref(r), _stream(stream)))
+        self._rows = self.cfg.n_points
 
     def run_kuramoto(self, n_begin, n_end, phi_in, phi_out, omega, r_out=None, stream=None):
         r = RunDesc()
@@ -258,6 +263,8 @@ class Ensemble:
         r.phi_in_dev, r.phi_out_dev, r.omega_dev = _ptr(phi_in), _ptr(phi_out), _ptr(omega)
         r.r_out_dev = _ptr(r_out)
         _check(lib().sde_run_ensemble(self._h, ctypes.byref(r), _stream(stream)))
+        M = self.sample_every
+        self._rows = -(-(n_end - n_begin) // M) + 1 if M > 0 else 0
 
     def position_histogram(self, w, w_lo, nbins, stream=None):
         """Per-point counts of the winding count w: (n_points, nbins + 2) int64
@@ -282,13 +289,10 @@ class Ensemble:
         """Synchronise and return the FP64 observables as a structured numpy array
         with fields mean, var, se, count, t."""
         n = ctypes.c_int64()
-        _check(lib().sde_observables(self._h, None, 0, ctypes.byref(n)))
-        cap = n.value if capacity is None else capacity
-        rows = (ObsRow * max(cap, 1))()
-        _check(lib().sde_observables(self._h, rows, cap, ctypes.byref(n)))
-        dt = np.dtype([("mean", "f8"), ("var", "f8"), ("se", "f8"), ("count", "f8"), ("t", "f8")])
-        out = np.frombuffer(bytearray(rows)[:ctypes.sizeof(ObsRow) * min(cap, n.value)], dtype=dt)
-        return out.copy()
+        cap = self._rows if capacity is None else capacity
+        rows = np.empty(cap, dtype=_OBS_DTYPE)
+        _check(lib().sde_observables(self._h, rows.ctypes.data_as(ctypes.POINTER(ObsRow)), cap, ctypes.byref(n)))
+        return rows[:min(cap, n.value)]
 
     def tuning(self):
         """(threads per block, paths or oscillators per thread, CTAs per replica)."""
