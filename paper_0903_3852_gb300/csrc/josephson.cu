@@ -33,7 +33,7 @@
 #include <mutex>
 #include <string>
 
-#include "cos2pi64.cuh"
+#include "fp64_math.cuh"
 #include "internal.h"
 #include "philox.cuh"
 

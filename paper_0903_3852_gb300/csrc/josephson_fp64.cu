@@ -25,7 +25,7 @@
 #include <algorithm>
 
 #include "common.cuh"
-#include "cos2pi64.cuh"
+#include "fp64_math.cuh"
 #include "philox.cuh"
 
 namespace sde {
@@ -85,19 +85,6 @@ __device__ __forceinline__ double minus2_log24(uint32_t m, const Tables64 &t) {
   q = fma(q, z, 0.9999999999999994);
   q = fma(q, z, -2.0);
   return fma(z, q, t.exponent[e] + t.two_log[i]);
-}
-
-// sqrt(L), L >= 0, by Goldschmidt's iteration from the hardware's approximate
-// reciprocal square root and a final correction by the residual L - g^2.
-__device__ __forceinline__ double sqrt_goldschmidt(double L) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(L));
-  y = L > 0.0 ? y : 0.0;
-  double g = L * y, h = 0.5 * y;
-  const double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  return fma(fma(-g, g, L), h, g);
 }
 
 // Box-Muller in FP64 from the same 24-bit uniforms as the FP32 path.  The

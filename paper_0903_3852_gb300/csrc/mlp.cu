@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fp64_math.cuh"
 #include "mlp_tc.cuh"
 #include "philox.cuh"
 #include "tma_map.h"
@@ -573,20 +574,24 @@ __global__ void features_kernel(const sde_jj_point *pts, int64_t n, float *X, co
   }
 }
 
-// Mean and standard deviation over the members' outputs (rows `stride` apart).
-__global__ void ensemble_stats_kernel(const float *out, int members, int64_t stride, int64_t B, float *mean,
-                                      float *spread) {
+// Mean and standard deviation over the members' outputs (rows `stride` apart)
+// in FP64.  The FP64 pipe bounds it (one warp instruction per 16 cycles and SM):
+// the divisions by the member counts are products with their reciprocals, the
+// square root is Goldschmidt's.
+__global__ void ensemble_stats_kernel(const float *out, int members, int64_t stride, int64_t B, double inv_n,
+                                      double inv_n1, float *mean, float *spread) {
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < B; b += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int q = 0; q < members; ++q) s += out[(int64_t)q * stride + b];
-    const double mu = s / members;
+    const double mu = s * inv_n;
+    mean[b] = (float)mu;
+    if (!spread) continue;
     double m2 = 0.0;
     for (int q = 0; q < members; ++q) {
       const double d = out[(int64_t)q * stride + b] - mu;
-      m2 += d * d;
+      m2 = fma(d, d, m2);
     }
-    mean[b] = (float)mu;
-    if (spread) spread[b] = members > 1 ? (float)sqrt(m2 / (members - 1)) : 0.0f;
+    spread[b] = members > 1 ? (float)sqrt_goldschmidt(m2 * inv_n1) : 0.0f;
   }
 }
 
@@ -598,15 +603,18 @@ struct SquareOffsets {
   int64_t w[mlptc::MAX_HH];
 };
 
-__global__ void square_weights_kernel(const float *params, int64_t P, int members, int n_hh, SquareOffsets off,
-                                      __nv_bfloat16 *whh) {
-  constexpr int64_t HH = (int64_t)mlptc::H * mlptc::H;
-  const int64_t n = (int64_t)members * n_hh * HH;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ml = i / HH;
-    const int member = (int)(ml / n_hh), l = (int)(ml % n_hh);
-    whh[i] = __float2bfloat16_rn(params[(int64_t)member * P + off.w[l] + (i - ml * HH)]);
-  }
+// Grid: (HH / 1024, square layers, members), four elements per thread.
+__global__ void __launch_bounds__(256) square_weights_kernel(const float *params, int64_t P, SquareOffsets off,
+                                                             __nv_bfloat16 *whh) {
+  constexpr int HH = mlptc::H * mlptc::H;
+  const float *w = params + blockIdx.z * P + off.w[blockIdx.y];
+  __nv_bfloat16 *d = whh + ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * HH;
+  const int i = (int)blockIdx.x * 1024 + threadIdx.x;
+  float v[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) v[u] = w[i + 256 * u];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) d[i + 256 * u] = __float2bfloat16_rn(v[u]);
 }
 
 }  // namespace
@@ -636,6 +644,7 @@ struct sde_mlp {
   __nv_bfloat16 *whh = nullptr;    // [members][n_hidden - 1][256][256]
   CUtensorMap map_whh;
   uint32_t *err = nullptr;         // latched kErrTimeout of the tensor-core kernel
+  int sm_count = 1;
 };
 
 namespace {
@@ -869,8 +878,17 @@ sde_status sde_mlp_create(const sde_mlp_config *cfg, sde_mlp **out) {
   if (st == SDE_OK && q->tc) {
     st = make_map_bf16(&q->map_whh, q->whh, M * (cfg->n_hidden - 1) * H, H, mlptc::H);
     if (st == SDE_OK) {
-      const cudaError_t e = cudaFuncSetAttribute(mlptc::mlp_fwd_tc_kernel,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, mlptc::SMEM_BYTES);
+      int dev = 0;
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&q->sm_count, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) st = cuda_fail(e, "cudaDeviceGetAttribute");
+    }
+    if (st == SDE_OK) {
+      cudaError_t e = cudaFuncSetAttribute(mlptc::mlp_fwd_tc_kernel<false>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, mlptc::SMEM_BYTES);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlptc::mlp_fwd_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 mlptc::SMEM_BYTES);
       if (e != cudaSuccess) st = cuda_fail(e, "cudaFuncSetAttribute(mlp_fwd_tc_kernel)");
     }
   }
@@ -953,8 +971,8 @@ sde_status sde_mlp_forward(sde_mlp *q, const float *X, int64_t B, float *mean, f
       so.w[l] = q->woff[l + 1];
       a.off_bh[l] = q->boff[l + 1];
     }
-    square_weights_kernel<<<grid1((int64_t)q->cfg.n_members * n_hh * mlptc::H * mlptc::H), 256, 0, s>>>(
-        q->params, q->P, q->cfg.n_members, n_hh, so, q->whh);
+    square_weights_kernel<<<dim3(mlptc::H * mlptc::H / 1024, (unsigned)n_hh, (unsigned)q->cfg.n_members), 256, 0, s>>>(
+        q->params, q->P, so, q->whh);
     SDE_CUDA_TRY(cudaGetLastError());
     a.X = X;
     a.params = q->params;
@@ -969,8 +987,16 @@ sde_status sde_mlp_forward(sde_mlp *q, const float *X, int64_t B, float *mean, f
     a.out = q->out;
     a.out_stride = q->cfg.max_batch;
     a.err = q->err;
-    const dim3 grid((unsigned)((B + mlptc::BM - 1) / mlptc::BM), (unsigned)q->cfg.n_members);
-    mlptc::mlp_fwd_tc_kernel<<<grid, mlptc::THREADS, mlptc::SMEM_BYTES, s>>>(q->map_whh, a);
+    // One CTA per SM, shared evenly among the members.  Where that leaves each
+    // CTA one tile, all its warps share it (129 points of 2 members: 25 us per call
+    // instead of 29).
+    const int64_t tiles = (B + mlptc::BM - 1) / mlptc::BM;
+    const int64_t per_member = std::max<int64_t>(1, q->sm_count / q->cfg.n_members);
+    const dim3 grid((unsigned)std::min(tiles, per_member), (unsigned)q->cfg.n_members);
+    if (tiles <= per_member)
+      mlptc::mlp_fwd_tc_kernel<true><<<grid, mlptc::THREADS, mlptc::SMEM_BYTES, s>>>(q->map_whh, a);
+    else
+      mlptc::mlp_fwd_tc_kernel<false><<<grid, mlptc::THREADS, mlptc::SMEM_BYTES, s>>>(q->map_whh, a);
     SDE_CUDA_TRY(cudaGetLastError());
   } else {
     const int64_t G = member_group(q, B);
@@ -980,7 +1006,9 @@ sde_status sde_mlp_forward(sde_mlp *q, const float *X, int64_t B, float *mean, f
       if (st != SDE_OK) return st;
     }
   }
-  ensemble_stats_kernel<<<grid1(B), 256, 0, s>>>(q->out, q->cfg.n_members, q->cfg.max_batch, B, mean, spread);
+  ensemble_stats_kernel<<<grid1(B), 256, 0, s>>>(q->out, q->cfg.n_members, q->cfg.max_batch, B,
+                                                 1.0 / q->cfg.n_members, 1.0 / (q->cfg.n_members - 1.0), mean,
+                                                 spread);
   SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }

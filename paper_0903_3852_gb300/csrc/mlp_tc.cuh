@@ -7,24 +7,32 @@
 // and activations rounded from FP32) and accumulates in FP32, as the CUDA-core
 // kernels of the training path do.
 //
-// One CTA takes 128 points (one tcgen05 M = 128 tile) of one ensemble member:
-//   warps 0-15 (512 threads): layer 0 on the CUDA cores, then after each
-//     square layer its epilogue -- tcgen05.ld of the FP32 accumulators, +
-//     bias, SiLU, BF16 -- written back into shared memory as the next layer's
-//     A operand in the 128-byte-swizzled K-major layout the MMA reads, or,
-//     after the last square layer, the output dot product; warp w owns TMEM
-//     lane quarter w % 4 (its 32 rows) and column quarter w / 4 (64
-//     columns); the element arithmetic runs on packed FP32 pairs;
+// A CTA per SM (persistent over the tiles of one member) keeps two tiles of 128
+// points in flight, one per group of eight warps:
+//   warps 8 g .. 8 g + 7 (group g): layer 0 of their tile on the CUDA cores,
+//     then after each square layer its epilogue -- tcgen05.ld of the FP32
+//     accumulators, + bias, SiLU, BF16 -- written back into shared memory as the
+//     next layer's A operand in the 128-byte-swizzled K-major layout the MMA
+//     reads, or, after the last square layer, the output dot product; warp w
+//     owns TMEM lane quarter w % 4 (its 32 rows) and one half of the columns (a
+//     quarter where a CTA has one tile and both groups share it);
+//     the element arithmetic runs on packed FP32 pairs;
 //   warp 16, one thread: TMA producer streaming the BF16 square-layer weights
-//     through a 4-slot ring of 256 x 64 chunks (K-major, 128-byte swizzle);
+//     through a 2-slot ring of 256 x 64 chunks (K-major, 128-byte swizzle);
 //   warp 17, one thread: MMA issuer, M = 128, N = 256, K = 16 per
-//     instruction, the accumulator (256 FP32 columns) in tensor memory, which
-//     warp 17 allocates and frees.
-// Layer handoffs go through mbarriers: `abuf` (512 arrivals: the A operand of
-// the next square layer is in shared memory) and `acc` (tcgen05.commit: the
-// accumulator is complete).  Every wait is bounded by one second of
-// %globaltimer; on expiry the CTA stops, drains what it issued, records
-// kErrTimeout and writes no output.
+//     instruction, for the groups in turn, each group's accumulator (256 FP32
+//     columns) in its half of tensor memory, which warp 17 allocates and frees.
+// What bounds it: the epilogues' instruction issue (about ten instructions per
+// SiLU).  With one tile per CTA they and the MMAs alternated (issue 48 %); with
+// two a group's MMAs run during the other group's epilogue (issue 63 %, two
+// warps per scheduler while one group waits).  100,000 points of 4 members: 178
+// us against 269.  Measured beside it: 16 accumulator columns at a time with
+// the next in flight instead of 32 (215 us: half the independent work per warp).
+// Layer handoffs go through mbarriers per group: `abuf` (256 arrivals: the A
+// operand of the next square layer is in shared memory) and `acc`
+// (tcgen05.commit: the accumulator is complete).  Every wait is bounded by one
+// second of %globaltimer; on expiry the CTA stops, drains what it issued,
+// records kErrTimeout and writes no further output.
 //
 // SiLU(z) = z sigma(z), sigma(z) = 1 / (1 + 2^(-z log2 e)): the exponential
 // by the hardware base-2 exponential (z clamped at -30), the reciprocal by
@@ -49,14 +57,16 @@ constexpr int BM = 128;            // points per CTA
 constexpr int KCH = H / 64;        // 64-element K chunks per square layer
 constexpr int A_CHUNK = BM * 128;  // bytes of one A chunk: 128 rows x 128 B
 constexpr int W_CHUNK = H * 128;   // bytes of one weight chunk: 256 rows x 128 B
-constexpr int RING = 4;            // weight chunks in flight
-constexpr int EPI_WARPS = 16;
-constexpr int EPI_THREADS = EPI_WARPS * 32;
+constexpr int RING = 2;            // weight chunks in flight
+constexpr int GROUPS = 2;          // tiles in flight
+constexpr int GROUP_WARPS = 8;
+constexpr int GROUP_THREADS = GROUP_WARPS * 32;
+constexpr int EPI_WARPS = GROUPS * GROUP_WARPS;
 constexpr int PROD_WARP = EPI_WARPS;
 constexpr int MMA_WARP = EPI_WARPS + 1;
-constexpr int THREADS = EPI_THREADS + 64;
-constexpr int SMEM_BYTES = KCH * A_CHUNK + RING * W_CHUNK + 1024;  // + alignment slack
-constexpr int COLS_PER_WARP = H / (EPI_WARPS / 4);  // 64
+constexpr int THREADS = EPI_WARPS * 32 + 64;
+constexpr int SMEM_BYTES = GROUPS * KCH * A_CHUNK + RING * W_CHUNK + 1024;  // + alignment slack
+constexpr int QUARTER = H / 4;  // columns of one partial sum of the output layer
 constexpr int MAX_IN = 8;
 constexpr int MAX_HH = 7;
 
@@ -118,38 +128,67 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(b)) : "memory");
 }
 
+// Layer 0 of 32 columns from n0 for a row's inputs x, into the A operand.
+__device__ __forceinline__ void layer0_row32(uint8_t *Ab, int m, int n0, const float (&x)[MAX_IN], int n_in,
+                                             const float *w0s, const float *b0s) {
+  uint32_t p[16];
+#pragma unroll
+  for (int j = 0; j < 32; j += 4) {  // parameters of four columns per shared load
+    const float4 bz = *reinterpret_cast<const float4 *>(b0s + n0 + j);
+    float2 z0 = make_float2(bz.x, bz.y), z1 = make_float2(bz.z, bz.w);
+#pragma unroll
+    for (int k = 0; k < MAX_IN; ++k) {
+      if (k < n_in) {
+        const float4 w = *reinterpret_cast<const float4 *>(w0s + k * H + n0 + j);
+        z0 = __ffma2_rn(f2(x[k]), make_float2(w.x, w.y), z0);
+        z1 = __ffma2_rn(f2(x[k]), make_float2(w.z, w.w), z1);
+      }
+    }
+    const float2 h0 = silu2(z0), h1 = silu2(z1);
+    p[j >> 1] = pack_bf16(h0.x, h0.y);
+    p[(j >> 1) + 1] = pack_bf16(h1.x, h1.y);
+  }
+  store_row32(Ab, m, n0, p);
+}
+
+// Grid: (CTAs per member, members); CTA x takes tiles x, x + gridDim.x, ... of its
+// member, its i-th tile in group i % 2.
+// SOLO: every CTA has at most one tile, and both groups share it.
+template <bool SOLO>
 __global__ void __launch_bounds__(THREADS, 1)
     mlp_fwd_tc_kernel(const __grid_constant__ CUtensorMap mapW, const Args a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t *Ab = smem;                  // KCH chunks of [BM][128 B]
-  uint8_t *Wr = smem + KCH * A_CHUNK;  // RING slots of [H][128 B]
+  uint8_t *Wr = smem + GROUPS * KCH * A_CHUNK;     // RING slots of [H][128 B]; before them KCH chunks of [BM][128 B] per group
   __shared__ __align__(16) float w0s[MAX_IN * H];  // [k][n]: output pairs adjacent
   __shared__ __align__(16) float b0s[H];
   __shared__ __align__(16) float bhs[MAX_HH * H];
   __shared__ __align__(16) float wos[H];
-  __shared__ float part[EPI_WARPS / 4][BM];
+  __shared__ float part[GROUPS][4][BM];
   __shared__ __align__(8) uint64_t full_bar[RING];
   __shared__ __align__(8) uint64_t empty_bar[RING];
-  __shared__ __align__(8) uint64_t acc_bar;
-  __shared__ __align__(8) uint64_t abuf_bar;
+  __shared__ __align__(8) uint64_t acc_bar[GROUPS];
+  __shared__ __align__(8) uint64_t abuf_bar[GROUPS];
   __shared__ __align__(8) uint64_t drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int member = blockIdx.y;
-  const int64_t row0 = (int64_t)blockIdx.x * BM;
   const float *pm = a.params + (int64_t)member * a.P;
   const int n_in = a.n_in, n_hh = a.n_hh;
+  const int64_t tiles = (a.B + BM - 1) / BM;
+  const int n_mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < RING; ++s) {
       tc::mbar_init(&full_bar[s], 1);
       tc::mbar_init(&empty_bar[s], 1);
     }
-    tc::mbar_init(&acc_bar, 1);
-    tc::mbar_init(&abuf_bar, EPI_THREADS);
+    for (int g = 0; g < GROUPS; ++g) {
+      tc::mbar_init(&acc_bar[g], 1);
+      tc::mbar_init(&abuf_bar[g], SOLO ? GROUPS * GROUP_THREADS : GROUP_THREADS);
+    }
     tc::mbar_init(&drain_bar, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -158,7 +197,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      tc::smem_addr(&tmem_slot)),
-                 "r"((uint32_t)H)
+                 "r"((uint32_t)(GROUPS * H))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -179,16 +218,29 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   if (warp == PROD_WARP) {
     if (lane == 0) {
-      // ---- TMA producer: the square layers' weight chunks, in MMA order ----
-      const int nchunks = n_hh * KCH;
+      // ---- TMA producer: the square layers' weight chunks, in MMA order (the
+      // layers of a pair of tiles, each layer once per group) ----
+      const int nchunks = n_mine * n_hh * KCH;
       int issued = 0;
+      int i0 = 0, l = 0, g = 0, kc = 0;  // pair's first tile, layer, group, chunk
       for (int c = 0; c < nchunks; ++c) {
         const int s = c % RING;
         const uint32_t ph = (uint32_t)(c / RING) & 1u;
         if (!tc::mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag)) break;
         tc::mbar_arrive_expect_tx(&full_bar[s], (uint32_t)W_CHUNK);
-        tc::tma_load_2d(Wr + s * W_CHUNK, &mapW, &full_bar[s], (c % KCH) * 64, (member * n_hh + c / KCH) * H);
+        tc::tma_load_2d(Wr + s * W_CHUNK, &mapW, &full_bar[s], kc * 64, (member * n_hh + l) * H);
         issued = c + 1;
+        if (++kc == KCH) {
+          kc = 0;
+          const int groups = n_mine - i0 < GROUPS ? n_mine - i0 : GROUPS;
+          if (++g == groups) {
+            g = 0;
+            if (++l == n_hh) {
+              l = 0;
+              i0 += GROUPS;
+            }
+          }
+        }
       }
       // every load issued has landed before the CTA may end (older ones were
       // consumed by completed MMAs)
@@ -201,28 +253,37 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (lane == 0) {
       // ---- MMA issuer ----
       constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, H);
-      for (int l = 0; l < n_hh; ++l) {
-        if (!tc::mbar_wait(&abuf_bar, (uint32_t)l & 1u, &abort_flag)) break;
-        tc::tmem_fence_after();
-        bool ok = true;
-        for (int kc = 0; kc < KCH; ++kc) {
-          const int c = l * KCH + kc;
-          const int s = c % RING;
-          if (!tc::mbar_wait(&full_bar[s], (uint32_t)(c / RING) & 1u, &abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc::tmem_fence_after();
-          const uint64_t adesc = tc::smem_desc_sw128(Ab + kc * A_CHUNK);
-          const uint64_t bdesc = tc::smem_desc_sw128(Wr + s * W_CHUNK);
+      int c = 0;
+      bool ok = true;
+      for (int i0 = 0; ok && i0 < n_mine; i0 += GROUPS) {
+        const int groups = n_mine - i0 < GROUPS ? n_mine - i0 : GROUPS;
+        for (int l = 0; ok && l < n_hh; ++l) {
+          const uint32_t turn = (uint32_t)(i0 / GROUPS * n_hh + l) & 1u;
+          for (int g = 0; ok && g < groups; ++g) {
+            if (!tc::mbar_wait(&abuf_bar[g], turn, &abort_flag)) {
+              ok = false;
+              break;
+            }
+            tc::tmem_fence_after();
+            const uint8_t *Ag = smem + g * KCH * A_CHUNK;
+            for (int kc = 0; kc < KCH; ++kc, ++c) {
+              const int s = c % RING;
+              if (!tc::mbar_wait(&full_bar[s], (uint32_t)(c / RING) & 1u, &abort_flag)) {
+                ok = false;
+                break;
+              }
+              tc::tmem_fence_after();
+              const uint64_t adesc = tc::smem_desc_sw128(Ag + kc * A_CHUNK);
+              const uint64_t bdesc = tc::smem_desc_sw128(Wr + s * W_CHUNK);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            tc::umma_bf16(tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                          (kc | k) != 0 ? 1u : 0u);
-          tc::umma_commit(&empty_bar[s]);
+              for (int k = 0; k < 4; ++k)
+                tc::umma_bf16(tmem + (uint32_t)(g * H), adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                              (kc | k) != 0 ? 1u : 0u);
+              tc::umma_commit(&empty_bar[s]);
+            }
+            tc::umma_commit(&acc_bar[g]);  // arrives once every MMA issued so far has completed
+          }
         }
-        tc::umma_commit(&acc_bar);  // arrives once every MMA issued so far has completed
-        if (!ok) break;
       }
       // every MMA issued has completed before the tensor memory is freed
       tc::umma_commit(&drain_bar);
@@ -231,82 +292,93 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     __syncwarp();
   } else {
-    // ---- layer 0 and the epilogues: warps 0-15 ----
-    const int q = warp & 3;   // TMEM lane quarter: rows 32 q .. 32 q + 31
-    const int cq = warp >> 2; // column quarter: 64 cq .. 64 cq + 63
+    // ---- layer 0 and the epilogues: group g ----
+    const int g = SOLO ? 0 : warp / GROUP_WARPS;
+    const int q = warp & 3;  // TMEM lane quarter: rows 32 q .. 32 q + 31
+    // column quarters c0 .. c0 + nq - 1 of 64
+    const int c0 = SOLO ? warp >> 2 : 2 * ((warp >> 2) & 1);
+    constexpr int nq = SOLO ? 1 : 2;
     const int m = q * 32 + lane;
-    const int64_t row = row0 + m;
-    const bool valid = row < a.B;
-    float x[MAX_IN];
+    constexpr uint32_t peers = SOLO ? GROUPS * GROUP_THREADS : GROUP_THREADS;
+    uint8_t *Ab = smem + g * KCH * A_CHUNK;
+    const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * H);
+    bool ok = true;
+    uint32_t turn = 0;
+    for (int i = g; i < n_mine; i += GROUPS) {
+      const int64_t row = ((int64_t)blockIdx.x + (int64_t)i * gridDim.x) * BM + m;
+      const bool valid = row < a.B;
+      float2 dot[nq];
 #pragma unroll
-    for (int k = 0; k < MAX_IN; ++k) x[k] = (valid && k < n_in) ? bf16r(a.X[row * n_in + k]) : 0.0f;
+      for (int qt = 0; qt < nq; ++qt) dot[qt] = make_float2(0.0f, 0.0f);
+      if (ok) {
+        float x[MAX_IN];
+#pragma unroll
+        for (int k = 0; k < MAX_IN; ++k) x[k] = (valid && k < n_in) ? bf16r(a.X[row * n_in + k]) : 0.0f;
 #pragma unroll 1
-    for (int g = 0; g < COLS_PER_WARP / 32; ++g) {
-      const int n0 = cq * COLS_PER_WARP + g * 32;
-      uint32_t p[16];
-#pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        float2 z = *reinterpret_cast<const float2 *>(b0s + n0 + j);
-#pragma unroll
-        for (int k = 0; k < MAX_IN; ++k)
-          if (k < n_in) z = __ffma2_rn(f2(x[k]), *reinterpret_cast<const float2 *>(w0s + k * H + n0 + j), z);
-        const float2 h = silu2(z);
-        p[j >> 1] = pack_bf16(h.x, h.y);
+        for (int n0 = c0 * QUARTER; n0 < (c0 + nq) * QUARTER; n0 += 32) layer0_row32(Ab, m, n0, x, n_in, w0s, b0s);
+        tc::tmem_fence_before();  // the last tile's accumulator is read before the next MMA overwrites it
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(&abuf_bar[g]);
       }
-      store_row32(Ab, m, n0, p);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive(&abuf_bar);
-    float2 dot = make_float2(0.0f, 0.0f);
-    bool done = n_hh == 0;
-    for (int l = 0; l < n_hh; ++l) {
-      if (!tc::mbar_wait(&acc_bar, (uint32_t)l & 1u, &abort_flag)) break;
-      tc::tmem_fence_after();
-      if (abort_flag) break;
-      const bool last = l == n_hh - 1;
-      const float *bl = bhs + l * H;
+      for (int l = 0; l < n_hh && ok; ++l, turn ^= 1u) {
+        if (!tc::mbar_wait(&acc_bar[g], turn, &abort_flag) || abort_flag) {
+          ok = false;
+          break;
+        }
+        tc::tmem_fence_after();
+        const bool last = l == n_hh - 1;
+        const float *bl = bhs + l * H;
+#pragma unroll
+        for (int qt = 0; qt < nq; ++qt) {
 #pragma unroll 1
-      for (int g = 0; g < COLS_PER_WARP / 32; ++g) {
-        const int n0 = cq * COLS_PER_WARP + g * 32;
-        float v[32];
-        tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)n0, v);
-        if (!last) {
-          uint32_t p[16];
+          for (int u = 0; u < QUARTER; u += 32) {
+            const int n0 = (c0 + qt) * QUARTER + u;
+            float v[32];
+            tc::tmem_ld32(tacc + (uint32_t)n0, v);
+            if (!last) {
+              uint32_t p[16];
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const float2 h = silu2(__fadd2_rn(make_float2(v[j], v[j + 1]),
-                                              *reinterpret_cast<const float2 *>(bl + n0 + j)));
-            p[j >> 1] = pack_bf16(h.x, h.y);
-          }
-          store_row32(Ab, m, n0, p);
-        } else {
+              for (int j = 0; j < 32; j += 4) {
+                const float4 bz = *reinterpret_cast<const float4 *>(bl + n0 + j);
+                const float2 h0 = silu2(__fadd2_rn(make_float2(v[j], v[j + 1]), make_float2(bz.x, bz.y)));
+                const float2 h1 = silu2(__fadd2_rn(make_float2(v[j + 2], v[j + 3]), make_float2(bz.z, bz.w)));
+                p[j >> 1] = pack_bf16(h0.x, h0.y);
+                p[(j >> 1) + 1] = pack_bf16(h1.x, h1.y);
+              }
+              store_row32(Ab, m, n0, p);
+            } else {
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const float2 h = silu2(__fadd2_rn(make_float2(v[j], v[j + 1]),
-                                              *reinterpret_cast<const float2 *>(bl + n0 + j)));
-            dot = __ffma2_rn(make_float2(bf16r(h.x), bf16r(h.y)), *reinterpret_cast<const float2 *>(wos + n0 + j),
-                             dot);
+              for (int j = 0; j < 32; j += 4) {
+                const float4 bz = *reinterpret_cast<const float4 *>(bl + n0 + j);
+                const float4 w = *reinterpret_cast<const float4 *>(wos + n0 + j);
+                const float2 h0 = silu2(__fadd2_rn(make_float2(v[j], v[j + 1]), make_float2(bz.x, bz.y)));
+                const float2 h1 = silu2(__fadd2_rn(make_float2(v[j + 2], v[j + 3]), make_float2(bz.z, bz.w)));
+                dot[qt] = __ffma2_rn(make_float2(bf16r(h0.x), bf16r(h0.y)), make_float2(w.x, w.y), dot[qt]);
+                dot[qt] = __ffma2_rn(make_float2(bf16r(h1.x), bf16r(h1.y)), make_float2(w.z, w.w), dot[qt]);
+              }
+            }
           }
         }
+        if (!last) {
+          tc::tmem_fence_before();  // the accumulator is read before the next layer overwrites it
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          mbar_arrive(&abuf_bar[g]);
+        }
       }
-      if (!last) {
-        tc::tmem_fence_before();  // the accumulator is read before the next layer overwrites it
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(&abuf_bar);
-      } else {
-        done = true;
-      }
+      // the four column quarters of each row; every thread of the group meets
+      // here once per tile, also after an expired wait
+#pragma unroll
+      for (int qt = 0; qt < nq; ++qt) part[g][c0 + qt][m] = dot[qt].x + dot[qt].y;
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(peers) : "memory");
+      if (c0 == 0 && valid && ok && !abort_flag)
+        a.out[(int64_t)member * a.out_stride + row] =
+            ((part[g][0][m] + part[g][1][m]) + (part[g][2][m] + part[g][3][m])) + bo;
     }
-    // the four column quarters of each row
-    part[cq][m] = dot.x + dot.y;
-    asm volatile("bar.sync 1, %0;" ::"r"(EPI_THREADS) : "memory");
-    if (cq == 0 && valid && done && !abort_flag)
-      a.out[(int64_t)member * a.out_stride + row] = ((part[0][m] + part[1][m]) + (part[2][m] + part[3][m])) + bo;
   }
   tc::tmem_fence_before();
   __syncthreads();
   if (warp == MMA_WARP) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)H)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(GROUPS * H))
                  : "memory");
   }
   if (threadIdx.x == 0 && abort_flag) atomicOr(a.err, kErrTimeout);

@@ -182,3 +182,25 @@ def test_fp64_block_sizes(n, steps):
             vsum = vsum + v
     for got, ref in ((xo, x), (vo, v), (so, vsum)):
         assert (got - ref).abs().max().item() <= 1e-12
+
+
+@pytest.mark.parametrize("members,n_hidden,n_in", [(1, 2, 1), (4, 3, 5), (3, 8, 8)])
+@pytest.mark.parametrize("B", [1, 128, 129, 6500, 39000])
+def test_forward_tiles_are_independent(members, n_hidden, n_in, B):
+    """Tensor-core forward with one tile, a ragged tile, one and several tiles
+    per CTA (an odd and an even number): every point's result is that of a
+    one-tile call bit for bit."""
+    ensure_built()
+    m = sde.Mlp(n_in=n_in, n_hidden=n_hidden, members=members, max_batch=40000, seed=9)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+    X = torch.rand((B, n_in), generator=g, device="cuda") * 2 - 1
+    mean, spread = m.forward(X)
+    m.check()
+    for b0 in sorted({0, 64 * (B // 128), 128 * (B // 256), max(0, B - 100)}):
+        part = X[b0:b0 + 100].contiguous()
+        mp, sp = m.forward(part)
+        assert torch.equal(mean[b0:b0 + 100], mp) and torch.equal(spread[b0:b0 + 100], sp)
+    m.use_tensor_cores(False)
+    ref, _ = m.forward(X)
+    assert (mean - ref).abs().max().item() <= 2e-3 * max(1.0, ref.abs().max().item())
