@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "philox.cuh"
 
 namespace sde {
 
@@ -72,7 +73,7 @@ struct KurArgs {
   float kc;      // (K / N) dt / (2 pi)
   float kh;      // kc / 2
   float sc;      // sqrt(2 D dt) / (2 pi)
-  uint64_t seed;
+  PhiloxKeys keys;
   uint32_t *err;
   uint64_t wait_ns;  // limit of each bounded mbarrier wait (asynchronous exchange)
 };

@@ -108,6 +108,41 @@ __device__ __forceinline__ void gauss4(uint32_t g, uint32_t c1, uint32_t c2, uin
   box_muller(r.z, r.w, z[2], z[3]);
 }
 
+// box_muller of two word pairs (of two streams) at once: the angles'
+// polynomials and the products on packed FP32 pairs, the same roundings
+// element by element.
+__device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1, float2 &z0,
+                                            float2 &z1) {
+  const float2 rho = make_float2(radius(-2.0f * logf(uniform24(a0))), radius(-2.0f * logf(uniform24(b0))));
+  float2 s, c;
+  sincos_turns2(((a1 >> 8) + 1u) << 8, ((b1 >> 8) + 1u) << 8, s, c);
+  z0 = __fmul2_rn(rho, c);
+  z1 = __fmul2_rn(rho, s);
+}
+
+// gauss4 of N streams (counter words c1[k]), two at a time.
+template <int N>
+__device__ __forceinline__ void gauss4_n(uint32_t g, const uint32_t (&c1)[N], uint32_t c2, uint32_t tag,
+                                         const PhiloxKeys &K, float (&z)[N][4]) {
+#pragma unroll
+  for (int k = 0; k + 1 < N; k += 2) {
+    const uint4 a = philox4x32_10(make_uint4(g, c1[k], c2, tag), K);
+    const uint4 b = philox4x32_10(make_uint4(g, c1[k + 1], c2, tag), K);
+    float2 z0, z1, z2, z3;
+    box_muller2(a.x, a.y, b.x, b.y, z0, z1);
+    box_muller2(a.z, a.w, b.z, b.w, z2, z3);
+    z[k][0] = z0.x;
+    z[k][1] = z1.x;
+    z[k][2] = z2.x;
+    z[k][3] = z3.x;
+    z[k + 1][0] = z0.y;
+    z[k + 1][1] = z1.y;
+    z[k + 1][2] = z2.y;
+    z[k + 1][3] = z3.y;
+  }
+  if (N & 1) gauss4(g, c1[N - 1], c2, tag, K, z[N - 1]);
+}
+
 // Box-Muller of the Josephson kernels, two shortcuts against box_muller:
 //  * the angle's sine and cosine from a table: the angle 2 pi u1,
 //    u1 = (j + 1) 2^-24 with j = w1 >> 8, is split into the table angle

@@ -16,26 +16,31 @@
 
 namespace sde {
 
+// v with the sign flipped where bit 31 of m is set.
+__device__ __forceinline__ float flip_sign(float v, uint32_t m) {
+  return __uint_as_float(__float_as_uint(v) ^ (m & 0x80000000u));
+}
+
 __device__ __forceinline__ void sincos_turns(uint32_t th, float &sn, float &cs) {
-  const uint32_t q = (th + 0x20000000u) >> 30;
-  const float x = (float)(int32_t)(th - (q << 30)) * 1.46291807926715968e-9f;  // 2 pi / 2^32
+  const uint32_t t = th + 0x20000000u;
+  const float x = (float)(int32_t)(th - (t & 0xC0000000u)) * 1.46291807926715968e-9f;  // 2 pi / 2^32
   const float x2 = x * x;
   const float s = fmaf(x * x2, fmaf(x2, fmaf(x2, -1.956071210e-4f, 8.332642727e-3f), -1.666666716e-1f), x);
   const float c = fmaf(x2, fmaf(x2, fmaf(x2, fmaf(x2, 2.456674520e-5f, -1.388842822e-3f), 4.166666791e-2f),
                                 -0.5f),
                        1.0f);
-  const float ss = (q & 1u) ? c : s;
-  const float cc = (q & 1u) ? s : c;
-  sn = (q & 2u) ? -ss : ss;
-  cs = ((q + 1u) & 2u) ? -cc : cc;
+  const bool swap = (t & 0x40000000u) != 0u;
+  sn = flip_sign(swap ? c : s, t);
+  cs = flip_sign(swap ? s : c, t + 0x40000000u);
 }
 
 // sincos_turns of two phases at once, the polynomials on packed FP32 pairs
 // (the same roundings as sincos_turns element by element).
 __device__ __forceinline__ void sincos_turns2(uint32_t ta, uint32_t tb, float2 &sn, float2 &cs) {
-  const uint32_t qa = (ta + 0x20000000u) >> 30, qb = (tb + 0x20000000u) >> 30;
-  const float2 x = __fmul2_rn(make_float2((float)(int32_t)(ta - (qa << 30)), (float)(int32_t)(tb - (qb << 30))),
-                              make_float2(1.46291807926715968e-9f, 1.46291807926715968e-9f));
+  const uint32_t qa = ta + 0x20000000u, qb = tb + 0x20000000u;
+  const float2 x = __fmul2_rn(
+      make_float2((float)(int32_t)(ta - (qa & 0xC0000000u)), (float)(int32_t)(tb - (qb & 0xC0000000u))),
+      make_float2(1.46291807926715968e-9f, 1.46291807926715968e-9f));
   const float2 x2 = __fmul2_rn(x, x);
   const float2 ps = __ffma2_rn(__ffma2_rn(x2, make_float2(-1.956071210e-4f, -1.956071210e-4f),
                                           make_float2(8.332642727e-3f, 8.332642727e-3f)),
@@ -46,10 +51,9 @@ __device__ __forceinline__ void sincos_turns2(uint32_t ta, uint32_t tb, float2 &
   pc = __ffma2_rn(x2, pc, make_float2(4.166666791e-2f, 4.166666791e-2f));
   pc = __ffma2_rn(x2, pc, make_float2(-0.5f, -0.5f));
   const float2 c = __ffma2_rn(x2, pc, make_float2(1.0f, 1.0f));
-  const float ssa = (qa & 1u) ? c.x : s.x, cca = (qa & 1u) ? s.x : c.x;
-  const float ssb = (qb & 1u) ? c.y : s.y, ccb = (qb & 1u) ? s.y : c.y;
-  sn = make_float2((qa & 2u) ? -ssa : ssa, (qb & 2u) ? -ssb : ssb);
-  cs = make_float2(((qa + 1u) & 2u) ? -cca : cca, ((qb + 1u) & 2u) ? -ccb : ccb);
+  const bool wa = (qa & 0x40000000u) != 0u, wb = (qb & 0x40000000u) != 0u;
+  sn = make_float2(flip_sign(wa ? c.x : s.x, qa), flip_sign(wb ? c.y : s.y, qb));
+  cs = make_float2(flip_sign(wa ? s.x : c.x, qa + 0x40000000u), flip_sign(wb ? s.y : c.y, qb + 0x40000000u));
 }
 
 // sincos_turns of n phases, two at a time on packed pairs (one alone if n is
