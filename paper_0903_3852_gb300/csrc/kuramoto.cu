@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_cluster_kernel(const Kur
     th[k] = valid[k] ? A.theta_in[base + i] : 0u;
     wdt[k] = valid[k] ? A.omega[base + i] * A.wscale : 0.0f;
   }
+  cluster.sync();  // every CTA of the cluster runs before the first remote store into it
   int buf = 0;
   int64_t sample_ctr = 0, sample_idx = 0;
   // cluster-wide (S, C)
