@@ -554,13 +554,51 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
 // ---- mean field over the whole grid ------------------------------------
 
 constexpr int kMfgThreads = 256;
-constexpr int kMfgIlp = 4;  // oscillators per thread per iteration (loads issued together)
+constexpr int kMfgIlp = 4;  // oscillators per thread per iteration: one 16-byte access per array
+
+// Four consecutive elements from index i0 of a replica's array in one access;
+// those outside [0, n) are not touched (zero) where the chunk is not whole.
+// STREAM marks what the next launch does not find in L2 anyway as first to be
+// evicted.
+template <bool STREAM, typename T>
+__device__ __forceinline__ void mfg_load4(const T *p, uint32_t i0, uint32_t n, bool vec, T (&v)[4]) {
+  if (vec) {
+    const uint4 *q = reinterpret_cast<const uint4 *>(p + i0);
+    const uint4 u = STREAM ? __ldcs(q) : *q;
+    memcpy(v, &u, 16);
+  } else {
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e) v[e] = i0 + e < n ? p[i0 + e] : T(0);
+  }
+}
+
+template <bool STREAM, typename T>
+__device__ __forceinline__ void mfg_store4(T *p, uint32_t i0, uint32_t n, bool vec, const T (&v)[4]) {
+  if (vec) {
+    uint4 u;
+    memcpy(&u, v, 16);
+    uint4 *q = reinterpret_cast<uint4 *>(p + i0);
+    if (STREAM)
+      __stcs(q, u);
+    else
+      *q = u;
+  } else {
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e)
+      if (i0 + e < n) p[i0 + e] = v[e];
+  }
+}
+
+int64_t mfg_plane(int64_t NR) { return (NR + 3) & ~3ll; }
 
 struct MfgArgs {
   uint32_t *theta;    // [R][N] theta_n; the corrector overwrites it with theta_{n+1}
   uint32_t *theta_t;  // [R][N] predictor phases theta~_n
   float *y;           // [R][N] first-stage part of the step: wdt + kh g1 + sc psi
-  float *psi;         // [3][R][N] Gaussians of steps 4g+1..4g+3 of the current Philox block
+  float *psi;         // [3][plane] Gaussians of steps 4g+1..4g+3 of the current Philox block
+  int64_t plane;      // R N rounded up to a multiple of 4
+  bool omega_vec;     // omega starts on a 16-byte boundary, as the library's arrays do
+  bool reverse;       // from the last oscillator to the first
   const float *omega;
   float2 *partials;   // [R][gridDim.x] per-block sums
   double *tot;        // [R][4]: (S, C) of theta_n, then (S, C) of theta~_n
@@ -584,6 +622,16 @@ struct MfgArgs {
 // strides over the replica; the block's FP32 sums go to `partials`, and the
 // block that finishes last adds all partials of the replica in block order
 // in FP64, so the totals do not depend on which block that is.
+//
+// What bounds it: HBM (16 B per oscillator for the corrector, 20 for the
+// predictor, 28 where it draws), then the noise of the drawing launch.  A thread
+// takes four consecutive oscillators in one 16-byte access per array: with four
+// 4-byte accesses the launches were bound by issue (153.7 us per step of 2^24
+// oscillators, 127.9 with 16-byte ones).  theta is the one array both launches
+// of a step use; the others are marked as first to leave L2 (120.2 us), and the
+// corrector runs from the last oscillator to the first, so that it starts with
+// what the predictor left there (2 us of it).  1,000,003 x 7, no row of which
+// but the first starts on a 16-byte boundary: 80.4 -> 66.5 us.
 template <int MODE>
 __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 5)) kur_mfg_kernel(const MfgArgs A) {
   constexpr bool kPred = MODE == 0 || MODE == 3;
@@ -591,9 +639,8 @@ __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 
   __shared__ float2 red[32];
   __shared__ double2 red64[32];
   __shared__ bool is_last;
-  const int rep = blockIdx.y;
+  const int rep = A.reverse ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   const int64_t N = A.N;
-  const int64_t NR = N * A.R;
   const int64_t base = (int64_t)rep * N;
   double *tot = A.tot + 4 * rep;
   float S = 0.0f, C = 0.0f;
@@ -606,97 +653,83 @@ __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 
   }
   const int j = (int)(A.n & 3);
   float ps = 0.0f, pc = 0.0f;
-  // per-replica base pointers, 32-bit oscillator indices (N < 2^31, so
-  // i0 + stride < 2^32 never wraps)
+  // per-replica base pointers, 32-bit oscillator indices: a chunk is four
+  // oscillators on a 16-byte boundary of the [R][N] arrays, so its first index
+  // is -lead (as an unsigned number) in a replica's first chunk.  N < 2^31: no
+  // sum below wraps onto a valid index.
   const uint32_t Nu = (uint32_t)N;
+  const uint32_t lead = (uint32_t)(base & 3);
   uint32_t *th_r = A.theta + base;
   uint32_t *tt_r = A.theta_t + base;
   float *y_r = A.y + base;
   const float *om_r = A.omega + base;
-  const float *psi_in = (kPred && !kGen && j > 0) ? A.psi + (int64_t)(j - 1) * NR + base : nullptr;
-  float *psi_out = A.psi + base;  // plane k - 1 at + (k - 1) NR
-  const uint32_t stride = gridDim.x * (uint32_t)(kMfgThreads * kMfgIlp);
-  for (uint32_t i0 = blockIdx.x * (uint32_t)(kMfgThreads * kMfgIlp) + threadIdx.x; i0 < Nu; i0 += stride) {
-    uint32_t t0[kMfgIlp], tt[kMfgIlp];
-    float a1[kMfgIlp], a2[kMfgIlp];
-    bool ok[kMfgIlp];
-#pragma unroll
-    for (int u = 0; u < kMfgIlp; ++u) {
-      const uint32_t i = i0 + u * kMfgThreads;
-      ok[u] = i < Nu;
-      const uint32_t ii = ok[u] ? i : 0u;
-      t0[u] = th_r[ii];
-      if (kPred) {
-        a1[u] = om_r[ii];
-        a2[u] = kGen ? 0.0f : psi_in[ii];
-      } else if (MODE == 1) {
-        tt[u] = tt_r[ii];
-        a1[u] = y_r[ii];
-      }
+  const float *psi_in = (kPred && !kGen && j > 0) ? A.psi + (int64_t)(j - 1) * A.plane + base : nullptr;
+  float *psi_out = A.psi + base;  // plane k - 1 at + (k - 1) A.plane
+  const uint32_t chunks = (lead + Nu + 3u) >> 2, stride = gridDim.x * (uint32_t)kMfgThreads;
+  for (uint32_t q = blockIdx.x * (uint32_t)kMfgThreads + threadIdx.x; q < chunks; q += stride) {
+    const uint32_t i0 = 4u * (A.reverse ? chunks - 1u - q : q) - lead;
+    const bool full = i0 < Nu && Nu - i0 >= 4u;
+    uint32_t t0[4], tt[4];
+    float a1[4], a2[4];
+    mfg_load4<false>(th_r, i0, Nu, full, t0);
+    if (kPred) {
+      mfg_load4<true>(om_r, i0, Nu, full && A.omega_vec, a1);
+      if (!kGen) mfg_load4<true>(psi_in, i0, Nu, full, a2);
+    } else if (MODE == 1) {
+      mfg_load4<true>(tt_r, i0, Nu, full, tt);
+      mfg_load4<true>(y_r, i0, Nu, full, a1);
     }
-    // oscillators u and u + 1 together: their sin/cos polynomials on packed
-    // FP32 pairs (sincos_turns2), the rest per oscillator
-    static_assert(kMfgIlp % 2 == 0, "oscillators are taken in pairs");
+    float z[4][4];
+    if (kGen) {
+      const uint32_t ids[4] = {i0, i0 + 1, i0 + 2, i0 + 3};
+      gauss4_n<4>((uint32_t)(A.n >> 2), ids, (uint32_t)rep, kTagKuramoto, A.keys, z);
 #pragma unroll
-    for (int u = 0; u < kMfgIlp; u += 2) {
-      float2 sn, cs;
-      if (MODE == 2) {
-        sincos_turns2(t0[u], t0[u + 1], sn, cs);
-      } else if (kPred) {
-        float2 s0, c0;
-        sincos_turns2(t0[u], t0[u + 1], s0, c0);
-        float z[2][4];
-        if (kGen) {
-          const uint32_t ids[2] = {i0 + u * kMfgThreads, i0 + (u + 1) * kMfgThreads};
-          gauss4_n<2>((uint32_t)(A.n >> 2), ids, (uint32_t)rep, kTagKuramoto, A.keys, z);
+      for (int e = 0; e < 4; ++e) a2[e] = pick4(z[e], j);
+#pragma unroll
+      for (int k = 1; k < 4; ++k)
+        if (k > j) {
+          const float zk[4] = {z[0][k], z[1][k], z[2][k], z[3][k]};
+          mfg_store4<true>(psi_out + (int64_t)(k - 1) * A.plane, i0, Nu, full, zk);
         }
-        uint32_t tp[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int v = u + e;
-          const uint32_t i = i0 + v * kMfgThreads;
-          const float g1 = (e ? c0.y : c0.x) * S - (e ? s0.y : s0.x) * C;
-          float psi = a2[v];
-          if (kGen) {
-            psi = pick4(z[e], j);
-            if (ok[v]) {
-#pragma unroll
-              for (int k = 1; k < 4; ++k)
-                if (k > j) psi_out[(int64_t)(k - 1) * NR + i] = z[e][k];
-            }
-          }
-          const float wdt = a1[v] * A.wscale;
-          const float d1 = fmaf(A.sc, psi, fmaf(A.kc, g1, wdt));
-          tp[e] = t0[v] + (uint32_t)__float2int_rn(d1 * 4294967296.0f);
-          if (ok[v]) {
-            tt_r[i] = tp[e];
-            y_r[i] = fmaf(A.sc, psi, fmaf(A.kh, g1, wdt));
-          }
-        }
-        sincos_turns2(tp[0], tp[1], sn, cs);
-      } else {
-        float2 s2, c2;
-        sincos_turns2(tt[u], tt[u + 1], s2, c2);
-        uint32_t t1[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int v = u + e;
-          const uint32_t i = i0 + v * kMfgThreads;
-          const float g2 = (e ? c2.y : c2.x) * S - (e ? s2.y : s2.x) * C;
-          t1[e] = t0[v] + (uint32_t)__float2int_rn(fmaf(A.kh, g2, a1[v]) * 4294967296.0f);
-          if (ok[v]) th_r[i] = t1[e];
-        }
-        sincos_turns2(t1[0], t1[1], sn, cs);
-      }
-      if (ok[u]) {
-        ps += sn.x;
-        pc += cs.x;
-      }
-      if (ok[u + 1]) {
-        ps += sn.y;
-        pc += cs.y;
-      }
     }
+    // the sin/cos polynomials of two oscillators at a time on packed FP32 pairs
+    float sn[4], cs[4];
+    if (MODE == 2) {
+      sincos_turns_n<4>(t0, sn, cs);
+    } else if (kPred) {
+      float s0[4], c0[4], y[4];
+      uint32_t tp[4];
+      sincos_turns_n<4>(t0, s0, c0);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float g1 = c0[e] * S - s0[e] * C;
+        const float wdt = a1[e] * A.wscale;
+        const float d1 = fmaf(A.sc, a2[e], fmaf(A.kc, g1, wdt));
+        tp[e] = t0[e] + (uint32_t)__float2int_rn(d1 * 4294967296.0f);
+        y[e] = fmaf(A.sc, a2[e], fmaf(A.kh, g1, wdt));
+      }
+      mfg_store4<true>(tt_r, i0, Nu, full, tp);
+      mfg_store4<true>(y_r, i0, Nu, full, y);
+      sincos_turns_n<4>(tp, sn, cs);
+    } else {
+      float s2[4], c2[4];
+      uint32_t t1[4];
+      sincos_turns_n<4>(tt, s2, c2);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float g2 = c2[e] * S - s2[e] * C;
+        t1[e] = t0[e] + (uint32_t)__float2int_rn(fmaf(A.kh, g2, a1[e]) * 4294967296.0f);
+      }
+      mfg_store4<false>(th_r, i0, Nu, full, t1);
+      sincos_turns_n<4>(t1, sn, cs);
+    }
+    if (!full) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (i0 + e >= Nu) sn[e] = cs[e] = 0.0f;
+    }
+    ps += (sn[0] + sn[1]) + (sn[2] + sn[3]);
+    pc += (cs[0] + cs[1]) + (cs[2] + cs[3]);
   }
   const float2 b = block_sum2(ps, pc, red);
   if (threadIdx.x == 0) {
@@ -947,7 +980,7 @@ __global__ void kur_order_kernel(const uint32_t *theta, int64_t N, int64_t R, do
 // times 2^66 / (2 pi) has turns 2^63 in its high word, within 2^-60 of the exact
 // product, closer than FP64's 53 bits; other values take the FP64 path.  FP64
 // multiplies on this GPU made the two kernels 189 and 125 us for 2^24 phases;
-// CVT_US.
+// with integers both take 50 us together.
 __device__ __forceinline__ uint32_t phase_to_turns(float phi) {
   const uint32_t bits = __float_as_uint(phi);
   if (bits >= 0x41000000u) {  // negative, >= 8, or not finite
@@ -1184,7 +1217,9 @@ MfgArgs mfg_args(KuramotoCtx *k, const float *omega, double *rbuf) {
   a.theta_t = k->theta_t;
   a.y = k->g1;
   a.psi = k->psi4;
+  a.plane = mfg_plane(k->N * k->R);
   a.omega = omega;
+  a.omega_vec = ((uintptr_t)omega & 15u) == 0u;
   a.partials = k->mfg_partials;
   a.tot = k->mfg_tot;
   a.count = k->mfg_count;
@@ -1208,11 +1243,13 @@ sde_status run_meanfield_grid(KuramotoCtx *k, int64_t n_begin, int64_t n_end, co
   const int *grid = k->mfg_grid;
   a.n = n_begin;
   a.sample_row = n_rows > 0 ? 0 : -1;
+  a.reverse = true;
   SDE_CUDA_TRY(launch_mfg(a, 2, grid[2], s));
   for (int64_t n = n_begin; n < n_end; ++n) {
     a.n = n;
     const int pred = (n == n_begin || (n & 3) == 0) ? 3 : 0;
     a.sample_row = -1;
+    a.reverse = false;
     SDE_CUDA_TRY(ktime_begin(k, s));
     SDE_CUDA_TRY(launch_mfg(a, pred, grid[pred], s));
     SDE_CUDA_TRY(ktime_end(k, s));
@@ -1223,6 +1260,7 @@ sde_status run_meanfield_grid(KuramotoCtx *k, int64_t n_begin, int64_t n_end, co
       else if ((m - n_begin) % k->M == 0)
         a.sample_row = (m - n_begin) / k->M;
     }
+    a.reverse = true;
     SDE_CUDA_TRY(ktime_begin(k, s));
     SDE_CUDA_TRY(launch_mfg(a, 1, grid[1], s));
     SDE_CUDA_TRY(ktime_end(k, s));
@@ -1398,7 +1436,7 @@ sde_status kuramoto_create(const sde_config *cfg, int sm_count, uint32_t *err, K
     alloc((void **)&k->mfg_partials, sizeof(float2) * (size_t)k->mfg_blocks * (size_t)k->R);
     alloc((void **)&k->mfg_tot, sizeof(double) * 4 * (size_t)k->R);
     alloc((void **)&k->mfg_count, sizeof(uint32_t) * (size_t)k->R);
-    alloc((void **)&k->psi4, sizeof(float) * 3 * NR);
+    alloc((void **)&k->psi4, sizeof(float) * 3 * (size_t)mfg_plane((int64_t)NR));
     if (st == SDE_OK && (e = cudaMemset(k->mfg_count, 0, sizeof(uint32_t) * (size_t)k->R)) != cudaSuccess)
       st = cuda_fail(e, "cudaMemset");
   }

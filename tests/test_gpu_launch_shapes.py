@@ -38,6 +38,29 @@ def test_pairwise_shapes_match_mean_field(N, R, euler):
     assert np.abs(r - r_mf).max() <= 2e-5
 
 
+@pytest.mark.parametrize("N,R", [(1, 3), (3, 5), (5, 2), (1023, 3), (4098, 2)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_grid_wide_chunks_match_replica_form(N, R, shift):
+    """The grid-wide mean field's 16-byte chunks where replicas start inside one,
+    and frequencies that start off a 16-byte boundary, against one CTA per
+    replica over steps 3 .. 9.  The replica form's sums are within N 2^-18, K dt / N
+    times that is 8e-8 per step, and phases come back in FP32 (2.4e-7): 1e-6."""
+    ensure_built()
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=R, seed=N)
+    phi0 = torch.from_numpy(w["phi0"]).cuda()
+    store = torch.zeros(N * R + shift, device="cuda")
+    omega = store[shift:].view(R, N)
+    omega.copy_(torch.from_numpy(w["omega"]))
+    got = []
+    for kw in (dict(schedule=sde.SDE_SCHED_GRID), dict(cluster_ctas=1)):
+        ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_MEANFIELD, N, R, 2.0, 0.05, 0.01, 3, sample_every=2, **kw)
+        phi, r = torch.empty_like(phi0), torch.empty((4, R), dtype=torch.float64, device="cuda")
+        ens.run_kuramoto(3, 9, phi0, phi, omega, r)
+        got.append((phi.cpu().numpy().astype(np.float64), r.cpu().numpy()))
+    assert np.abs(angle_diff(got[0][0], got[1][0])).max() <= 1e-6
+    assert np.abs(got[0][1] - got[1][1]).max() <= 2e-5
+
+
 @pytest.mark.parametrize("N,R", [(8, 1), (16, 3), (136, 13), (264, 25), (512, 100), (1000, 7), (3000, 28)])
 def test_fp32_gemm_shapes(N, R):
     """Coupling sums of the FP32 form against FP64: every chain of N FMAs errs by
