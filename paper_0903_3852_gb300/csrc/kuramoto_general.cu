@@ -130,19 +130,23 @@ __global__ void kg_to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t 
 // ---- FP32 CUDA-core GEMM (baseline): Dt[c][i] = sum_j K[i][j] B[c][j] ----
 //
 // One CTA of 128 threads: 256 rows x 8 TN columns of D over a share of K, 16 x
-// TN outputs per thread as packed FP32 pairs along the rows.  K slices of 8
-// are staged transposed in shared memory, double buffered, the next slice's
-// global loads in flight during the current slice's FMAs and each k's
-// fragments read while the previous k is multiplied.  Partial sums of a K
-// split go to planes of Dt and are added by the kernel that reads them.
+// TN outputs per thread as packed FP32 pairs along the rows.  K slices of 16
+// come into shared memory transposed, by 4-byte asynchronous copies three slices
+// deep: no registers hold them on the way, and each copy instruction of a warp
+// reads four whole 32-byte sectors.  Each k's fragments are read while the
+// previous k is multiplied.  Partial sums of a K split go to planes of Dt and are
+// added by the kernel that reads them.
 // What bounds it: shared memory returns 128 bytes per cycle to the SM's four
 // schedulers, 4 (16 + TN) cycles per k against 16 TN cycles of packed FMAs, so
 // the FMA pipe is the limit from TN = 6 up; and how evenly the tiles fill the
-// GPU (sgemm_shape).  3000 x 200 x 3000: 109 us (33 TFLOP/s; 42 % of the FMA
-// pipe, waiting for the global loads of a slice) against 538 us for 128 x 128
-// tiles of scalar FMAs, which gave 48 CTAs; with the columns stored as (b, b)
-// pairs in shared memory 232 us (its return path at 130 % of the FMA time).
-constexpr int SG_BM = 256, SG_BK = 8, SG_THREADS = 128, SG_TM = 16;
+// GPU (sgemm_shape).  M x columns x K, us per step of two GEMMs and sub-steps,
+// against slices of 8 held in registers on the way (16-byte loads, a row per
+// lane): 4000 x 256 x 4000 405 and 488 (40 TFLOP/s), 3992 x 32 x 3992 97 and 138,
+// 1000 x 128 x 1000 46 and 56, 1000 x 14 x 1000 35 and 48, 3000 x 200 x 3000 204
+// and 210 (538 us for one GEMM with 128 x 128 tiles of scalar FMAs, which gave 48
+// CTAs).  With the columns stored as (b, b) pairs in shared memory its return
+// path is at 130 % of the FMA time; slices of 16 through registers spilled.
+constexpr int SG_BM = 256, SG_BK = 16, SG_THREADS = 128, SG_TM = 16, SG_STAGES = 3;
 
 struct SgemmShape {
   int tn = 0;     // columns per thread
@@ -150,52 +154,59 @@ struct SgemmShape {
   int kshare = 0; // K per share, a multiple of SG_BK
 };
 
+// Columns of a B slice in shared memory: the swizzle stays within 32.
+__host__ __device__ constexpr int sg_cols(int tn) { return (8 * tn + 31) / 32 * 32; }
+constexpr int sg_smem_bytes(int tn) { return SG_STAGES * SG_BK * (SG_BM + sg_cols(tn)) * 4; }
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Four bytes, zero where `bytes` is 0.
+__device__ __forceinline__ void copy4_async(uint32_t dst, const float *src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
 template <int TN>
 __global__ void __launch_bounds__(SG_THREADS, TN <= 7 ? 2 : 1)
     sgemm_nt_kernel(const float *__restrict__ A, const float *__restrict__ B, float *__restrict__ Dt, int M, int Ncols,
                     int Kdim, int kshare) {
   constexpr int BN = 8 * TN;
-  constexpr int NB = (BN * SG_BK / 4 + SG_THREADS - 1) / SG_THREADS;  // float4 loads of B per thread
-  __shared__ __align__(16) float As[2][SG_BK][SG_BM + 4];
-  __shared__ float Bs[2][SG_BK][BN + 4];
+  constexpr int BS = sg_cols(TN);
+  constexpr int NA = SG_BM / 16, NB = (BN + 15) / 16;  // rows (columns) per thread, 16 apart
+  extern __shared__ __align__(16) float sg_smem[];
+  auto As = reinterpret_cast<float (*)[SG_BK][SG_BM]>(sg_smem);
+  auto Bs = reinterpret_cast<float (*)[SG_BK][BS]>(sg_smem + SG_STAGES * SG_BK * SG_BM);
   const int tid = threadIdx.x;
   const int tx = tid & 7, ty = tid >> 3;  // columns tx + 8 j; rows 64 i + 4 ty .. + 3, i = 0 .. 3
   const int m0 = blockIdx.x * SG_BM, n0 = blockIdx.y * BN;
   const int kb = blockIdx.z * kshare, ke = min(kb + kshare, Kdim);
-  const bool ok0 = m0 + tid < M, ok1 = m0 + 128 + tid < M;
-  const float *A0 = A + (size_t)(ok0 ? m0 + tid : 0) * Kdim, *A1 = A + (size_t)(ok1 ? m0 + 128 + tid : 0) * Kdim;
-  float4 ra[4], rb[NB];
-  // Kdim and kshare are multiples of 8: a slice lies wholly inside or outside
-  auto load = [&](int k0) {
-    const float4 zero = make_float4(0, 0, 0, 0);
-    ra[0] = ok0 ? *(const float4 *)(A0 + k0) : zero;
-    ra[1] = ok0 ? *(const float4 *)(A0 + k0 + 4) : zero;
-    ra[2] = ok1 ? *(const float4 *)(A1 + k0) : zero;
-    ra[3] = ok1 ? *(const float4 *)(A1 + k0 + 4) : zero;
+  // A copy instruction of a warp: a 32-byte sector of each of four rows.  Element
+  // (k, r) lies at [k][r ^ 4 (k mod 8)]: the 32 words on 32 banks, and four rows
+  // of one k still together.  Rows past the end repeat the last one (their
+  // outputs are not stored).
+  const int lk = tid & 7, lr = tid >> 3;
+  const float *Ab = A + (size_t)m0 * Kdim + lk, *Bb = B + (size_t)n0 * Kdim + lk;
+  uint32_t oa[NA], ob[NB];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int c = tid + q * SG_THREADS, n = c >> 1;
-      rb[q] = (n < BN && n0 + n < Ncols) ? *(const float4 *)(B + (size_t)(n0 + n) * Kdim + k0 + 4 * (c & 1)) : zero;
-    }
-  };
-  auto store = [&](int buf) {
+  for (int q = 0; q < NA; ++q) oa[q] = (uint32_t)min(lr + 16 * q, M - 1 - m0) * (uint32_t)Kdim;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int m = tid + 128 * (q >> 1), k = 4 * (q & 1);
-      As[buf][k + 0][m] = ra[q].x;
-      As[buf][k + 1][m] = ra[q].y;
-      As[buf][k + 2][m] = ra[q].z;
-      As[buf][k + 3][m] = ra[q].w;
-    }
+  for (int q = 0; q < NB; ++q) ob[q] = (uint32_t)min(lr + 16 * q, Ncols - 1 - n0) * (uint32_t)Kdim;
+  // lr ^ 4 lk, its bit 4 (of lk alone) applied to 16 q
+  const int low = (lr ^ (4 * lk)) & 15, high = lk >> 2;
+  const uint32_t da = smem_addr(&As[0][lk][low]), db = smem_addr(&Bs[0][lk][low]);
+  // Kdim and kshare are multiples of 8: eight k's lie wholly inside the share or
+  // are zero
+  auto load = [&](int k0, int stage) {
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int c = tid + q * SG_THREADS, n = c >> 1, k = 4 * (c & 1);
-      if (n < BN) {
-        Bs[buf][k + 0][n] = rb[q].x;
-        Bs[buf][k + 1][n] = rb[q].y;
-        Bs[buf][k + 2][n] = rb[q].z;
-        Bs[buf][k + 3][n] = rb[q].w;
-      }
+    for (int h = 0; h < 2; ++h) {
+      const int k = k0 + 8 * h, bytes = k < ke ? 4 : 0;
+      const int ks = k < ke ? k : kb;
+      const uint32_t sa = da + (uint32_t)(stage * SG_BK + 8 * h) * (SG_BM * 4);
+      const uint32_t sb = db + (uint32_t)(stage * SG_BK + 8 * h) * (BS * 4);
+#pragma unroll
+      for (int q = 0; q < NA; ++q) copy4_async(sa + 64u * (uint32_t)(q ^ high), Ab + ks + oa[q], bytes);
+#pragma unroll
+      for (int q = 0; q < NB; ++q)
+        if (BN % 16 == 0 || lr + 16 * q < BN) copy4_async(sb + 64u * (uint32_t)(q ^ high), Bb + ks + ob[q], bytes);
     }
   };
   float2 acc[SG_TM / 2][TN];
@@ -203,20 +214,26 @@ __global__ void __launch_bounds__(SG_THREADS, TN <= 7 ? 2 : 1)
   for (int i = 0; i < SG_TM / 2; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
-  load(kb);
-  store(0);
-  __syncthreads();
-  int buf = 0;
+#pragma unroll
+  for (int q = 0; q + 1 < SG_STAGES; ++q) {
+    if (kb + q * SG_BK < ke) load(kb + q * SG_BK, q);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  int stage = 0;
   for (int k0 = kb; k0 < ke; k0 += SG_BK) {
-    const bool more = k0 + SG_BK < ke;
-    if (more) load(k0 + SG_BK);
+    asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
+    __syncthreads();  // this slice is there, and nobody reads the one before it any more
+    const int next = k0 + (SG_STAGES - 1) * SG_BK;
+    if (next < ke) load(next, stage == 0 ? SG_STAGES - 1 : stage - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
     float4 fa[2][4];
     float fb[2][TN];
     auto frag = [&](int q, int kk) {
+      const int r = (4 * ty) ^ (4 * (kk & 7));
 #pragma unroll
-      for (int i = 0; i < 4; ++i) fa[q][i] = *(const float4 *)&As[buf][kk][64 * i + 4 * ty];
+      for (int i = 0; i < 4; ++i) fa[q][i] = *(const float4 *)&As[stage][kk][64 * i + r];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) fb[q][j] = Bs[buf][kk][tx + 8 * j];
+      for (int j = 0; j < TN; ++j) fb[q][j] = Bs[stage][kk][(tx ^ (4 * (kk & 1))) + 8 * (j ^ ((kk & 7) >> 1))];
     };
     frag(0, 0);
 #pragma unroll
@@ -233,11 +250,7 @@ __global__ void __launch_bounds__(SG_THREADS, TN <= 7 ? 2 : 1)
         }
       }
     }
-    if (more) {
-      buf ^= 1;
-      store(buf);
-      __syncthreads();
-    }
+    stage = stage + 1 == SG_STAGES ? 0 : stage + 1;
   }
   float *D = Dt + (size_t)blockIdx.z * Ncols * M;
 #pragma unroll
@@ -287,19 +300,28 @@ SgemmShape sgemm_shape(int64_t M, int64_t Ncols, int64_t Kdim, int sm_count) {
   return best;
 }
 
+template <int TN>
+cudaError_t launch_sgemm_tn(const SgemmShape &p, const float *A, const float *B, float *Dt, int M, int Ncols, int Kdim,
+                            bool configure, cudaStream_t s) {
+  if (configure)
+    return cudaFuncSetAttribute(sgemm_nt_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, sg_smem_bytes(TN));
+  const dim3 grid((M + SG_BM - 1) / SG_BM, (Ncols + 8 * TN - 1) / (8 * TN), p.split);
+  sgemm_nt_kernel<TN><<<grid, SG_THREADS, sg_smem_bytes(TN), s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare);
+  return cudaGetLastError();
+}
+
+// configure: the kernel's shared memory instead of a launch.
 cudaError_t launch_sgemm(const SgemmShape &p, const float *A, const float *B, float *Dt, int M, int Ncols, int Kdim,
-                         cudaStream_t s) {
-  const dim3 grid((M + SG_BM - 1) / SG_BM, (Ncols + 8 * p.tn - 1) / (8 * p.tn), p.split);
+                         cudaStream_t s, bool configure = false) {
   switch (p.tn) {
-    case 1: sgemm_nt_kernel<1><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
-    case 2: sgemm_nt_kernel<2><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
-    case 3: sgemm_nt_kernel<3><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
-    case 5: sgemm_nt_kernel<5><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
-    case 7: sgemm_nt_kernel<7><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
-    case 8: sgemm_nt_kernel<8><<<grid, SG_THREADS, 0, s>>>(A, B, Dt, M, Ncols, Kdim, p.kshare); break;
+    case 1: return launch_sgemm_tn<1>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
+    case 2: return launch_sgemm_tn<2>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
+    case 3: return launch_sgemm_tn<3>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
+    case 5: return launch_sgemm_tn<5>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
+    case 7: return launch_sgemm_tn<7>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
+    case 8: return launch_sgemm_tn<8>(p, A, B, Dt, M, Ncols, Kdim, configure, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 constexpr int64_t kTimedStepStride = 8;
@@ -578,6 +600,8 @@ sde_status kuramoto_general_alloc(KuramotoCtx *k) {
       }
     }
   } else {
+    if ((e = launch_sgemm(g->sg, nullptr, nullptr, nullptr, 0, 0, 0, nullptr, true)) != cudaSuccess)
+      return cuda_fail(e, "cudaFuncSetAttribute(sgemm_nt_kernel)");
     if ((e = device_alloc((void **)&k->Kf32, NN * 4)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
     if ((e = device_alloc((void **)&k->Bt32, NR * 2 * 4 * 2)) != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   }
