@@ -938,6 +938,307 @@ cudaError_t launch_pairwise(const KurPairArgs &a, int64_t R, const PairShape &p,
   return cudaGetLastError();
 }
 
+// ---- pairwise form, a replica per cluster --------------------------------
+//
+// All steps in one launch, for populations whose stages are shorter than a
+// launch: a cluster of CS CTAs holds a replica, every CTA the sines and cosines
+// of all its N oscillators in shared memory (twice: theta, theta~) and the
+// state of its own share of the receivers in registers.  A stage is the sums
+// over one buffer, the sub-step of the own receivers, and their new sines and
+// cosines copied into the other buffer of every CTA of the cluster (one bulk
+// copy each, counted by the receiver's mbarrier; two alternate).  Nobody still
+// reads the buffer being written, or copies from it: a CTA sends stage s + 1
+// after it has received stage s from everyone, and each sent that after its
+// sums over the buffer that stage s + 1 replaces.  For the same reason a
+// receiver has armed a mbarrier again before the next data for it can arrive.
+//
+// Each warp takes every 16th group of four source pairs for all receivers of
+// the CTA, 64 at a time: eight lanes hold eight receivers each, and the four
+// groups of eight lanes take different pairs, so that one 16-byte load still
+// feeds sixteen packed FMAs (kur_pairwise_stage) however few receivers a CTA
+// has, and no warp has more to do than another.
+//
+// What bounds it: the latency of a stage's steps one after the other (1.5 us at
+// 100 oscillators), then the FMA pipe at about half its rate.  1000 oscillators,
+// 3 replicas: 4.3 us per step of two stages against 8.6 with a launch per stage;
+// with ordinary remote stores and a cluster barrier for the exchange 5.4.
+constexpr int kPcThreads = 512, kPcWarps = kPcThreads / 32;
+constexpr int kPcGroup = 64;  // receivers taken together
+
+struct PairClusterArgs {
+  uint32_t *theta;
+  const float *omega;
+  double *r_out;  // [samples][R]
+  int64_t N, R;
+  int64_t n_begin, n_end;
+  int32_t M;
+  int32_t chunk;   // receivers per CTA, even, <= kPcThreads
+  int32_t npairs;  // source pairs, a multiple of 64
+  float wscale, kc, kh, sc_noise;
+  PhiloxKeys keys;
+  uint32_t *err;
+  uint64_t wait_ns;  // limit of each wait for the other CTAs' stage
+};
+
+constexpr size_t kPcMaxSmem = 200 * 1024;
+
+// Receivers per CTA (whole source pairs) and source pairs (whole rounds of the warps).
+__host__ __device__ inline int64_t pair_cluster_chunk(int64_t N, int cs) { return ((N + cs - 1) / cs + 1) & ~1ll; }
+__host__ __device__ inline int64_t pair_cluster_pairs(int64_t N) { return ((N + 1) / 2 + 63) / 64 * 64; }
+size_t pair_cluster_smem(int64_t chunk, int64_t npairs) {
+  const size_t groups = (size_t)((chunk + kPcGroup - 1) / kPcGroup);
+  return 2 * sizeof(float4) * (size_t)npairs + sizeof(float) * groups * kPcGroup * kPcWarps;
+}
+
+template <bool EULER>
+__global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const PairClusterArgs A) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ float4 pc_smem[];  // [2][npairs] (s0, s1, -c0, -c1), then the warps' partial sums
+  __shared__ float2 red_r[32];
+  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ int expired;
+  const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int rep = blockIdx.x / cs;
+  const int N = (int)A.N, chunk = A.chunk, npairs = A.npairs;
+  const int groups = (chunk + kPcGroup - 1) / kPcGroup;
+  const int64_t base = (int64_t)rep * A.N;
+  float *part = reinterpret_cast<float *>(pc_smem + 2 * npairs);  // [warp][groups * 64]
+  const int i = crank * chunk + t;  // this thread's receiver
+  const bool own = t < chunk && i < N;
+  const bool active = (t & ~31) < chunk;  // this warp has receivers
+  // all sources of theta; pairs beyond N stay zero in both buffers
+  for (int p = t; p < npairs; p += kPcThreads) {
+    float s0 = 0.0f, c0 = 0.0f, s1 = 0.0f, c1 = 0.0f;
+    if (2 * p < N) sincos_turns(A.theta[base + 2 * p], s0, c0);
+    if (2 * p + 1 < N) sincos_turns(A.theta[base + 2 * p + 1], s1, c1);
+    pc_smem[p] = make_float4(s0, s1, -c0, -c1);
+    pc_smem[npairs + p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+  uint32_t th = own ? A.theta[base + i] : 0u;
+  const float wdt = own ? A.omega[base + i] * A.wscale : 0.0f;
+  // this CTA's pairs in a buffer, and the bytes a stage brings from the others
+  const int first = crank * chunk / 2, mine = max(0, min(chunk / 2, npairs - first));
+  const uint32_t bytes = 16u * (uint32_t)(min(npairs, cs * chunk / 2) - mine);
+  const uint32_t bar0 = smem_u32(&mbar[0]);
+  if (t == 0) {
+    expired = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * q) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 8 * q), "r"(bytes) : "memory");
+  }
+  cluster.sync();  // every CTA's buffers and barriers are there before the first copy into them
+  uint32_t stage = 0;
+
+  // sum_j sin(x_j - x_i) over the sources of buffer b for this thread's receiver
+  auto sums = [&](int b) -> float {
+    const float4 *src = pc_smem + b * npairs;
+    const int l = lane & 7;
+    for (int g = 0; g < groups; ++g) {
+      float si[8], ci[8];
+      float2 acc[8];
+      const int p0 = (crank * chunk + g * kPcGroup) / 2 + l * 4;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 v = p0 + k < npairs ? src[p0 + k] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        si[2 * k] = v.x;
+        si[2 * k + 1] = v.y;
+        ci[2 * k] = -v.z;
+        ci[2 * k + 1] = -v.w;
+        acc[2 * k] = acc[2 * k + 1] = make_float2(0.0f, 0.0f);
+      }
+#pragma unroll 2
+      for (int p = warp * 4 + (lane >> 3); p < npairs; p += 4 * kPcWarps) pair_terms<8>(src[p], si, ci, acc);
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = acc[k].x + acc[k].y;
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], 8);
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
+      }
+      if (lane < 8) {
+        float4 *o = reinterpret_cast<float4 *>(part + (warp * groups + g) * kPcGroup + l * 8);
+        o[0] = make_float4(v[0], v[1], v[2], v[3]);
+        o[1] = make_float4(v[4], v[5], v[6], v[7]);
+      }
+    }
+    __syncthreads();
+    float sum = 0.0f;
+    if (t < chunk) {
+#pragma unroll
+      for (int w = 0; w < kPcWarps; ++w) sum += part[w * groups * kPcGroup + t];
+    }
+    return sum;
+  };
+  // the new sine and cosine of the own receiver into buffer b of every CTA
+  auto publish = [&](uint32_t phase, int b) {
+    float4 *dst = pc_smem + b * npairs;
+    if (active) {
+      float sn, cs_;
+      sincos_turns(phase, sn, cs_);
+      if (!own) sn = cs_ = 0.0f;
+      const float s1 = __shfl_xor_sync(0xffffffffu, sn, 1), c1 = __shfl_xor_sync(0xffffffffu, cs_, 1);
+      if ((t & 1) == 0 && t / 2 < mine) {
+        dst[first + t / 2] = make_float4(sn, s1, -cs_, -c1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+    }
+    __syncthreads();
+    if (lane == 0 && warp < cs && warp != crank && mine > 0 && !*(volatile int *)&expired) {
+      const uint32_t from = smem_u32(dst + first);
+      asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       cluster_map(from, (uint32_t)warp)),
+                   "r"(from), "r"(16u * (uint32_t)mine), "r"(cluster_map(bar0 + 8 * (stage & 1u), (uint32_t)warp))
+                   : "memory");
+    }
+  };
+  // the other CTAs' part of the stage; once a wait has expired the CTA records it
+  // and runs to its end without waiting or sending (the others' waits expire too)
+  auto receive = [&]() {
+    if (bytes > 0) {
+      const uint32_t bar = bar0 + 8 * (stage & 1u), parity = (stage >> 1) & 1u;
+      const bool ok = !*(volatile int *)&expired && mbar_wait_bounded(bar, parity, A.wait_ns);
+      if (!ok) {
+        expired = 1;
+        atomicOr(A.err, kErrTimeout);
+      }
+      if (t == 0 && ok)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    }
+    ++stage;
+  };
+  auto order = [&](int b, int64_t row) {  // r(t) of the replica, by the CTA of rank 0
+    float S = 0.0f, C = 0.0f;
+    for (int p = t; p < npairs; p += kPcThreads) {
+      const float4 v = pc_smem[b * npairs + p];
+      S += v.x + v.y;
+      C -= v.z + v.w;
+    }
+    const float2 sc = block_sum2(S, C, red_r);
+    if (t == 0) {
+      const double Sd = sc.x, Cd = sc.y;
+      A.r_out[row * A.R + rep] = sqrt(Sd * Sd + Cd * Cd) / (double)N;
+    }
+    __syncthreads();
+  };
+
+  int b = 0;  // the buffer of theta_n
+  int64_t row = 0;
+  int m = 0;  // (n - n_begin) mod M
+  float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  auto draw = [&](int64_t n) {
+    if (active) gauss4((uint32_t)(n >> 2), (uint32_t)i, (uint32_t)rep, kTagKuramoto, A.keys, z);
+  };
+  if (A.n_begin < A.n_end) draw(A.n_begin);
+  for (int64_t n = A.n_begin; n < A.n_end; ++n) {
+    if (A.M > 0) {
+      if (m == 0) {
+        if (crank == 0) order(b, row);
+        ++row;
+      }
+      if (++m == A.M) m = 0;
+    }
+    const float psi = pick4(z, (int)(n & 3));
+    const float g1 = sums(b);
+    const float d1 = fmaf(A.sc_noise, psi, fmaf(A.kc, g1, wdt));
+    const uint32_t tp = th + (uint32_t)__float2int_rn(d1 * 4294967296.0f);
+    if (EULER) {
+      th = tp;
+      b ^= 1;
+    } else {
+      publish(tp, 1);
+      receive();
+      const float g2 = sums(1);
+      const float d = fmaf(A.sc_noise, psi, fmaf(A.kh, g1 + g2, wdt));
+      th += (uint32_t)__float2int_rn(d * 4294967296.0f);
+    }
+    publish(th, b);
+    if (((n + 1) & 3) == 0) draw(n + 1);  // while the others' data arrives
+    receive();
+  }
+  if (A.M > 0 && crank == 0) order(b, row);
+  if (own) A.theta[base + i] = th;
+  cluster.sync();
+  // every copy has arrived, unless a wait expired: then the last ones get time to
+  if (cs > 1 && *(volatile int *)&expired) __nanosleep(200000);
+}
+
+// Shared memory and cluster size of the kernel's launches (not under capture).
+cudaError_t pair_cluster_configure() {
+  for (const void *fn : {(const void *)kur_pair_cluster_kernel<false>, (const void *)kur_pair_cluster_kernel<true>}) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPcMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaLaunchConfig_t pair_cluster_config(int64_t N, int64_t R, int cs, cudaLaunchAttribute *attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(R * cs));
+  cfg.blockDim = dim3(kPcThreads);
+  cfg.dynamicSmemBytes = pair_cluster_smem(pair_cluster_chunk(N, cs), pair_cluster_pairs(N));
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cs;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+cudaError_t launch_pair_cluster(const PairClusterArgs &a, int cs, bool euler, cudaStream_t s) {
+  cudaLaunchAttribute attr;
+  cudaLaunchConfig_t cfg = pair_cluster_config(a.N, a.R, cs, &attr);
+  cfg.stream = s;
+  if (euler) return cudaLaunchKernelEx(&cfg, kur_pair_cluster_kernel<true>, a);
+  return cudaLaunchKernelEx(&cfg, kur_pair_cluster_kernel<false>, a);
+}
+
+// CTAs per replica of the cluster form, or 0 where a launch per stage is the
+// faster one, from a model of both in ns per stage.  A launch: 3.6 us and the
+// busiest SM's blocks at the rate that their receivers per thread reach; a
+// cluster stage: 1.3 us of sums, sub-step and exchange, and per 64 receivers 0.33
+// us and 1.17 ns per source pair, times the waves of clusters.  Both sides
+// measured, us per stage, launch and cluster: 1000 oscillators x 3 replicas 4.3
+// and 2.2, x 19 6.4 and 5.2, x 40 8.4 and 8.9; 2000 x 1 6.4 and 4.5, x 9 8.4 and
+// 7.5, x 18 10.5 and 13.0; 3000 x 2 6.4 and 7.8; 4096 x 1 8.4 and 12; 900 x 64
+// 10.5 and 8.9; 300 x 200 6.4 and 9.1.
+int pair_cluster_size(int64_t N, int64_t R, bool euler, int sm_count) {
+  const double terms_per_ns = 128.0 / 2 * 1.9;  // of an SM: two FMAs per term
+  const PairShape shape = pair_shape(N, R, sm_count);
+  const int64_t blocks = (N + shape.receivers() - 1) / shape.receivers() * R;
+  const double slack = shape.rpt == 8 ? 1.25 : (shape.rpt == 4 ? 1.6 : 2.2);  // shared loads per FMA
+  const double busiest = (double)((blocks + sm_count - 1) / sm_count) * shape.receivers() * (double)N;
+  double best = 3600.0 + slack * busiest / terms_per_ns + (euler ? 3000.0 : 0.0);  // PROG2's second launch
+  int best_cs = 0;
+  for (int cs = 16; cs >= 1; cs >>= 1) {
+    const int64_t chunk = pair_cluster_chunk(N, cs), npairs = pair_cluster_pairs(N);
+    if (chunk > kPcThreads || R * cs > 1 << 20 || pair_cluster_smem(chunk, npairs) > kPcMaxSmem) continue;
+    const double groups = (double)((chunk + kPcGroup - 1) / kPcGroup);
+    const double stage = 1300.0 + groups * (330.0 + 1.17 * (double)npairs);
+    if (stage * (double)((R * cs + sm_count - 1) / sm_count) >= best) continue;  // without asking the driver
+    if (pair_cluster_configure() != cudaSuccess) break;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = pair_cluster_config(N, R, cs, &attr);
+    int resident = 0;
+    if (cudaOccupancyMaxActiveClusters(&resident, (const void *)kur_pair_cluster_kernel<false>, &cfg) != cudaSuccess ||
+        resident < 1)
+      continue;
+    const double ns = stage * (double)((R + resident - 1) / resident);
+    if (ns < best) {
+      best = ns;
+      best_cs = cs;
+    }
+  }
+  cudaGetLastError();  // a form that the device does not take is no error
+  return best_cs;
+}
+
 // PROG2's AdvanceSystem with Euler-Maruyama: theta += wdt + kc g + sc psi
 // for every oscillator of every replica, g the stored coupling sums.
 __global__ void kur_advance_euler_kernel(const KurPairArgs A, int64_t R) {
@@ -1425,11 +1726,14 @@ sde_status kuramoto_create(const sde_config *cfg, int sm_count, uint32_t *err, K
   // the grid-wide form is a candidate when few replicas leave SMs idle
   const bool grid_possible =
       mf && (grid_forced || (cfg->cluster_ctas == 0 && cfg->block_threads == 0 && cfg->n_replicas * 4 < sm_count));
-  if (cfg->model == SDE_KURAMOTO_PAIRWISE || grid_possible) {
+  const bool pairwise = cfg->model == SDE_KURAMOTO_PAIRWISE;
+  if (pairwise)
+    k->pair_cs = pair_cluster_size(k->N, k->R, (cfg->flags & SDE_FLAG_EULER) != 0, sm_count);
+  if ((pairwise && k->pair_cs == 0) || grid_possible) {
     alloc((void **)&k->theta_t, NR * 4);
     alloc((void **)&k->g1, NR * 4);
   }
-  if (cfg->model == SDE_KURAMOTO_PAIRWISE) alloc((void **)&k->pair_sc, NR * 2 * sizeof(float2));
+  if (pairwise && k->pair_cs == 0) alloc((void **)&k->pair_sc, NR * 2 * sizeof(float2));
   if (grid_possible) {
     mfg_grid_for(k->N, k->R, sm_count, k->mfg_grid);
     k->mfg_blocks = *std::max_element(k->mfg_grid, k->mfg_grid + 4);
@@ -1485,7 +1789,11 @@ sde_status kuramoto_create(const sde_config *cfg, int sm_count, uint32_t *err, K
     }
     k->block = block;
     k->opt = opt;
-  } else if (cfg->model == SDE_KURAMOTO_PAIRWISE) {
+  } else if (pairwise && k->pair_cs > 0) {
+    k->cs = k->pair_cs;
+    k->block = kPcThreads;
+    k->opt = 1;
+  } else if (pairwise) {
     const PairShape p = pair_shape(k->N, k->R, sm_count);
     k->block = p.threads();
     k->opt = p.rpt;
@@ -1615,6 +1923,29 @@ sde_status kuramoto_run(KuramotoCtx *k, const sde_run_desc *r, cudaStream_t s, c
     a.err = k->err;
     a.wait_ns = k->wait_ns;
     SDE_CUDA_TRY(launch_meanfield(a, k->block, k->opt, k->cs, k->mf_async, s));
+  } else if (k->model == SDE_KURAMOTO_PAIRWISE && k->pair_cs > 0) {
+    PairClusterArgs a{};
+    a.theta = k->theta;
+    a.omega = r->omega_dev;
+    a.r_out = rbuf;
+    a.N = k->N;
+    a.R = k->R;
+    a.n_begin = r->n_begin;
+    a.n_end = r->n_end;
+    a.M = k->M;
+    a.chunk = (int32_t)pair_cluster_chunk(k->N, k->pair_cs);
+    a.npairs = (int32_t)pair_cluster_pairs(k->N);
+    a.wscale = (float)(k->dt * inv2pi);
+    a.kc = (float)(k->K / (double)k->N * k->dt * inv2pi);
+    a.kh = (float)(0.5 * k->K / (double)k->N * k->dt * inv2pi);
+    a.sc_noise = (float)(sqrt(2.0 * k->D * k->dt) * inv2pi);
+    a.keys = philox_round_keys(k->seed);
+    a.err = k->err;
+    a.wait_ns = k->wait_ns;
+    const bool euler = (k->flags & SDE_FLAG_EULER) != 0;
+    SDE_CUDA_TRY(ktime_begin(k, s));
+    SDE_CUDA_TRY(launch_pair_cluster(a, k->pair_cs, euler, s));
+    SDE_CUDA_TRY(ktime_end(k, s, (euler ? 1 : 2) * (r->n_end - r->n_begin)));  // per stage
   } else if (k->model == SDE_KURAMOTO_PAIRWISE) {
     KurPairArgs a{};
     a.theta = k->theta;

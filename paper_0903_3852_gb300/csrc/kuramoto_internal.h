@@ -37,6 +37,7 @@ struct KuramotoCtx {
   uint32_t *theta_t = nullptr;  // predictor phases (pairwise, general, grid-wide mean field)
   float *g1 = nullptr;          // first-stage coupling sums (pairwise, general); grid-wide
                                 // mean field: the first-stage part of the step increment
+  int pair_cs = 0;              // pairwise: CTAs per replica of the cluster form, 0 = a launch per stage
   float2 *pair_sc = nullptr;    // pairwise: [2][R][N] (sin, cos) of theta, then of theta~
   double *r_scratch = nullptr;  // r samples when the caller passes none
   int64_t r_scratch_rows = 0;

@@ -67,6 +67,23 @@ def test_async_meanfield_wait_expiry_is_reported_and_recovered():
     assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
 
 
+def test_pairwise_cluster_wait_expiry_is_reported_and_recovered():
+    N, R, steps = 1000, 2, 200
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=R, seed=33)
+    ensure_built()
+    ref = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, 2.0, 0.05, 0.01, 4, sample_every=50)
+    phi_ref, r_ref, _ = kur_run(ref, w["phi0"], w["omega"], 0, steps)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, 2.0, 0.05, 0.01, 4, sample_every=50)
+    assert ens.tuning()[2] > 1
+    ens.set_wait_limit(1)
+    with pytest.raises(sde.SDEError) as e:
+        kur_run(ens, w["phi0"], w["omega"], 0, steps)
+    assert e.value.status == sde.SDE_ERR_TIMEOUT
+    ens.set_wait_limit(0)
+    phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+    assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
+
+
 @pytest.mark.parametrize("kind", ["josephson", "kuramoto_general", "mlp"])
 def test_every_injected_allocation_failure_reports_no_memory(kind):
     ensure_built()

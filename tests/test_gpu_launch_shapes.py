@@ -61,6 +61,29 @@ def test_grid_wide_chunks_match_replica_form(N, R, shift):
     assert np.abs(got[0][1] - got[1][1]).max() <= 2e-5
 
 
+@pytest.mark.parametrize("N,R", [(1, 1), (2, 3), (129, 9), (512, 1), (513, 20), (1023, 2), (2000, 4)])
+@pytest.mark.parametrize("euler", [False, True])
+def test_pairwise_cluster_form_resumes(N, R, euler):
+    """A replica per cluster, at the edges of its groups of receivers and rounds of
+    sources: steps 3 .. 10 in one run and in two (the phases return in FP32
+    between them: 2.4e-7, grown by at most 1 + K dt per step), and against the
+    mean-field form with the bound above."""
+    ensure_built()
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=R, seed=N)
+    kw = dict(K=2.0, D=0.05, dt=0.01, seed=3, sample_every=3)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, flags=sde.SDE_FLAG_EULER if euler else 0, **kw)
+    assert ens.tuning()[0] == 512 and ens.tuning()[1] == 1  # the cluster form
+    phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 3, 10)
+    half, _, _ = kur_run(ens, w["phi0"], w["omega"], 3, 6)
+    two, _, _ = kur_run(ens, half.astype(np.float32), w["omega"], 6, 10)
+    assert np.abs(angle_diff(phi, two)).max() <= 1e-6
+    if not euler:
+        mf = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_MEANFIELD, N, R, **kw)
+        phi_mf, r_mf, _ = kur_run(mf, w["phi0"], w["omega"], 3, 10)
+        assert np.abs(angle_diff(phi, phi_mf)).max() <= 1e-6
+        assert np.abs(r - r_mf).max() <= 2e-5
+
+
 @pytest.mark.parametrize("N,R", [(8, 1), (16, 3), (136, 13), (264, 25), (512, 100), (1000, 7), (3000, 28)])
 def test_fp32_gemm_shapes(N, R):
     """Coupling sums of the FP32 form against FP64: every chain of N FMAs errs by
