@@ -15,7 +15,7 @@
 // with stored pre-activations, backward, Adam) runs on the CUDA cores, every
 // sum over k in ascending order with one FMA per term: about a dozen launches
 // per step for all members together (members are a grid dimension):
-// 180 us for 4 members of 1024 points, 1.70 ms when each member's layers were
+// 155 us for 4 members of 1024 points, 1.70 ms when each member's layers were
 // launched by themselves.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -66,7 +66,11 @@ __device__ __forceinline__ float bf16_round(float v) { return __bfloat162float(_
 // gradients of both square layers (one member's layer at a time: 17, 27 and 84
 // us each).  Measured beside it: 4 x 4 outputs in 256 threads (23, 26, 37 us);
 // 8 x 8 (gradients 8 x 4) in 64 threads from BF16 in shared memory, half the
-// shared traffic but one warp per scheduler (28, 32, 59 us).
+// shared traffic but one warp per scheduler (28, 32, 59 us); these tiles from
+// BF16 in shared memory (a step of all launches 8 us longer: the conversions cost
+// more than the loads).  Matrix instructions would take 94 us per step, but another
+// order of summation flips BF16 roundings of activations and moves the parameters
+// by 4e-5 within eight steps.
 enum Epi { EPI_FWD = 0, EPI_DSILU = 1, EPI_DW = 2 };
 
 constexpr int TM = 64, TN = 64, TK = 32, GT = 128, TPAD = 4, kF = 2;
@@ -143,6 +147,8 @@ __global__ void __launch_bounds__(GT) mlp_gemm_kernel(const GemmArgs g) {
   constexpr bool A_T = EPI == EPI_DW, B_T = EPI != EPI_FWD;
   __shared__ __align__(16) float As[2][TK][TM + TPAD];
   __shared__ __align__(16) float Bs[2][TK][TN + TPAD];
+  // the small gradients, which need nothing from this launch, may start
+  if (EPI == EPI_DW) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int layer = EPI == EPI_DW ? (int)(blockIdx.z % g.n_layers) : 0;
   const int64_t member = EPI == EPI_DW ? blockIdx.z / g.n_layers : blockIdx.z;
@@ -160,6 +166,15 @@ __global__ void __launch_bounds__(GT) mlp_gemm_kernel(const GemmArgs g) {
   sa.store(As[0]);
   sb.store(Bs[0]);
   __syncthreads();
+  float4 zv[8];  // EPI_DSILU: the pre-activations, in flight during the slices
+  if (EPI == EPI_DSILU) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int64_t m = m0 + (i < 4 ? 0 : 32) + ty * 4 + (i & 3);
+      zv[i] = m < B ? *reinterpret_cast<const float4 *>(g.z + (member * g.rows + m) * H + n0 + tx * 4)
+                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+  }
   float2 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -229,7 +244,7 @@ __global__ void __launch_bounds__(GT) mlp_gemm_kernel(const GemmArgs g) {
         *reinterpret_cast<float4 *>(g.z + o) = make_float4(c[0], c[1], c[2], c[3]);
         *reinterpret_cast<uint2 *>(g.h + o) = *reinterpret_cast<const uint2 *>(hv);
       } else {
-        const float4 z = *reinterpret_cast<const float4 *>(g.z + o);
+        const float4 z = zv[i];
         *reinterpret_cast<float4 *>(g.z + o) =
             make_float4(bf16_round(silu_grad(c[0], z.x)), bf16_round(silu_grad(c[1], z.y)),
                         bf16_round(silu_grad(c[2], z.z)), bf16_round(silu_grad(c[3], z.w)));
@@ -487,7 +502,7 @@ __device__ __forceinline__ void chain_grad(const T *D, int64_t ldd, const float 
     if (kq + k < nk) out[(int64_t)(n0 + col) * nk + kq + k] = acc[k];
 }
 
-__global__ void __launch_bounds__(256) mlp_small_grad_kernel(const SmallArgs a) {
+__device__ __forceinline__ void small_grad(const SmallArgs &a) {
   __shared__ __align__(16) float Ds[kChainRows][64];
   __shared__ __align__(16) float Fs[kChainRows][8];
   __shared__ float red[32];
@@ -537,6 +552,16 @@ __global__ void __launch_bounds__(256) mlp_small_grad_kernel(const SmallArgs a) 
     grad[a.bo] = s;
     if (a.loss) a.loss[member] = sq / (float)a.B;
   }
+}
+
+// Launched so that it runs beside the square layers' weight gradients, which
+// leave most of an SM's warps free: its inputs were complete before that launch
+// began.  The wait at its end makes it end after them.  4 members x 1024 points:
+// 172.6 us per step with the two launches one after the other, 155.5 together;
+// 20,000 points 2.19 and 1.94 ms.
+__global__ void __launch_bounds__(256) mlp_small_grad_kernel(const SmallArgs a) {
+  small_grad(a);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) for weights and biases.
@@ -778,7 +803,16 @@ sde_status mlp_grad_members(sde_mlp *q, int64_t m0, int64_t G, const float *X, i
   a.bo = q->boff[nh];
   a.grad = grad;
   a.loss = loss;
-  mlp_small_grad_kernel<<<dim3((unsigned)(2 * (H / 64) + nh * (H / 8) + 1), (unsigned)G), 256, 0, s>>>(a);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * (H / 64) + nh * (H / 8) + 1), (unsigned)G);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = nh > 1 ? 1 : 0;  // only behind the weight-gradient launch
+  SDE_CUDA_TRY(cudaLaunchKernelEx(&cfg, mlp_small_grad_kernel, a));
   SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }
