@@ -42,6 +42,7 @@ PAPER_FLOP_PER_STEP = 79  # Table 1 (Appendix): FLOP per SRK2 step of Eq. 1, wei
 COUNTED_FLOP_PER_PATH_STEP = 52.27
 PAPER_FLOP_MEANFIELD = 66  # Fig. 5: operations per step of PROG3 (Eq. 3, mean field)
 PAPER_FLOP_PAIR = 6  # Fig. 5: 44 + 6N operations per step of PROG2, 6 per pair term
+COUNTED_FLOP_PAIR = 4  # two FMAs per pair term, as the stage kernel executes them
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -422,8 +423,8 @@ def run_ours(args, rank, world, device):
         else:
             units = float(w["n_osc"] ** 2 * w["replicas"] * S)
             metric = "pair-terms/sec"
-            flop_per_unit = PAPER_FLOP_PAIR
-            launches_per_step = 2 * S + S // w["sample_every"] + 4
+            flop_per_unit = COUNTED_FLOP_PAIR
+            launches_per_step = 2 * S + S // w["sample_every"] + 5
             flop_per_launch = flop_per_unit * w["n_osc"] ** 2 * w["replicas"]  # one stage launch
         cfg = {"workload": kuramoto_workload_name(args.workload, euler, w["n_osc"], w["replicas"]),
                "steps_per_bench_step": S, "K": w["K"], "D": w["D"], "dt": w["dt"],
@@ -557,6 +558,7 @@ def run_ours(args, rank, world, device):
         peak_note = ("FP32 FMA probe measured in this run (%.1f TFLOP/s at %s MHz; %.1f derived from 128 "
                      "lanes x 2 FLOP x 2070 MHz)" % (fp32["tflops"], fp32["sm_mhz"], fp32["derived_2070mhz"]))
         flop_note = ("2 N (2R) N FLOP per GEMM launch (FP32 FMA)" if args.workload == "kuramoto-general-fp32"
+                     else "4 FLOP per pair term (two FMAs; the paper counts 6)" if args.workload == "kuramoto-pairwise"
                      else "%d FLOP per unit (paper Table 1 weighting)" % flop_per_unit)
     counted = args.workload in ("sweep", "plain", "fig2") and not args.euler
     if args.workload in ("sweep", "plain", "fig2"):
@@ -577,7 +579,7 @@ def run_ours(args, rank, world, device):
         traffic = 8.23 * n  # 8.23 B per path: the initial state read once
         traffic_src = "ncu capture of the sweep kernel (2000-step cap), scaled by paths"
     elif args.workload == "kuramoto-fig4":
-        traffic = 16.6 * w["n_osc"] * w["replicas"]  # mean over the launches of 4 steps
+        traffic = 15.7 * w["n_osc"] * w["replicas"]  # mean over the launches of 4 steps
         traffic_src = "ncu capture of the grid-wide mean-field launches"
     elif (args.workload == "kuramoto-general" and fused and not args.gemm_single_cta
           and not args.gemm_stream_k):
@@ -585,10 +587,10 @@ def run_ours(args, rank, world, device):
         traffic_src = ("ncu capture of the fused CTA-pair GEMM (mean of its predictor and corrector "
                        "launches)")
     elif args.workload == "kuramoto-meanfield":
-        traffic = 2.26e6  # phases and omega read once per run; results stay in L2
+        traffic = 2.16e6  # phases and omega read once per run; results stay in L2
         traffic_src = "ncu capture of the asynchronous-exchange cluster mean-field kernel"
     elif args.workload == "kuramoto-pairwise" and not args.euler:
-        traffic = 2.11e6
+        traffic = 4.7e6  # mean of the two stages: phases, their sines and cosines, omega
         traffic_src = "ncu capture of the pairwise stage kernel"
     res = {
         "metric": metric,
