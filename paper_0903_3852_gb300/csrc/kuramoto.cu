@@ -553,6 +553,19 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
 
 // ---- mean field over the whole grid ------------------------------------
 
+// The launches of a step follow one another closely: each starts while the one
+// before it ends (its blocks take the places as they become free) and waits here
+// until that one's results are all there.  It lets the next one do the same; a
+// grid that waits has started all its blocks, so nothing it needs is kept out.
+// Per step, against plain launches: 16.7 -> 13.0 us for 3 replicas of 20,000
+// oscillators, 21.1 -> 17.0 for 8 of 91,126, 118.5 -> 115.4 for one of 2^24.  The
+// pairwise stages are not launched so: their blocks are few and long, and started
+// early they land unevenly on the SMs (6000 x 1: 18 -> 32 us).
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int kMfgThreads = 256;
 constexpr int kMfgIlp = 4;  // oscillators per thread per iteration: one 16-byte access per array
 
@@ -634,6 +647,7 @@ struct MfgArgs {
 // but the first starts on a 16-byte boundary: 80.4 -> 66.5 us.
 template <int MODE>
 __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 5)) kur_mfg_kernel(const MfgArgs A) {
+  chain_begin();
   constexpr bool kPred = MODE == 0 || MODE == 3;
   constexpr bool kGen = MODE == 3;
   __shared__ float2 red[32];
@@ -1456,14 +1470,21 @@ void mfg_grid_for(int64_t N, int64_t R, int sm_count, int grid[4]) {
 }
 
 cudaError_t launch_mfg(const MfgArgs &a, int mode, int blocks, cudaStream_t s) {
-  const dim3 grid((unsigned)blocks, (unsigned)a.R);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, (unsigned)a.R);
+  cfg.blockDim = dim3(kMfgThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;  // chain_begin
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   switch (mode) {
-    case 0: kur_mfg_kernel<0><<<grid, kMfgThreads, 0, s>>>(a); break;
-    case 1: kur_mfg_kernel<1><<<grid, kMfgThreads, 0, s>>>(a); break;
-    case 3: kur_mfg_kernel<3><<<grid, kMfgThreads, 0, s>>>(a); break;
-    default: kur_mfg_kernel<2><<<grid, kMfgThreads, 0, s>>>(a); break;
+    case 0: return cudaLaunchKernelEx(&cfg, kur_mfg_kernel<0>, a);
+    case 1: return cudaLaunchKernelEx(&cfg, kur_mfg_kernel<1>, a);
+    case 3: return cudaLaunchKernelEx(&cfg, kur_mfg_kernel<3>, a);
+    default: return cudaLaunchKernelEx(&cfg, kur_mfg_kernel<2>, a);
   }
-  return cudaGetLastError();
 }
 
 // Oscillators per thread the replica kernels are built for, the smallest that
