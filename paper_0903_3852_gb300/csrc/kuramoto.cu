@@ -12,9 +12,10 @@
 //    block to finish (fixed-order FP64 sum of the per-block partials, no
 //    waiting between blocks).
 //  * pairwise (Alg. 3 / Fig. 3): the direct all-pairs sum, tiles of source
-//    phases staged in shared memory; one launch per SRK2 stage with the
-//    sub-step fused into the epilogue (Sec. 4.2 splits it into UpdateRHS and
-//    AdvanceSystem; higher order by interleaving stages).
+//    sines and cosines staged in shared memory; one launch per SRK2 stage with
+//    the sub-step fused into the epilogue (Sec. 4.2 splits it into UpdateRHS and
+//    AdvanceSystem; higher order by interleaving stages), or, for small
+//    populations, all steps in one launch with a replica per cluster.
 //  * general K_ij: the sum as a GEMM against [sin x | cos x] (see
 //    kuramoto_general.cu).
 //
