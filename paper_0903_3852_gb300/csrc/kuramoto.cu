@@ -1031,6 +1031,8 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     pc_smem[p] = make_float4(s0, s1, -c0, -c1);
     pc_smem[npairs + p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
+  // the others' copies overwrite these through the asynchronous proxy: ordered after them
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   uint32_t th = own ? A.theta[base + i] : 0u;
   const float wdt = own ? A.omega[base + i] * A.wscale : 0.0f;
   // this CTA's pairs in a buffer, and the bytes a stage brings from the others
