@@ -385,6 +385,45 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
+// The end of a cluster kernel whose CTAs send one another a stage's data
+// asynchronously, counted by two alternating mbarriers of the receiver (bar0
+// and the next; stage s on barrier s & 1), when a wait may have expired.  A CTA
+// barrier of the cluster orders threads, not the copies they issued, and a CTA
+// that ends while a copy still reads or writes its shared memory is a fault;
+// so if any CTA of the cluster gave up, every CTA stays until all that was sent
+// to it has arrived.  Both open phases of its barriers (stages got and got + 1:
+// nobody sends a later one before this CTA has sent stage got + 1) are credited
+// with what was never sent, `missing(stage)` bytes, so they complete when the
+// last copy in flight lands; the wait for that is bounded by a second whatever
+// the context's limit.  Nothing is waited for when no wait expired: then every
+// stage was received by everyone before this.
+//
+// late: this thread's wait expired (any thread of the CTA may say so); got:
+// stages that thread 0 received; flag: a word of shared memory, zero since
+// before the kernel's first cluster barrier.  All threads of the cluster call it.
+template <typename Missing>
+__device__ __forceinline__ void cluster_drain(bool late, uint32_t got, uint32_t bar0, int *flag, int cs,
+                                              Missing missing) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  late = __syncthreads_or(late);
+  if (late && (int)threadIdx.x < cs)  // their CTAs are still there: they have not passed the barrier below
+    *(volatile int *)cluster.map_shared_rank(flag, threadIdx.x) = 1;
+  cluster.sync();  // every copy that ever will be is issued, every count of them written
+  if (*(volatile int *)flag == 0) return;
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (uint32_t s = got; s < got + 2u; ++s) {
+      const uint32_t bytes = missing(s);
+      if (bytes > 0)
+        asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8u * (s & 1u)), "r"(bytes)
+                     : "memory");
+    }
+    for (uint32_t s = got; s < got + 2u; ++s) mbar_wait_bounded(bar0 + 8u * (s & 1u), (s >> 1) & 1u, 1000000000ull);
+  }
+  cluster.sync();  // everything sent has arrived everywhere: no CTA's memory is in use any more
+}
+
 // The cluster mean field with the exchange done by st.async: every warp
 // sends its (S, C) pair into its slot of every CTA of the cluster with an
 // asynchronous remote store that completes on the receiving CTA's mbarrier
@@ -1012,7 +1051,8 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   extern __shared__ float4 pc_smem[];  // [2][npairs] (s0, s1, -c0, -c1), then the warps' partial sums
   __shared__ float2 red_r[32];
   __shared__ __align__(8) uint64_t mbar[2];
-  __shared__ int expired;
+  __shared__ int gave_up;       // some CTA of the cluster did
+  __shared__ uint32_t sent_s;   // stages this CTA sent
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int rep = blockIdx.x / cs;
@@ -1040,7 +1080,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   const uint32_t bytes = 16u * (uint32_t)(min(npairs, cs * chunk / 2) - mine);
   const uint32_t bar0 = smem_u32(&mbar[0]);
   if (t == 0) {
-    expired = 0;
+    gave_up = 0;
 #pragma unroll
     for (int q = 0; q < 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * q) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1049,7 +1089,9 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 8 * q), "r"(bytes) : "memory");
   }
   cluster.sync();  // every CTA's buffers and barriers are there before the first copy into them
-  uint32_t stage = 0;
+  uint32_t stage = 0, sent = 0, got = 0;  // got: stages received, as thread 0 counts them
+  bool late = false;                      // a wait of this thread expired
+  bool stop = false;                      // a wait of this CTA did, known to all its threads
 
   // sum_j sin(x_j - x_i) over the sources of buffer b for this thread's receiver
   auto sums = [&](int b) -> float {
@@ -1091,7 +1133,8 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     }
     return sum;
   };
-  // the new sine and cosine of the own receiver into buffer b of every CTA
+  // the new sine and cosine of the own receiver into buffer b of every CTA; nothing
+  // is sent once a wait of this CTA has expired (the others' waits expire too)
   auto publish = [&](uint32_t phase, int b) {
     float4 *dst = pc_smem + b * npairs;
     if (active) {
@@ -1104,8 +1147,10 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
     }
-    __syncthreads();
-    if (lane == 0 && warp < cs && warp != crank && mine > 0 && !*(volatile int *)&expired) {
+    stop = __syncthreads_or(late);
+    if (stop) return;
+    ++sent;
+    if (lane == 0 && warp < cs && warp != crank && mine > 0) {
       const uint32_t from = smem_u32(dst + first);
       asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                        cluster_map(from, (uint32_t)warp)),
@@ -1113,18 +1158,17 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
                    : "memory");
     }
   };
-  // the other CTAs' part of the stage; once a wait has expired the CTA records it
-  // and runs to its end without waiting or sending (the others' waits expire too)
+  // the other CTAs' part of the stage
   auto receive = [&]() {
     if (bytes > 0) {
       const uint32_t bar = bar0 + 8 * (stage & 1u), parity = (stage >> 1) & 1u;
-      const bool ok = !*(volatile int *)&expired && mbar_wait_bounded(bar, parity, A.wait_ns);
-      if (!ok) {
-        expired = 1;
+      if (!mbar_wait_bounded(bar, parity, A.wait_ns)) {
+        late = true;
         atomicOr(A.err, kErrTimeout);
-      }
-      if (t == 0 && ok)
+      } else if (t == 0) {
+        ++got;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+      }
     }
     ++stage;
   };
@@ -1168,20 +1212,28 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
       b ^= 1;
     } else {
       publish(tp, 1);
+      if (stop) break;
       receive();
       const float g2 = sums(1);
       const float d = fmaf(A.sc_noise, psi, fmaf(A.kh, g1 + g2, wdt));
       th += (uint32_t)__float2int_rn(d * 4294967296.0f);
     }
     publish(th, b);
+    if (stop) break;
     if (((n + 1) & 3) == 0) draw(n + 1);  // while the others' data arrives
     receive();
   }
-  if (A.M > 0 && crank == 0) order(b, row);
+  if (A.M > 0 && crank == 0 && !stop) order(b, row);
   if (own) A.theta[base + i] = th;
-  cluster.sync();
-  // every copy has arrived, unless a wait expired: then the last ones get time to
-  if (cs > 1 && *(volatile int *)&expired) __nanosleep(200000);
+  if (cs == 1) return;
+  if (t == 0) sent_s = sent;
+  cluster_drain(late, got, bar0, &gave_up, cs, [&](uint32_t s) {
+    uint32_t miss = 0;
+    for (int q = 0; q < cs; ++q)
+      if (q != crank && *(volatile uint32_t *)cluster.map_shared_rank(&sent_s, q) <= s)
+        miss += 16u * (uint32_t)max(0, min(chunk / 2, npairs - q * chunk / 2));
+    return miss;
+  });
 }
 
 // Shared memory and cluster size of the kernel's launches (not under capture).

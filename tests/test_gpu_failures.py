@@ -122,3 +122,29 @@ def test_every_injected_allocation_failure_reports_no_memory(kind):
         ens.run_josephson(0, 300, x, v, xo, vo, wo, so)
         assert np.all(np.isfinite(ens.observables()["mean"]))
         ens.close()
+
+
+@pytest.mark.parametrize("steps", [1, 2, 5])
+@pytest.mark.parametrize("euler", [False, True])
+def test_pairwise_cluster_waits_that_expire_in_the_last_stages(steps, euler):
+    """Limits around the length of a stage: some CTAs of a cluster give up in the
+    last stage or the one before it while others receive everything, and all
+    stay until what was sent has arrived.  The run reports SDE_ERR_TIMEOUT or is
+    the reference bit for bit, and so is the next one."""
+    N, R = 1000, 8
+    ensure_built()
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=R, seed=34)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, 2.0, 0.05, 0.01, 4, sample_every=1,
+                                flags=sde.SDE_FLAG_EULER if euler else 0)
+    assert ens.tuning()[0] == 512 and ens.tuning()[2] > 1
+    phi_ref, r_ref, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+    for ns in (1, 200, 500, 1000, 1500, 2000, 3000, 5000):
+        ens.set_wait_limit(ns)
+        try:
+            phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+            assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
+        except sde.SDEError as e:
+            assert e.status == sde.SDE_ERR_TIMEOUT
+        ens.set_wait_limit(0)
+        phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+        assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
