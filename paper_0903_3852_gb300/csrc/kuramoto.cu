@@ -436,15 +436,16 @@ __device__ __forceinline__ void cluster_drain(bool late, uint32_t got, uint32_t 
 // while it is read, and the receiver has re-armed the buffer's mbarrier
 // (after its own stage s wait, before its stage s + 1 sends) before any
 // stage s + 2 store can arrive.  Waits are bounded (A.wait_ns, one second by
-// default): on expiry the kernel records
-// kErrTimeout, leaves the step loop (warp-uniformly) and meets the others at
-// the final cluster barrier.
+// default): on expiry the kernel records kErrTimeout, leaves the step loop
+// (warp-uniformly) and meets the others in cluster_drain.
 template <int OPT, bool FULL>
 __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurArgs A) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ int2 slots[2][32];
   __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ int gave_up;           // some CTA of the cluster did
+  __shared__ uint32_t sent_s[16];   // stages each warp sent
   const int cs = (int)cluster.num_blocks();
   const int crank = (int)cluster.block_rank();
   const int nwarps = blockDim.x >> 5;
@@ -452,6 +453,7 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
   const int nslots = cs * nwarps;  // <= 32, checked by the host
   const uint32_t bytes = (uint32_t)nslots * 8u;
   if (threadIdx.x == 0) {
+    gave_up = 0;
     // each phase is armed (arrival + expected bytes) before any store of it can
     // arrive: stages 0 and 1 here, stage s + 2 right after stage s completes
     // (no sender reaches stage s + 2 before this CTA has sent stage s + 1)
@@ -490,9 +492,10 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
   const uint32_t rslot1 = lane < cs ? cluster_map(my_slot1, (uint32_t)lane) : 0u;
   const uint32_t rbar0 = lane < cs ? cluster_map(smem_u32(&mbar[0]), (uint32_t)lane) : 0u;
   const uint32_t rbar1 = lane < cs ? cluster_map(smem_u32(&mbar[1]), (uint32_t)lane) : 0u;
-  uint32_t stage = 0;
-  bool failed = false;  // warp-uniform
+  uint32_t stage = 0, got = 0;  // stages sent by this warp; received, as thread 0 counts them
+  bool failed = false;          // warp-uniform
   auto cluster_sum = [&](int S, int C) -> float2 {
+    if (failed) return make_float2(0.0f, 0.0f);  // a stage is sent only after the one before it was received
     const int2 part = warp_qsum(S, C);
     const int b = (int)(stage & 1u);
     const uint32_t parity = (stage >> 1) & 1u;
@@ -507,8 +510,10 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
       failed = true;
       if (lane == 0) atomicOr(A.err, kErrTimeout);
     }
-    if (threadIdx.x == 0 && ok)  // arm this buffer's next phase (stage + 2)
+    if (threadIdx.x == 0 && ok) {  // arm this buffer's next phase (stage + 2)
+      ++got;
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    }
     const int2 v = lane < nslots ? slots[b][lane] : make_int2(0, 0);
     ++stage;
     return unquant(warp_qsum(v.x, v.y));
@@ -588,7 +593,15 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
 #pragma unroll
   for (int k = 0; k < OPT; ++k)
     if (valid[k]) A.theta_out[base + oid[k]] = th[k];
-  cluster.sync();  // no CTA leaves while remote stores into it may be in flight
+  if (lane == 0) sent_s[warp] = stage;
+  cluster_drain(failed, got, smem_u32(&mbar[0]), &gave_up, cs, [&](uint32_t s) {
+    uint32_t miss = 0;
+    for (int q = 0; q < cs; ++q) {
+      const volatile uint32_t *sent = cluster.map_shared_rank(sent_s, q);
+      for (int w = 0; w < nwarps; ++w) miss += sent[w] <= s ? 8u : 0u;
+    }
+    return miss;
+  });
 }
 
 // ---- mean field over the whole grid ------------------------------------

@@ -148,3 +148,24 @@ def test_pairwise_cluster_waits_that_expire_in_the_last_stages(steps, euler):
         ens.set_wait_limit(0)
         phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
         assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 5])
+def test_async_meanfield_waits_that_expire_in_the_last_stages(steps):
+    """The same for the mean field's asynchronous exchange."""
+    N, R = 4096, 8
+    ensure_built()
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=R, seed=35)
+    kw = dict(sample_every=1, block_threads=256, cluster_ctas=4, flags=sde.SDE_FLAG_ASYNC_EXCHANGE)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_MEANFIELD, N, R, 2.0, 0.05, 0.01, 4, **kw)
+    phi_ref, r_ref, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+    for ns in (1, 200, 400, 600, 800, 1000, 1500, 2000):
+        ens.set_wait_limit(ns)
+        try:
+            phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+            assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
+        except sde.SDEError as e:
+            assert e.status == sde.SDE_ERR_TIMEOUT
+        ens.set_wait_limit(0)
+        phi, r, _ = kur_run(ens, w["phi0"], w["omega"], 0, steps)
+        assert np.array_equal(phi, phi_ref) and np.array_equal(r, r_ref)
