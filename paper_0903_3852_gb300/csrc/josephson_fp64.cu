@@ -12,13 +12,13 @@
 //
 // What bounds it: the FP64 pipe, one warp instruction per 16 cycles and SM.  So
 // the transcendental functions are written in as few FP64 operations as their
-// arguments allow (ranges known, no special cases): 14 for a force, 16 for a
-// Gaussian, 8 for the rest of a step, 52 per step against 86 with the
-// library's cospi, log, sqrt and sincospi; the drive term, the tables of the
-// logarithm and of the angle's sine and cosine are formed once per block, and
-// integers become doubles through their bit patterns.  Blocks are sized so that
-// every SM holds the same number of paths.  65536 paths, 400 steps: 4.96 -> 2.64
-// ms (9.9e9 path-steps/s); 3000 paths 2.48 -> 0.69 ms.
+// arguments allow (ranges known, no special cases) without losing accuracy to the
+// library's: 11 for a force, 18 for a Gaussian, 9 for the rest of a step, 49 per
+// step against 86 with the library's cospi, log, sqrt and sincospi; the drive
+// term and the tables are put into shared memory once per block, integers become
+// doubles through their bit patterns, comparisons are made on high words.
+// Blocks are sized so that every SM holds the same number of paths.  65536 paths,
+// 400 steps: 4.96 -> 2.54 ms (1.03e10 path-steps/s).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -45,52 +45,133 @@ struct JJ64Args {
   PhiloxKeys keys;
 };
 
-// Tables of a block (shared memory).
+// Tables, each value as a sum hi + lo: hi rounded to a multiple of 2^-43 (2^-52
+// for the angles), lo the rest.  Formed by the compiler in integers, as
+// multiples of 2^-96 and 2^-62, so they are the same wherever it runs.
 constexpr int kLogTable = 128;   // leading 7 bits of a mantissa
 constexpr int kAngleTable = 64;  // sixty-fourths of a turn
 struct Tables64 {
-  double inv[kLogTable];     // c_i ~ 1 / (1 + (i + 1/2) / 128), at most 14 bits; c_0 = 1, c_127 = 1/2
-  double two_log[kLogTable]; // 2 ln c_i
-  double exponent[25];       // -2 (e - 24) ln 2
-  double cs[kAngleTable], sn[kAngleTable];
+  double inv[kLogTable];        // c_i ~ 1 / (1 + (i + 1/2) / 128), at most 14 bits; c_0 = 1, c_127 = 1/2
+  double2 two_log[kLogTable];   // 2 ln c_i
+  double2 exponent[26];         // -2 (e - 24) ln 2 (the last is padding)
+  double2 cs[kAngleTable], sn[kAngleTable];
 };
+
+// c_i in units of 2^-13.
+constexpr int log_scale(int i) {
+  return i == 0 ? 8192 : (i == kLogTable - 1 ? 4096 : (8192 * 512 + 257 + 2 * i) / (2 * (257 + 2 * i)));
+}
+
+struct HiLo {
+  double hi, lo;
+};
+
+// 2 ln(k / 8192), k <= 8192: -4 atanh(y), y = (8192 - k) / (8192 + k) <= 1/3, by its series.
+constexpr HiLo two_log_of(int k) {
+  const unsigned __int128 num = 8192 - k, den = 8192 + k;
+  unsigned __int128 term = (num << 98) / den, sum = 0;  // 4 y^(2 q + 1) 2^96
+  for (int q = 0; term != 0; ++q) {
+    sum += term / (2 * q + 1);
+    term = (term * num / den) * num / den;
+  }
+  const long long hi = (long long)((sum + ((unsigned __int128)1 << 52)) >> 53);
+  const long long lo = (long long)((__int128)sum - ((__int128)hi << 53));
+  return {-(double)hi / (double)(1ll << 43), -(double)lo / (double)(1ll << 48) / (double)(1ll << 48)};
+}
+
+// cos(2 pi i / 64) 2^62, i in [0, 16], by half angles: cos^2(x / 2) = (1 + cos x) / 2.
+constexpr long long cos64_of(int i) {
+  if (i == 0) return 1ll << 62;
+  if (i == 16) return 0;
+  const long long c = 2 * i <= 16 ? cos64_of(2 * i) : -cos64_of(32 - 2 * i);
+  const unsigned __int128 sq = (unsigned __int128)((unsigned long long)((1ll << 62) + c)) << 61;
+  unsigned long long r = 0;
+  for (int bit = 62; bit >= 0; --bit) {
+    const unsigned long long t = r | (1ull << bit);
+    if ((unsigned __int128)t * t <= sq) r = t;
+  }
+  return (long long)r;
+}
+
+constexpr HiLo split62(long long v) {
+  const long long hi = (v + 512) >> 10;
+  return {(double)hi / (double)(1ll << 52), (double)(v - hi * 1024) / (double)(1ll << 62)};
+}
+
+struct TableData {
+  double inv[kLogTable], log_hi[kLogTable], log_lo[kLogTable];
+  double cos_hi[kAngleTable / 4 + 1], cos_lo[kAngleTable / 4 + 1];  // a quarter turn
+};
+
+constexpr TableData make_tables() {
+  TableData t{};
+  for (int i = 0; i < kLogTable; ++i) {
+    t.inv[i] = log_scale(i) / 8192.0;
+    const HiLo v = two_log_of(log_scale(i));
+    t.log_hi[i] = v.hi;
+    t.log_lo[i] = v.lo;
+  }
+  for (int i = 0; i <= kAngleTable / 4; ++i) {
+    const HiLo v = split62(cos64_of(i));
+    t.cos_hi[i] = v.hi;
+    t.cos_lo[i] = v.lo;
+  }
+  return t;
+}
+
+__device__ constexpr TableData kTables = make_tables();
+
+// cos(2 pi i / 64) of a whole turn from the quarter.
+__device__ __forceinline__ double2 cos_entry(int i) {
+  const int h = i & 31, q = h <= 16 ? h : 32 - h;
+  const bool neg = (h > 16) != ((i & 32) != 0);
+  const double hi = kTables.cos_hi[q], lo = kTables.cos_lo[q];
+  return neg ? make_double2(-hi, -lo) : make_double2(hi, lo);
+}
 
 __device__ __forceinline__ void fill_tables64(Tables64 &t) {
   for (int i = threadIdx.x; i < kLogTable; i += blockDim.x) {
-    const double c = i == 0 ? 1.0 : (i == kLogTable - 1 ? 0.5 : rint(8192.0 / (1.0 + (i + 0.5) / kLogTable)) / 8192.0);
-    t.inv[i] = c;
-    t.two_log[i] = 2.0 * log(c);
+    t.inv[i] = kTables.inv[i];
+    t.two_log[i] = make_double2(kTables.log_hi[i], kTables.log_lo[i]);
   }
-  for (int i = threadIdx.x; i < 25; i += blockDim.x) t.exponent[i] = (24 - i) * (2.0 * log(2.0));
-  for (int i = threadIdx.x; i < kAngleTable; i += blockDim.x) sincospi(i / 32.0, &t.sn[i], &t.cs[i]);
+  // from -2 ln(1/2) = -two_log[127]; 24 times a multiple of 2^-43 below 2 is exact
+  for (int i = threadIdx.x; i < 25; i += blockDim.x)
+    t.exponent[i] = make_double2((i - 24) * kTables.log_hi[kLogTable - 1], (i - 24) * kTables.log_lo[kLogTable - 1]);
+  for (int i = threadIdx.x; i < kAngleTable; i += blockDim.x) {
+    t.cs[i] = cos_entry(i);
+    t.sn[i] = cos_entry((i + 48) & (kAngleTable - 1));
+  }
 }
 
 // -2 ln(m 2^-24) for m in [1, 2^24].  m = 2^e f, f in [1, 2); with c_i from the
 // leading bits of f, z = f c_i - 1 is exact and in (-0.004, 1/128], and
-// -2 ln u = -2 (e - 24) ln 2 + 2 ln c_i - 2 ln(1 + z), the last as z times a
-// degree-6 polynomial (interpolation at the Chebyshev nodes of the interval,
-// within 1e-20).  c_0 = 1 and c_127 = 1/2 make the table terms cancel for u
-// near 1, so the result keeps its relative accuracy there; u = 1 gives 0.
+// -2 ln u = -2 (e - 24) ln 2 + 2 ln c_i - 2 z + z^2 r(z), r of degree 5
+// (interpolation at the Chebyshev nodes of the interval, within 1e-20).  The
+// first three terms are multiples of 2^-43 (z of 2^-36) and their sum is exact;
+// the rest is small, so the result is rounded once: within 0.54 ulp over all m
+// (0.52 for a correctly rounded logarithm doubled; 25 without the low parts).
+// c_0 = 1 and c_127 = 1/2 make the table terms cancel for u near 1; u = 1 gives 0.
 __device__ __forceinline__ double minus2_log24(uint32_t m, const Tables64 &t) {
   const uint32_t bits = __float_as_uint((float)m);  // exact: 24 bits
   const uint32_t mant = bits & 0x7FFFFFu;
   const int e = (int)(bits >> 23) - 127, i = (int)(mant >> 16);
   const double f = __hiloint2double((int)(0x3FF00000u | (mant >> 3)), (int)(mant << 29));
   const double z = fma(f, t.inv[i], -1.0);
-  double q = -0.2828473837233479;
-  q = fma(q, z, 0.3333355763843714);
-  q = fma(q, z, -0.4000000966277093);
-  q = fma(q, z, 0.5000000000732646);
-  q = fma(q, z, -0.6666666666658018);
-  q = fma(q, z, 0.9999999999999994);
-  q = fma(q, z, -2.0);
-  return fma(z, q, t.exponent[e] + t.two_log[i]);
+  const double2 te = t.exponent[e], tl = t.two_log[i];
+  double r = -0.2828473837233479;
+  r = fma(r, z, 0.3333355763843714);
+  r = fma(r, z, -0.4000000966277093);
+  r = fma(r, z, 0.5000000000732646);
+  r = fma(r, z, -0.6666666666658018);
+  r = fma(r, z, 0.9999999999999994);
+  return fma(-2.0, z, te.x + tl.x) + fma(z * z, r, te.y + tl.y);
 }
 
 // Box-Muller in FP64 from the same 24-bit uniforms as the FP32 path.  The
 // angle 2 pi (j + 1) 2^-24 is the nearest sixty-fourth of a turn plus b, |b| <=
 // pi / 64: sin b and cos b from short polynomials (interpolation at the
-// Chebyshev nodes, within 3e-17), combined with the table by angle addition.
+// Chebyshev nodes, within 3e-17), combined with the table by angle addition,
+// the largest term last: sine and cosine within 8.3e-17.
 __device__ __forceinline__ void box_muller64(uint32_t w0, uint32_t w1, const Tables64 &t, double &z0, double &z1) {
   const double rho = sqrt_goldschmidt(minus2_log24((w0 >> 8) + 1u, t));
   const int j = (int)(w1 >> 8) + 1;
@@ -106,32 +187,47 @@ __device__ __forceinline__ void box_muller64(uint32_t w0, uint32_t w1, const Tab
   double pc = fma(b2, -0.001388799249796147, 0.041666666585670434);
   pc = fma(b2, pc, -0.4999999999999892);
   const double cm1 = b2 * pc;  // cos b - 1
-  const double C = t.cs[q & (kAngleTable - 1)], S = t.sn[q & (kAngleTable - 1)];
-  z0 = rho * fma(C, cm1, fma(-S, sb, C));
-  z1 = rho * fma(S, cm1, fma(C, sb, S));
+  const double2 C = t.cs[q & (kAngleTable - 1)], S = t.sn[q & (kAngleTable - 1)];
+  z0 = rho * (C.x + fma(C.x, cm1, fma(-S.x, sb, C.y)));
+  z1 = rho * (S.x + fma(S.x, cm1, fma(C.x, sb, S.y)));
 }
 
-// A - 2 pi cos(2 pi x).
+// A - 2 pi cos(2 pi x).  With d = |x - rint(x)|, the cosine is an even polynomial
+// of d (d < 1/8) or of 1/2 - d (d >= 3/8, with the other sign), or an odd one of
+// 1/4 - d; each of these differences is exact.  Coefficients: least squares over
+// [0, 1/8] of the function less its leading FP64 constant.  Without A within
+// 9.6e-16 (RMS 2.8e-16; 2 pi times a correctly rounded cosine 1.04e-15, 3.2e-16).
+// The selections between the polynomials cost no FP64 issue.
 __device__ __forceinline__ double jj_force64(double x, double A) {
-  const double b = 0.25 - fabs(x - rint(x));
-  const double s = b * b;
-  double p = -0.6339542652986321;  // -2 pi times the coefficients of sin2pi64_poly
-  p = fma(p, s, 4.509654417248789);
-  p = fma(p, s, -24.00131607613064);
-  p = fma(p, s, 94.84243079652464);
-  p = fma(p, s, -264.2625677114168);
-  p = fma(p, s, 481.9571309735275);
-  p = fma(p, s, -512.7409032401533);
-  p = fma(p, s, 259.7575760906731);
-  p = fma(p, s, -39.47841760435743);
-  return fma(b, p, A);
+  const double d = fabs(x - rint(x));
+  const int hi = __double2hiint(d);  // compared as an integer: 1/8 and 3/8 have no low bits
+  const bool far = hi >= 0x3FD80000, odd = hi >= 0x3FC00000 && !far;
+  const double t = (odd ? 0.25 : (far ? 0.5 : 0.0)) - d;
+  const double s = t * t;
+  double p = odd ? -23.72575465200541 : -49.07454462882556;
+  p = fma(p, s, odd ? 94.8355962158329 : 166.02855703122987);
+  p = fma(p, s, odd ? -264.2624799289404 : -378.52811281837717);
+  p = fma(p, s, odd ? 481.95713035499193 : 536.9410175504025);
+  p = fma(p, s, odd ? -512.7409032378275 : -408.02624637851824);
+  p = fma(p, s, odd ? 259.75757609066903 : 124.02510672119752);
+  p = fma(p, s, odd ? -39.47841760435743 : -6.283185307179586);
+  return fma(odd ? t : (far ? -1.0 : 1.0), p, A);
+}
+
+// cos(2 pi k / P), k in [0, P], from an argument of at most an eighth of a turn,
+// whose rounding is that much smaller than k / P's.
+__device__ __forceinline__ double drive64(int k, int P) {
+  const int m = k <= P - k ? k : P - k;
+  if (8 * m < P) return cospi((double)(2 * m) / (double)P);
+  if (8 * m <= 3 * P) return sinpi((double)(P - 4 * m) / (double)(2 * P));
+  return -cospi((double)(P - 2 * m) / (double)P);
 }
 
 __global__ void __launch_bounds__(512) jj64_kernel(const JJ64Args A) {
   extern __shared__ double drive_s[];  // [P]: a cos(2 pi k / P) + f
   __shared__ Tables64 tab;
   for (int k = threadIdx.x; k < A.P; k += blockDim.x)
-    drive_s[k] = fma(A.a, cos2pi64((double)k / (double)A.P), A.f);
+    drive_s[k] = fma(A.a, drive64(k, A.P), A.f);
   fill_tables64(tab);
   __syncthreads();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -162,3 +162,52 @@ def test_fp64_invalid_arguments_and_nonfinite():
     # a state that overflows: the error word gets the non-finite bit
     x2, v2, _, err = _run64(dict(FIG2, gamma=1e300), 100, 20, 1, np.zeros(8), np.ones(8))
     assert err == 1
+
+
+def _one_step(D, x0, n):
+    """v after the single step n from v = 0 with dt = 1, no drive and a vanishing
+    gamma: the force at x0 (D = 0), or the step's Gaussian where the force is
+    zero (x0 = 1/4, sqrt(2 gamma D dt) = 1)."""
+    pt = dict(gamma=2.0 ** -600, a=0.0, omega=2 * np.pi, f=0.0, D=D)
+    x = torch.from_numpy(x0).cuda()
+    v = torch.zeros_like(x)
+    sde.josephson_run_fp64(pt, 1, 2, 21, n, n + 1, x, v, x, v, point_index=4)
+    return v.cpu().numpy().astype(np.longdouble)
+
+
+def test_fp64_force_is_as_exact_as_a_rounded_cosine():
+    """-2 pi cos(2 pi x) against extended precision.  2 pi times a correctly
+    rounded cosine errs by at most 2^-54 2 pi (the cosine) + 2.5e-16 (2 pi) +
+    2^-51 (the product) = 1.04e-15, RMS 3.2e-16: the kernel's force may not err more."""
+    ensure_built()
+    rng = np.random.default_rng(8)
+    x = np.concatenate([rng.uniform(0, 1, 300000), rng.uniform(-900, 900, 50000), np.arange(-8, 9) / 8.0])
+    two_pi = 2 * np.arccos(np.longdouble(-1))
+    r = x.astype(np.longdouble) - np.rint(x)
+    err = np.abs(_one_step(0.0, x, 0) + two_pi * np.cos(two_pi * r)).astype(np.float64)
+    print("fp64 force: max %.3e rms %.3e" % (err.max(), np.sqrt(np.mean(err ** 2))))
+    assert err.max() <= 1.04e-15 and np.sqrt(np.mean(err ** 2)) <= 3.2e-16
+
+
+def test_fp64_gaussians_are_as_exact_as_rounded_functions():
+    """The two Gaussians of a pair of words against extended precision.  With
+    every function correctly rounded the radius errs relatively by 2^-54 (the
+    logarithm, halved by the root) + 2^-53 (the root), a product by 2^-53 more, the
+    sines by 2^-54 absolutely: sqrt(z0^2 + z1^2) within 4e-16 of its value, and an RMS
+    error of 8.1e-17 per Gaussian, 5 % above it allowed."""
+    ensure_built()
+    n = 1 << 19
+    ctr = torch.zeros((n, 4), dtype=torch.int32, device="cuda")
+    ctr[:, 1], ctr[:, 2], ctr[:, 3] = torch.arange(n, device="cuda"), 4, 1
+    w = (sde.philox4x32_10(ctr, 21).cpu().numpy().astype(np.int64) & 0xFFFFFFFF)
+    u = ((w >> 8) + 1).astype(np.longdouble) / 2 ** 24
+    two_pi = 2 * np.arccos(np.longdouble(-1))
+    rho = np.sqrt(-2 * np.log(u[:, 0]))
+    ref = rho * np.cos(two_pi * u[:, 1]), rho * np.sin(two_pi * u[:, 1])
+    z = [_one_step(2.0 ** 599, np.full(n, 0.25), k) for k in range(2)]
+    rms = max(float(np.sqrt(np.mean((a - b) ** 2))) for a, b in zip(z, ref))
+    ok = rho > 0
+    rel = np.abs(np.sqrt(z[0] ** 2 + z[1] ** 2)[ok] / rho[ok] - 1).astype(np.float64)
+    print("fp64 Gaussians: rms %.3e, radius max %.3e" % (rms, rel.max()))
+    assert rms <= 8.5e-17 and rel.max() <= 4e-16
+    assert all(abs(a[~ok]).max(initial=0) == 0 for a in z)
