@@ -846,7 +846,14 @@ __global__ void __launch_bounds__(kMfgThreads, MODE == 3 ? 4 : (MODE == 2 ? 8 : 
 // FMAs on the sines and cosines of the two phases (each within 7e-8, from the
 // fixed-point phases; the kernel that writes a phase writes its pair too).
 // Both products of a term enter the receiver's running sum one after the
-// other, so the sum stays as small as the sum of the sines and rounds like it.
+// other, and in between the sum carries s_j c_i, which rounds at 6e-8 s_j c_i
+// however small the term.  So the phases are taken relative to one near
+// oscillator 0's: the frame drops out of every difference, and in a population
+// that is nearly in step the sines are as small as the terms (spread 1e-3 rad:
+// 1e-9 per source, 4e-8 in a fixed frame).  Where the phases are spread the terms
+// themselves are of order 1.  The frame of a stage's phases is oscillator 0's phase
+// one stage earlier, which every block can read while they are written, moved on
+// by its own frequency where the stage is a whole step.
 //
 // What bounds it: the FMA pipe, once the shared loads are kept below it.  Two
 // sources share a packed FP32 FMA (a receiver's sums over even and odd sources
@@ -866,6 +873,11 @@ struct PairShape {
   int threads() const { return 32 * s; }
 };
 
+// A step at oscillator 0's own frequency, in units of the phases.
+__device__ __forceinline__ uint32_t frame_step(float omega0, float wscale) {
+  return (uint32_t)__float2int_rn(omega0 * wscale * 4294967296.0f);
+}
+
 template <int RPT>
 __device__ __forceinline__ void pair_terms(const float4 &src, const float (&si)[RPT], const float (&ci)[RPT],
                                            float2 (&acc)[RPT]) {
@@ -880,7 +892,8 @@ __device__ __forceinline__ void pair_terms(const float4 &src, const float (&si)[
 // phases theta, writes theta~ and the first-stage coupling sum g1; STAGE 1
 // (corrector) takes the sums over theta~ and writes the new theta.  STAGE 2
 // is PROG2's UpdateRHS: the sums over theta, stored in g1 for the
-// AdvanceSystem kernel of the Euler-Maruyama scheme.
+// AdvanceSystem kernel of the Euler-Maruyama scheme, and that kernel's frame in
+// theta~'s first place.
 template <int STAGE, int RPT, int S>
 __global__ void __launch_bounds__(32 * S) kur_pairwise_stage(const KurPairArgs A) {
   constexpr int THREADS = 32 * S, RPC = RPT * 32;
@@ -937,6 +950,7 @@ __global__ void __launch_bounds__(32 * S) kur_pairwise_stage(const KurPairArgs A
   __syncthreads();
   const uint2 key = seed_to_key(A.seed);
   const int64_t n = A.n;
+  if (STAGE == 2 && blockIdx.x == 0 && threadIdx.x == 0) A.theta_t[base] = A.theta[base] + frame_step(A.omega[base], A.wscale);
   for (int rl = threadIdx.x; rl < RPC; rl += THREADS) {
     const int64_t i = i0 + rl;
     if (i >= N) break;
@@ -953,29 +967,30 @@ __global__ void __launch_bounds__(32 * S) kur_pairwise_stage(const KurPairArgs A
     const float psi = pick4(z, (int)(n & 3));
     const float wdt = A.omega[gi] * A.wscale;
     uint32_t th = A.theta[gi];
+    const uint32_t frame = STAGE == 0 ? A.theta[base] + frame_step(A.omega[base], A.wscale) : A.theta_t[base];
     float sn, cs;
     if (STAGE == 0) {
       const float d1 = fmaf(A.sc_noise, psi, fmaf(A.kc, g, wdt));
       th += (uint32_t)__float2int_rn(d1 * 4294967296.0f);
       A.theta_t[gi] = th;
       A.g1[gi] = g;
-      sincos_turns(th, sn, cs);
+      sincos_turns(th - frame, sn, cs);
       A.sc_t[gi] = make_float2(sn, cs);
     } else {
       const float d = fmaf(A.sc_noise, psi, fmaf(A.kh, A.g1[gi] + g, wdt));
       th += (uint32_t)__float2int_rn(d * 4294967296.0f);
       A.theta[gi] = th;
-      sincos_turns(th, sn, cs);
+      sincos_turns(th - frame, sn, cs);
       A.sc[gi] = make_float2(sn, cs);
     }
   }
 }
 
 // sin and cos of every phase, the sources of the first pairwise stage.
-__global__ void kur_sincos_kernel(const uint32_t *theta, float2 *sc, int64_t n) {
+__global__ void kur_sincos_kernel(const uint32_t *theta, float2 *sc, int64_t N, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     float sn, cs;
-    sincos_turns(theta[i], sn, cs);
+    sincos_turns(theta[i] - theta[i / N * N], sn, cs);
     sc[i] = make_float2(sn, cs);
   }
 }
@@ -1076,11 +1091,13 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   const int i = crank * chunk + t;  // this thread's receiver
   const bool own = t < chunk && i < N;
   const bool active = (t & ~31) < chunk;  // this warp has receivers
+  uint32_t frame = A.theta[base];  // of the sines and cosines sent next (see pair_terms)
+  const uint32_t step0 = frame_step(A.omega[base], A.wscale);
   // all sources of theta; pairs beyond N stay zero in both buffers
   for (int p = t; p < npairs; p += kPcThreads) {
     float s0 = 0.0f, c0 = 0.0f, s1 = 0.0f, c1 = 0.0f;
-    if (2 * p < N) sincos_turns(A.theta[base + 2 * p], s0, c0);
-    if (2 * p + 1 < N) sincos_turns(A.theta[base + 2 * p + 1], s1, c1);
+    if (2 * p < N) sincos_turns(A.theta[base + 2 * p] - frame, s0, c0);
+    if (2 * p + 1 < N) sincos_turns(A.theta[base + 2 * p + 1] - frame, s1, c1);
     pc_smem[p] = make_float4(s0, s1, -c0, -c1);
     pc_smem[npairs + p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
@@ -1110,6 +1127,12 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   auto sums = [&](int b) -> float {
     const float4 *src = pc_smem + b * npairs;
     const int l = lane & 7;
+    // The next frame: oscillator 0's phase in this buffer, to a first order that
+    // follows it within a few stages, and a step on if the phases sent next are.
+    // Every CTA holds the same bits of its sine.
+    const float s0 = src[0].x;
+    frame += (uint32_t)__float2int_rn(683565276.0f * (src[0].z < 0.0f ? s0 : copysignf(1.0f, s0)));  // 2^32 / (2 pi)
+    if (EULER || b == 0) frame += step0;
     for (int g = 0; g < groups; ++g) {
       float si[8], ci[8];
       float2 acc[8];
@@ -1152,7 +1175,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     float4 *dst = pc_smem + b * npairs;
     if (active) {
       float sn, cs_;
-      sincos_turns(phase, sn, cs_);
+      sincos_turns(phase - frame, sn, cs_);
       if (!own) sn = cs_ = 0.0f;
       const float s1 = __shfl_xor_sync(0xffffffffu, sn, 1), c1 = __shfl_xor_sync(0xffffffffu, cs_, 1);
       if ((t & 1) == 0 && t / 2 < mine) {
@@ -1335,7 +1358,7 @@ __global__ void kur_advance_euler_kernel(const KurPairArgs A, int64_t R) {
     const uint32_t th = A.theta[gi] + (uint32_t)__float2int_rn(d * 4294967296.0f);
     A.theta[gi] = th;
     float sn, cs;
-    sincos_turns(th, sn, cs);
+    sincos_turns(th - A.theta_t[rep * A.N], sn, cs);
     A.sc[gi] = make_float2(sn, cs);
   }
 }
@@ -2051,7 +2074,7 @@ sde_status kuramoto_run(KuramotoCtx *k, const sde_run_desc *r, cudaStream_t s, c
     a.seed = k->seed;
     const PairShape shape = pair_shape(k->N, k->R, k->sm_count);
     if (r->n_end > r->n_begin) {
-      kur_sincos_kernel<<<cvt_grid, 256, 0, s>>>(k->theta, k->pair_sc, NR);
+      kur_sincos_kernel<<<cvt_grid, 256, 0, s>>>(k->theta, k->pair_sc, k->N, NR);
       SDE_CUDA_TRY(cudaGetLastError());
     }
     int64_t sample = 0;

@@ -250,3 +250,46 @@ def test_forward_tiles_are_independent(members, n_hidden, n_in, B):
     m.use_tensor_cores(False)
     ref, _ = m.forward(X)
     assert (mean - ref).abs().max().item() <= 2e-3 * max(1.0, ref.abs().max().item())
+
+
+def _turns_step(th, K, omega, dt, euler):
+    """One step without noise on fixed-point phases, the sums in FP64."""
+    def drift(t):
+        d = (t[:, None, :] - t[:, :, None] + 2 ** 31) % 2 ** 32 - 2 ** 31
+        return omega * dt / (2 * np.pi) + K * dt / (2 * np.pi) * np.sin(2 * np.pi / 2 ** 32 * d).mean(2)
+
+    def add(t, d):
+        return (t + np.rint(d * 2.0 ** 32).astype(np.int64)) % 2 ** 32
+
+    d1 = drift(th)
+    return add(th, d1) if euler else add(th, 0.5 * (d1 + drift(add(th, d1))))
+
+
+@pytest.mark.parametrize("N,R", [(1000, 3), (1024, 60), (2500, 1), (300, 400)])
+@pytest.mark.parametrize("euler", [False, True])
+@pytest.mark.parametrize("spread", [0.0, 1e-5])
+def test_pairwise_terms_of_a_population_in_step(N, R, euler, spread):
+    """Phases within `spread` of one another, strong coupling and a common
+    frequency, one SRK2 or two Euler steps: the coupling per source, as read off
+    the result, is within 8e-9 of the FP64 sums.  Its parts: the phases come back
+    in FP32 (6e-8 below 2 rad, over K dt = 50: 1.2e-9), a fixed-point unit of the
+    first stage grown by the second (1.5e-9 K dt, over K dt), and the sums' own
+    rounding, 6e-8 of sines below the frame's lag (0.05 rad) and the spread
+    (3e-9).  A population wholly in step turns by the same number of units
+    everywhere."""
+    ensure_built()
+    K, dt, omega, steps = 5000.0, 0.01, 5.0, 2 if euler else 1
+    rng = np.random.default_rng(N)
+    phi0 = (1.0 + spread * rng.uniform(-1, 1, (R, N))).astype(np.float32)
+    om = np.full((R, N), omega, np.float32)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, K, 0.0, dt, 3, sample_every=1,
+                                flags=sde.SDE_FLAG_EULER if euler else 0)
+    phi, _, _ = kur_run(ens, phi0, om, 0, steps)
+    if spread == 0.0:
+        assert (phi == phi[0, 0]).all()
+    th = np.rint(phi0[:2].astype(np.float64) / (2 * np.pi) * 2 ** 32).astype(np.int64)
+    for _ in range(steps):
+        th = _turns_step(th, K, omega, dt, euler)
+    err = np.abs(angle_diff(phi[:2], th * (2 * np.pi / 2 ** 32))).max() / (K * dt)
+    print("N=%d R=%d euler=%d spread %g: %.2e per source" % (N, R, euler, spread, err))
+    assert err <= 8e-9
