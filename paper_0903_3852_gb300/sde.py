@@ -198,7 +198,7 @@ class Ensemble:
         _check(lib().sde_create(ctypes.byref(cfg), ctypes.byref(h)))
         self._h = h
         self.cfg = cfg
-        self._rows = 0  # observable rows of the last run
+        self._rows = 0  # observable rows of the last run made through this object
 
     @classmethod
     def josephson(cls, points, paths, steps, seed, steps_per_period=200,
@@ -263,7 +263,7 @@ class Ensemble:
         r.phi_in_dev, r.phi_out_dev, r.omega_dev = _ptr(phi_in), _ptr(phi_out), _ptr(omega)
         r.r_out_dev = _ptr(r_out)
         _check(lib().sde_run_ensemble(self._h, ctypes.byref(r), _stream(stream)))
-        M = self.sample_every
+        M = self.cfg.sample_every
         self._rows = -(-(n_end - n_begin) // M) + 1 if M > 0 else 0
 
     def position_histogram(self, w, w_lo, nbins, stream=None):
@@ -290,9 +290,12 @@ class Ensemble:
         with fields mean, var, se, count, t."""
         n = ctypes.c_int64()
         cap = self._rows if capacity is None else capacity
-        rows = np.empty(cap, dtype=_OBS_DTYPE)
-        _check(lib().sde_observables(self._h, rows.ctypes.data_as(ctypes.POINTER(ObsRow)), cap, ctypes.byref(n)))
-        return rows[:min(cap, n.value)]
+        while True:
+            rows = np.empty(max(cap, 0), dtype=_OBS_DTYPE)
+            _check(lib().sde_observables(self._h, rows.ctypes.data_as(ctypes.POINTER(ObsRow)), cap, ctypes.byref(n)))
+            if capacity is not None or n.value <= cap:
+                return rows[:min(cap, n.value)]
+            cap = n.value  # a run made through the C functions had more rows than this object's last one
 
     def tuning(self):
         """(threads per block, paths or oscillators per thread, CTAs per replica)."""
