@@ -492,10 +492,10 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
   const uint32_t rslot1 = lane < cs ? cluster_map(my_slot1, (uint32_t)lane) : 0u;
   const uint32_t rbar0 = lane < cs ? cluster_map(smem_u32(&mbar[0]), (uint32_t)lane) : 0u;
   const uint32_t rbar1 = lane < cs ? cluster_map(smem_u32(&mbar[1]), (uint32_t)lane) : 0u;
-  uint32_t stage = 0, got = 0;  // stages sent by this warp; received, as thread 0 counts them
-  bool failed = false;          // warp-uniform
+  uint32_t stage = 0;    // stages sent by this warp
+  bool failed = false;   // a wait of the last of them expired (warp-uniform)
+  bool mine_ok = true;   // not this thread's
   auto cluster_sum = [&](int S, int C) -> float2 {
-    if (failed) return make_float2(0.0f, 0.0f);  // a stage is sent only after the one before it was received
     const int2 part = warp_qsum(S, C);
     const int b = (int)(stage & 1u);
     const uint32_t parity = (stage >> 1) & 1u;
@@ -508,12 +508,11 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
     const bool ok = mbar_wait_bounded(bar, parity, A.wait_ns);
     if (__any_sync(0xffffffffu, !ok)) {
       failed = true;
+      mine_ok = ok;
       if (lane == 0) atomicOr(A.err, kErrTimeout);
     }
-    if (threadIdx.x == 0 && ok) {  // arm this buffer's next phase (stage + 2)
-      ++got;
+    if (threadIdx.x == 0 && ok)  // arm this buffer's next phase (stage + 2)
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    }
     const int2 v = lane < nslots ? slots[b][lane] : make_int2(0, 0);
     ++stage;
     return unquant(warp_qsum(v.x, v.y));
@@ -539,6 +538,7 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
         C += quant(cs_[k]);
       }
       float2 sc = cluster_sum(S, C);
+      if (failed) continue;  // a stage is sent only after the one before it was received
       if (A.M > 0 && sample_ctr == 0) {
         if (threadIdx.x == 0 && crank == 0 && A.r_out) {
           const double Sd = sc.x, Cd = sc.y;
@@ -594,6 +594,7 @@ __global__ void __launch_bounds__(512, 1) kur_meanfield_async_kernel(const KurAr
   for (int k = 0; k < OPT; ++k)
     if (valid[k]) A.theta_out[base + oid[k]] = th[k];
   if (lane == 0) sent_s[warp] = stage;
+  const uint32_t got = failed && !mine_ok ? stage - 1 : stage;  // stages thread 0 received
   cluster_drain(failed, got, smem_u32(&mbar[0]), &gave_up, cs, [&](uint32_t s) {
     uint32_t miss = 0;
     for (int q = 0; q < cs; ++q) {
@@ -1080,6 +1081,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   __shared__ float2 red_r[32];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ int gave_up;       // some CTA of the cluster did
+  __shared__ int late_s;        // a thread of this CTA did
   __shared__ uint32_t sent_s;   // stages this CTA sent
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1110,7 +1112,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
   const uint32_t bytes = 16u * (uint32_t)(min(npairs, cs * chunk / 2) - mine);
   const uint32_t bar0 = smem_u32(&mbar[0]);
   if (t == 0) {
-    gave_up = 0;
+    gave_up = late_s = 0;
 #pragma unroll
     for (int q = 0; q < 2; ++q) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * q) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1119,9 +1121,8 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 8 * q), "r"(bytes) : "memory");
   }
   cluster.sync();  // every CTA's buffers and barriers are there before the first copy into them
-  uint32_t stage = 0, sent = 0, got = 0;  // got: stages received, as thread 0 counts them
-  bool late = false;                      // a wait of this thread expired
-  bool stop = false;                      // a wait of this CTA did, known to all its threads
+  uint32_t stage = 0, got = 0;  // stages sent; received, as thread 0 counts them
+  bool stop = false;                      // a wait of this CTA expired, as all its threads see it
 
   // sum_j sin(x_j - x_i) over the sources of buffer b for this thread's receiver
   auto sums = [&](int b) -> float {
@@ -1162,6 +1163,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
       }
     }
     __syncthreads();
+    stop = *(volatile int *)&late_s != 0;  // written before this barrier or after publish's
     float sum = 0.0f;
     if (t < chunk) {
 #pragma unroll
@@ -1169,8 +1171,8 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     }
     return sum;
   };
-  // the new sine and cosine of the own receiver into buffer b of every CTA; nothing
-  // is sent once a wait of this CTA has expired (the others' waits expire too)
+  // the new sine and cosine of the own receiver into buffer b of every CTA; not
+  // called once a wait of this CTA has expired (the others' waits expire too)
   auto publish = [&](uint32_t phase, int b) {
     float4 *dst = pc_smem + b * npairs;
     if (active) {
@@ -1183,9 +1185,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
     }
-    stop = __syncthreads_or(late);
-    if (stop) return;
-    ++sent;
+    __syncthreads();
     if (lane == 0 && warp < cs && warp != crank && mine > 0) {
       const uint32_t from = smem_u32(dst + first);
       asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -1199,7 +1199,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     if (bytes > 0) {
       const uint32_t bar = bar0 + 8 * (stage & 1u), parity = (stage >> 1) & 1u;
       if (!mbar_wait_bounded(bar, parity, A.wait_ns)) {
-        late = true;
+        *(volatile int *)&late_s = 1;
         atomicOr(A.err, kErrTimeout);
       } else if (t == 0) {
         ++got;
@@ -1241,6 +1241,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
     }
     const float psi = pick4(z, (int)(n & 3));
     const float g1 = sums(b);
+    if (stop) break;
     const float d1 = fmaf(A.sc_noise, psi, fmaf(A.kc, g1, wdt));
     const uint32_t tp = th + (uint32_t)__float2int_rn(d1 * 4294967296.0f);
     if (EULER) {
@@ -1248,22 +1249,22 @@ __global__ void __launch_bounds__(kPcThreads, 1) kur_pair_cluster_kernel(const P
       b ^= 1;
     } else {
       publish(tp, 1);
-      if (stop) break;
       receive();
       const float g2 = sums(1);
+      if (stop) break;
       const float d = fmaf(A.sc_noise, psi, fmaf(A.kh, g1 + g2, wdt));
       th += (uint32_t)__float2int_rn(d * 4294967296.0f);
     }
     publish(th, b);
-    if (stop) break;
     if (((n + 1) & 3) == 0) draw(n + 1);  // while the others' data arrives
     receive();
   }
-  if (A.M > 0 && crank == 0 && !stop) order(b, row);
+  if (A.M > 0 && crank == 0 && !stop) order(b, row);  // meaningless after an expired wait, like theta
   if (own) A.theta[base + i] = th;
   if (cs == 1) return;
-  if (t == 0) sent_s = sent;
-  cluster_drain(late, got, bar0, &gave_up, cs, [&](uint32_t s) {
+  if (t == 0) sent_s = stage;
+  __syncthreads();
+  cluster_drain(*(volatile int *)&late_s != 0, got, bar0, &gave_up, cs, [&](uint32_t s) {
     uint32_t miss = 0;
     for (int q = 0; q < cs; ++q)
       if (q != crank && *(volatile uint32_t *)cluster.map_shared_rank(&sent_s, q) <= s)
