@@ -18,7 +18,8 @@
 //     quarter where a CTA has one tile and both groups share it);
 //     the element arithmetic runs on packed FP32 pairs;
 //   warp 16, one thread: TMA producer streaming the BF16 square-layer weights
-//     through a 2-slot ring of 256 x 64 chunks (K-major, 128-byte swizzle);
+//     through a ring of 256 x 64 chunks (K-major, 128-byte swizzle), two slots, or
+//     four where a CTA has one tile and needs no second one's activations;
 //   warp 17, one thread: MMA issuer, M = 128, N = 256, K = 16 per
 //     instruction, for the groups in turn, each group's accumulator (256 FP32
 //     columns) in its half of tensor memory, which warp 17 allocates and frees.
@@ -57,7 +58,8 @@ constexpr int BM = 128;            // points per CTA
 constexpr int KCH = H / 64;        // 64-element K chunks per square layer
 constexpr int A_CHUNK = BM * 128;  // bytes of one A chunk: 128 rows x 128 B
 constexpr int W_CHUNK = H * 128;   // bytes of one weight chunk: 256 rows x 128 B
-constexpr int RING = 2;            // weight chunks in flight
+constexpr int RING = 2;            // weight chunks in flight with two tiles of activations
+constexpr int RING_SOLO = 4;       // with one, in the same shared memory
 constexpr int GROUPS = 2;          // tiles in flight
 constexpr int GROUP_WARPS = 8;
 constexpr int GROUP_THREADS = GROUP_WARPS * 32;
@@ -66,6 +68,7 @@ constexpr int PROD_WARP = EPI_WARPS;
 constexpr int MMA_WARP = EPI_WARPS + 1;
 constexpr int THREADS = EPI_WARPS * 32 + 64;
 constexpr int SMEM_BYTES = GROUPS * KCH * A_CHUNK + RING * W_CHUNK + 1024;  // + alignment slack
+static_assert(KCH * A_CHUNK + RING_SOLO * W_CHUNK <= GROUPS * KCH * A_CHUNK + RING * W_CHUNK, "one tile's layout fits");
 constexpr int QUARTER = H / 4;  // columns of one partial sum of the output layer
 constexpr int MAX_IN = 8;
 constexpr int MAX_HH = 7;
@@ -159,14 +162,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     mlp_fwd_tc_kernel(const __grid_constant__ CUtensorMap mapW, const Args a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t *Wr = smem + GROUPS * KCH * A_CHUNK;     // RING slots of [H][128 B]; before them KCH chunks of [BM][128 B] per group
+  constexpr int ring = SOLO ? RING_SOLO : RING;
+  uint8_t *Wr = smem + (SOLO ? 1 : GROUPS) * KCH * A_CHUNK;  // ring slots of [H][128 B]; before them KCH chunks of [BM][128 B] per group
   __shared__ __align__(16) float w0s[MAX_IN * H];  // [k][n]: output pairs adjacent
   __shared__ __align__(16) float b0s[H];
   __shared__ __align__(16) float bhs[MAX_HH * H];
   __shared__ __align__(16) float wos[H];
   __shared__ float part[GROUPS][4][BM];
-  __shared__ __align__(8) uint64_t full_bar[RING];
-  __shared__ __align__(8) uint64_t empty_bar[RING];
+  __shared__ __align__(8) uint64_t full_bar[ring];
+  __shared__ __align__(8) uint64_t empty_bar[ring];
   __shared__ __align__(8) uint64_t acc_bar[GROUPS];
   __shared__ __align__(8) uint64_t abuf_bar[GROUPS];
   __shared__ __align__(8) uint64_t drain_bar;
@@ -181,7 +185,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int n_mine = blockIdx.x < tiles ? (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < RING; ++s) {
+    for (int s = 0; s < ring; ++s) {
       tc::mbar_init(&full_bar[s], 1);
       tc::mbar_init(&empty_bar[s], 1);
     }
@@ -224,8 +228,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       int issued = 0;
       int i0 = 0, l = 0, g = 0, kc = 0;  // pair's first tile, layer, group, chunk
       for (int c = 0; c < nchunks; ++c) {
-        const int s = c % RING;
-        const uint32_t ph = (uint32_t)(c / RING) & 1u;
+        const int s = c % ring;
+        const uint32_t ph = (uint32_t)(c / ring) & 1u;
         if (!tc::mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag)) break;
         tc::mbar_arrive_expect_tx(&full_bar[s], (uint32_t)W_CHUNK);
         tc::tma_load_2d(Wr + s * W_CHUNK, &mapW, &full_bar[s], kc * 64, (member * n_hh + l) * H);
@@ -245,8 +249,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       // every load issued has landed before the CTA may end (older ones were
       // consumed by completed MMAs)
       volatile int no_abort = 0;
-      for (int c = issued - RING < 0 ? 0 : issued - RING; c < issued; ++c)
-        tc::mbar_wait(&full_bar[c % RING], (uint32_t)(c / RING) & 1u, &no_abort);
+      for (int c = issued - ring < 0 ? 0 : issued - ring; c < issued; ++c)
+        tc::mbar_wait(&full_bar[c % ring], (uint32_t)(c / ring) & 1u, &no_abort);
     }
     __syncwarp();
   } else if (warp == MMA_WARP) {
@@ -267,8 +271,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc::tmem_fence_after();
             const uint8_t *Ag = smem + g * KCH * A_CHUNK;
             for (int kc = 0; kc < KCH; ++kc, ++c) {
-              const int s = c % RING;
-              if (!tc::mbar_wait(&full_bar[s], (uint32_t)(c / RING) & 1u, &abort_flag)) {
+              const int s = c % ring;
+              if (!tc::mbar_wait(&full_bar[s], (uint32_t)(c / ring) & 1u, &abort_flag)) {
                 ok = false;
                 break;
               }
