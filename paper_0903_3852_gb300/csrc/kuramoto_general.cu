@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <utility>
 
 #include "kuramoto.h"
@@ -90,14 +91,26 @@ __global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__
     ok[u] = i < N;
     const int64_t ii = ok[u] ? i : 0;
     const int64_t idx = r * N + ii;
-    ps[u] = plane_sum(Dt, (2 * r) * N + ii, planes, 2 * a.NR);
-    pc[u] = plane_sum(Dt, (2 * r + 1) * N + ii, planes, 2 * a.NR);
+    ps[u] = Dt[(2 * r) * N + ii];
+    pc[u] = Dt[(2 * r + 1) * N + ii];
     th[u] = a.theta[idx];
     th_s[u] = STAGE == 0 ? th[u] : a.theta_t[idx];
     om[u] = a.omega[idx];
     g1[u] = STAGE == 1 ? a.g1[idx] : 0.0f;
     psi[u] = (STAGE == 0 && a.fresh) ? 0.0f : tc::psi_plane(a, a.n >> 2, (int)(a.n & 3))[idx];
   }
+  // the other planes of the FP32 GEMM's K shares; a loop among the loads above would
+  // keep them apart (BF16, 1024 x 64: 0.5 us per stage)
+  if (std::is_same<T, float>::value)
+    for (int p = 1; p < planes; ++p) {
+      const float *D = Dt + p * 2 * a.NR;
+#pragma unroll
+      for (int u = 0; u < kStageIlp; ++u) {
+        const int64_t ii = ok[u] ? i0 + u * 256 : 0;
+        ps[u] += D[(2 * r) * N + ii];
+        pc[u] += D[(2 * r + 1) * N + ii];
+      }
+    }
 #pragma unroll
   for (int u = 0; u < kStageIlp; ++u) {
     if (!ok[u]) continue;
