@@ -18,6 +18,15 @@ __device__ __forceinline__ double sin2pi64_poly(double s) {
   return fma(p, s, 6.283185307179586);
 }
 
+// cos(2 pi k / P), k in [0, P], inv4P = 1 / (4 P): sin(2 pi b) with b = 1/4 - min(k, P -
+// k) / P, whose numerator is an exact integer.  Within 2.7e-16 for P up to 4096 (a
+// correctly rounded cosine of the rounded quotient k / P: 3.6e-16).
+__device__ __forceinline__ double cos_ratio64(int k, int P, double inv4P) {
+  const int m = k <= P - k ? k : P - k;
+  const double b = (double)(P - 4 * m) * inv4P;
+  return b * sin2pi64_poly(b * b);
+}
+
 // sqrt(L), L >= 0 (0 below 2^-1022), by Goldschmidt's iteration from the hardware's
 // approximate reciprocal square root and a final correction by the residual L -
 // g^2.  The test for zero and the halving are done on the high word, off the FP64

@@ -1042,13 +1042,8 @@ struct NoallocArgs {
   Moments *partials;  // device address of g_noalloc_partials
 };
 
-// cos(2 pi k / P) rounded to FP32, k in [0, P]: sin(2 pi b) with b = 1/4 - min(k, P
-// - k) / P, whose numerator is an exact integer.
-__device__ __forceinline__ float drive_entry(int k, int P, double inv4P) {
-  const int kk = k <= P - k ? k : P - k;
-  const double b = (double)(P - 4 * kk) * inv4P;
-  return (float)(b * sin2pi64_poly(b * b));
-}
+// cos(2 pi k / P) rounded to FP32, k in [0, P].
+__device__ __forceinline__ float drive_entry(int k, int P, double inv4P) { return (float)cos_ratio64(k, P, inv4P); }
 
 // ILP paths per thread (2 or 4, packed pairs as in the persistent kernels), the moments taken per 32 paths as with one path per thread: the
 // same arithmetic and unit decomposition as the plain schedule with one path

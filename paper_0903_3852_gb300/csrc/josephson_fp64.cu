@@ -31,11 +31,17 @@
 namespace sde {
 namespace {
 
+// Threads of a block at least: a warp alone would take longer over the tables than
+// over a few steps.
+constexpr int kMinThreads64 = 128;
+
 struct JJ64Args {
   double gamma, a, f;
   double dt, h, s;  // dt, dt / 2, sqrt(2 gamma D dt)
+  double inv4P;     // 1 / (4 P)
   int32_t P;
   uint32_t point;   // noise counter word c2
+  int32_t block_paths;  // paths per block, one per thread; the other threads help with the tables
   int64_t n_paths;
   int64_t n_begin, n_end;
   int64_t wstart;   // the window holds state indices (wstart, S]
@@ -214,24 +220,15 @@ __device__ __forceinline__ double jj_force64(double x, double A) {
   return fma(odd ? t : (far ? -1.0 : 1.0), p, A);
 }
 
-// cos(2 pi k / P), k in [0, P], from an argument of at most an eighth of a turn,
-// whose rounding is that much smaller than k / P's.
-__device__ __forceinline__ double drive64(int k, int P) {
-  const int m = k <= P - k ? k : P - k;
-  if (8 * m < P) return cospi((double)(2 * m) / (double)P);
-  if (8 * m <= 3 * P) return sinpi((double)(P - 4 * m) / (double)(2 * P));
-  return -cospi((double)(P - 2 * m) / (double)P);
-}
-
 __global__ void __launch_bounds__(512) jj64_kernel(const JJ64Args A) {
   extern __shared__ double drive_s[];  // [P]: a cos(2 pi k / P) + f
   __shared__ Tables64 tab;
   for (int k = threadIdx.x; k < A.P; k += blockDim.x)
-    drive_s[k] = fma(A.a, drive64(k, A.P), A.f);
+    drive_s[k] = fma(A.a, cos_ratio64(k, A.P, A.inv4P), A.f);
   fill_tables64(tab);
   __syncthreads();
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= A.n_paths) return;
+  const int64_t j = (int64_t)blockIdx.x * A.block_paths + threadIdx.x;
+  if ((int)threadIdx.x >= A.block_paths || j >= A.n_paths) return;
   double x = A.x_in[j], v = A.v_in[j];
   double vs = A.vsum_in ? A.vsum_in[j] : 0.0;
   int32_t k = (int32_t)(A.n_begin % A.P);
@@ -276,7 +273,7 @@ __global__ void __launch_bounds__(512) jj64_kernel(const JJ64Args A) {
   if (A.vsum_out) A.vsum_out[j] = vs;
 }
 
-// Threads per block for n paths: the SMs' shares of the paths rounded up to
+// Paths per block for n paths: the SMs' shares of the paths rounded up to
 // whole warps, in as few blocks per SM as hold them (the busiest SM has at most
 // 32 paths per block more than its share: 65536 paths in blocks of 256 left
 // some SMs with two blocks and some with one).
@@ -335,10 +332,11 @@ extern "C" sde_status sde_josephson_run_fp64(const sde_jj_point *point, int32_t 
   int dev = 0, sms = 0;
   SDE_CUDA_TRY(cudaGetDevice(&dev));
   SDE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int block = jj64_block(n_paths, sms);
+  a.block_paths = jj64_block(n_paths, sms);
+  a.inv4P = 1.0 / (4.0 * (double)steps_per_period);
   const size_t smem = sizeof(double) * (size_t)steps_per_period;
-  const unsigned grid = (unsigned)((n_paths + block - 1) / block);
-  jj64_kernel<<<grid, block, smem, (cudaStream_t)stream>>>(a);
+  const unsigned grid = (unsigned)((n_paths + a.block_paths - 1) / a.block_paths);
+  jj64_kernel<<<grid, std::max(a.block_paths, kMinThreads64), smem, (cudaStream_t)stream>>>(a);
   SDE_CUDA_TRY(cudaGetLastError());
   return SDE_OK;
 }
