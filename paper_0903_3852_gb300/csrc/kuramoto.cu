@@ -898,7 +898,7 @@ __device__ __forceinline__ void pair_terms(const float4 &src, const float (&si)[
 template <int STAGE, int RPT, int S>
 __global__ void __launch_bounds__(32 * S) kur_pairwise_stage(const KurPairArgs A) {
   constexpr int THREADS = 32 * S, RPC = RPT * 32;
-  constexpr int TILE = 1024;  // sources
+  constexpr int TILE = S == 1 ? 64 : 1024;  // sources
   constexpr int NP = TILE / 2 / THREADS;
   __shared__ float4 src_s[TILE / 2];
   __shared__ float red[S * RPC];
@@ -1001,8 +1001,12 @@ __global__ void kur_sincos_kernel(const uint32_t *theta, float2 *sc, int64_t N, 
 // SM's schedulers one warp of every block (with two, 1024 blocks on 152 SMs
 // left 3 warps on one scheduler and 4 on another: 92 us per stage at N = 4096,
 // 64 replicas, against 76 us).  Below about twelve warps per SM more slices
-// take the place of receivers per thread.
+// take the place of receivers per thread.  A replica of at most 32 oscillators is
+// a single warp's, in a block of little shared memory: with many of them a stage
+// lasts as long as its blocks take to come and go (N = 2, 30,000 replicas: 53 us per
+// stage with {8, 4}, 19 so; N = 33, 30,000: 69 with {8, 4}).
 PairShape pair_shape(int64_t N, int64_t R, int sm_count) {
+  if (N <= 32) return {1, 1};
   const int64_t want = (int64_t)sm_count * 12;
   if ((N + 255) / 256 * R * 4 >= want) return {8, 4};
   if ((N + 127) / 128 * R * 8 >= want) return {4, 8};
@@ -1016,6 +1020,8 @@ cudaError_t launch_pairwise(const KurPairArgs &a, int64_t R, const PairShape &p,
     kur_pairwise_stage<STAGE, 8, 4><<<grid, p.threads(), 0, s>>>(a);
   else if (p.s == 8)
     kur_pairwise_stage<STAGE, 4, 8><<<grid, p.threads(), 0, s>>>(a);
+  else if (p.s == 1)
+    kur_pairwise_stage<STAGE, 1, 1><<<grid, p.threads(), 0, s>>>(a);
   else
     kur_pairwise_stage<STAGE, 2, 16><<<grid, p.threads(), 0, s>>>(a);
   return cudaGetLastError();

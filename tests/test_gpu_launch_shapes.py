@@ -293,3 +293,14 @@ def test_pairwise_terms_of_a_population_in_step(N, R, euler, spread):
     err = np.abs(angle_diff(phi[:2], th * (2 * np.pi / 2 ** 32))).max() / (K * dt)
     print("N=%d R=%d euler=%d spread %g: %.2e per source" % (N, R, euler, spread, err))
     assert err <= 8e-9
+
+
+@pytest.mark.parametrize("N,R", [(1, 3000), (8, 1000), (31, 1500), (32, 900), (33, 900)])
+@pytest.mark.parametrize("euler", [False, True])
+def test_pairwise_many_small_replicas(N, R, euler):
+    """A warp per replica up to 32 oscillators, and one more: the bounds of
+    test_pairwise_shapes_match_mean_field."""
+    test_pairwise_shapes_match_mean_field(N, R, euler)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, 2.0, 0.05, 0.01, 3,
+                                flags=sde.SDE_FLAG_EULER if euler else 0)
+    assert (ens.tuning()[:2] == (32, 1)) == (N <= 32)
