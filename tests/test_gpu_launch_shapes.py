@@ -304,3 +304,81 @@ def test_pairwise_many_small_replicas(N, R, euler):
     ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, R, 2.0, 0.05, 0.01, 3,
                                 flags=sde.SDE_FLAG_EULER if euler else 0)
     assert (ens.tuning()[:2] == (32, 1)) == (N <= 32)
+
+
+@pytest.mark.parametrize("N,block,cluster,flags,opt", [
+    (700, 256, 1, 0, 3), (600, 128, 1, 0, 5), (750, 128, 1, 0, 6), (1400, 256, 2, 0, 3), (2399, 128, 4, 0, 5),
+    (3000, 128, 4, 0, 6), (4600, 128, 8, 0, 5), (1400, 256, 2, sde.SDE_FLAG_ASYNC_EXCHANGE, 3),
+    (2399, 128, 4, sde.SDE_FLAG_ASYNC_EXCHANGE, 5), (3000, 128, 4, sde.SDE_FLAG_ASYNC_EXCHANGE, 6),
+    (4600, 128, 8, sde.SDE_FLAG_ASYNC_EXCHANGE, 5)])
+def test_odd_counts_per_thread_equal_a_power_of_two(N, block, cluster, flags, opt):
+    """The mean field with 3, 5 and 6 oscillators per thread against 8 or 16 in one
+    CTA: the sums are exact integers, so phases and r(t) agree bit for bit."""
+    ensure_built()
+    w = inputs.kuramoto_uniform(n_osc=N, replicas=3, seed=N)
+    kw = dict(K=2.0, D=0.05, dt=0.01, seed=3, sample_every=3)
+    got = []
+    for shape in (dict(block_threads=block, cluster_ctas=cluster, flags=flags),
+                  dict(block_threads=(-(-N // 16) + 31) // 32 * 32, cluster_ctas=1)):
+        ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_MEANFIELD, N, 3, **kw, **shape)
+        got.append((ens.tuning(), *kur_run(ens, w["phi0"], w["omega"], 2, 13)[:2]))
+    assert got[0][0][:2] == (block, opt) and got[1][0][1] in (8, 16)
+    assert np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][2], got[1][2])
+
+
+@pytest.mark.parametrize("shift_in,shift_out", [(0, 0), (1, 0), (0, 3), (2, 1)])
+def test_phases_of_any_range_and_alignment(shift_in, shift_out):
+    """A run of no steps returns every phase reduced to [0, 2 pi): the fixed-point
+    turns are those of the FP64 quotient within one unit (2^-32 turn), the result
+    their FP32 rounding (2.4e-7 below 2 pi, one unit 1.5e-9)."""
+    ensure_built()
+    rng = np.random.default_rng(5)
+    phi = np.concatenate([rng.uniform(0, 8, 20000), rng.uniform(-60, 60, 20000), rng.uniform(-1e-9, 1e-9, 200),
+                          [0.0, -0.0, 1e-30, 1e-12, -1e-12, 3.0, 6.2831850, 6.2831855, 7.9999995, 8.0, -8.0, 1e4, -1e4,
+                           1e7]]).astype(np.float32)
+    phi = np.concatenate([phi, phi[: 3 - phi.size % 4]])  # not a multiple of four
+    N = phi.size
+    src, dst = torch.zeros(N + shift_in, device="cuda"), torch.full((N + shift_out + 1,), -1.0, device="cuda")
+    src[shift_in:] = torch.from_numpy(phi)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_PAIRWISE, N, 1, 1.0, 0.0, 0.01, 1, sample_every=0)
+    omega = torch.zeros(N, device="cuda")
+    ens.run_kuramoto(4, 4, src[shift_in:].view(1, N), dst[shift_out:shift_out + N].view(1, N), omega.view(1, N))
+    out = dst.cpu().numpy().astype(np.float64)
+    assert (out[:shift_out] == -1).all() and out[-1] == -1
+    out = out[shift_out:shift_out + N]
+    t = phi.astype(np.float64) / (2 * np.pi)
+    ref = (t - np.floor(t)) * (2 * np.pi)
+    assert out.min() >= 0.0 and out.max() <= np.float32(2 * np.pi)
+    assert np.abs(angle_diff(out, ref)).max() <= 2.4e-7 + 1.5e-9
+    near = np.abs(phi) < 1e-3
+    assert np.abs(angle_diff(out[near & (phi >= 0)], ref[near & (phi >= 0)])).max() <= 1.5e-9
+
+
+@pytest.mark.parametrize("N,R,tn", [(8, 3, 1), (136, 7, 1), (264, 64, 2), (520, 33, 2), (512, 100, 3), (1000, 33, 3),
+                                    (264, 200, 5), (512, 400, 7), (2000, 25, 7), (1496, 64, 8)])
+def test_fp32_gemm_errs_like_fp32(N, R, tn):
+    """Every count of columns per thread.  Along a chain of N FMAs whose terms
+    change sign at random the partial sums grow like sqrt(k): RMS error 0.15 2^-24
+    sum|K| whatever N, ten times that allowed; the sines (2^-23) enter as
+    independent errors of the terms, 2^-24 sum|K| / sqrt(N), six times that.
+    (Operands rounded to BF16 or TF32 would err by 2^-8 or 2^-11 of that.)"""
+    ensure_built()
+    w = inputs.kuramoto_general(n_osc=N, replicas=R, seed=N)
+    ens = sde.Ensemble.kuramoto(sde.SDE_KURAMOTO_GENERAL_FP32, N, R, 0.0, 0.02, 0.005, 1)
+    assert ens.tuning()[1] == 8 * tn
+    K = torch.from_numpy(w["Kmat"]).cuda()
+    ens.set_coupling(K)
+    phi = torch.from_numpy(w["phi0"]).cuda()
+    got = ens.coupling(phi).double()
+    x, Kt = phi.double(), K.double().t()
+    s, c = torch.sin(x), torch.cos(x)
+    err = ((got - (c * (s @ Kt) - s * (c @ Kt))).abs() / K.double().abs().sum(1)).max().item() * 2 ** 24
+    print("N=%d R=%d: %.2f x 2^-24 sum|K|, bound %.2f" % (N, R, err, 1.5 + 6 / math.sqrt(N)))
+    assert err <= 1.5 + 6 / math.sqrt(N)
+
+
+def test_members_train_in_uneven_groups():
+    """Three members whose batches fill the activation rows two at a time: the
+    last group is one member (the comparison of
+    test_members_train_together_as_alone)."""
+    test_members_train_together_as_alone(256, 2, 5, 16000, 16000)
