@@ -272,6 +272,17 @@ def host_cpu_model():
     return platform.processor() or platform.machine()
 
 
+def pairwise_launches(tuning, steps, every):
+    """Kernels one pairwise run launches: the phases' conversions in and out and
+    the observables, and either all steps in one launch (a replica per cluster:
+    512 threads, one oscillator per thread) or the first sines, two launches per
+    step and one per r(t) sample."""
+    if tuple(tuning[:2]) == (512, 1):
+        return 4
+    return 4 + 2 * steps + (-(-steps // every) + 1)
+
+
+
 def run_ours(args, rank, world, device):
     import torch
     from paper_0903_3852_gb300 import build as sde_build
@@ -424,7 +435,7 @@ def run_ours(args, rank, world, device):
             units = float(w["n_osc"] ** 2 * w["replicas"] * S)
             metric = "pair-terms/sec"
             flop_per_unit = COUNTED_FLOP_PAIR
-            launches_per_step = 2 * S + S // w["sample_every"] + 5
+            launches_per_step = pairwise_launches(ens.tuning(), S, w["sample_every"])
             flop_per_launch = flop_per_unit * w["n_osc"] ** 2 * w["replicas"]  # one stage launch
         cfg = {"workload": kuramoto_workload_name(args.workload, euler, w["n_osc"], w["replicas"]),
                "steps_per_bench_step": S, "K": w["K"], "D": w["D"], "dt": w["dt"],

@@ -72,7 +72,8 @@ typedef enum sde_schedule {
 /* Flags for sde_config.flags. */
 #define SDE_FLAG_NO_GRAPH 1u     /* launch kernels directly instead of replaying a graph */
 #define SDE_FLAG_TIME_KERNELS 2u /* Kuramoto pairwise / general: CUDA events around every
-                                    launch of the dominant kernel (stage / GEMM); for the
+                                    launch of the dominant kernel (stage, or the run with a
+                                    replica per cluster / GEMM); for the
                                     general coupling around the GEMMs of every 8th step only,
                                     or with SDE_FLAG_FUSED around the whole run of back-to-back
                                     GEMMs (events between GEMMs keep the next one's prologue
@@ -240,9 +241,10 @@ void sde_destroy(sde_ctx *ctx);
 /*
  * Failure detection (the paper has no counterpart).  Kernels that wait on
  * other threads through mbarriers -- the tensor-core GEMM of
- * SDE_KURAMOTO_GENERAL (its TMA producer and MMA issuer) and the Kuramoto
- * mean field with SDE_FLAG_ASYNC_EXCHANGE -- bound every such wait by a
- * limit of the GPU's nanosecond timer.  When one expires the kernel stops
+ * SDE_KURAMOTO_GENERAL (its TMA producer and MMA issuer), the Kuramoto mean
+ * field where it exchanges asynchronously (SDE_FLAG_ASYNC_EXCHANGE, or so
+ * chosen by the autotuner) and the pairwise form with a replica per cluster --
+ * bound every such wait by a limit of the GPU's nanosecond timer.  When one expires the kernel stops
  * issuing work, drains what it has issued (with waits of at most one second,
  * whatever the limit), latches SDE_ERR_TIMEOUT for the next sde_observables
  * and returns; the context stays usable.  This sets the limit for the
@@ -272,7 +274,9 @@ const char *sde_last_error(void);
    one path per thread with its noise drawn by a second warp, the shape of
    small ensembles) or
    oscillators (Kuramoto) per thread, and CTAs per replica (the thread-block
-   cluster of the mean-field kernel; 0 for the grid-wide mean field, whose
+   cluster of the mean-field kernel, or of the pairwise kernel that holds a
+   replica per cluster, which has 512 threads and one oscillator per thread;
+   0 for the grid-wide mean field, whose
    per-thread count is then the oscillators each thread strides over; for the
    general coupling's tensor-core GEMM, the CTAs per tile: 2 for the CTA-pair
    GEMM, whose per-thread value is then the D columns of a tile, 0 for the
@@ -286,7 +290,9 @@ sde_status sde_get_tuning(const sde_ctx *ctx, int32_t *block_threads, int32_t *p
  * Device time of the dominant kernel of the last run, from CUDA events
  * recorded on the run's stream around it: the persistent or per-point
  * Josephson launches, the mean-field kernel, or -- with
- * SDE_FLAG_TIME_KERNELS -- each pairwise stage launch, each GEMM launch of
+ * SDE_FLAG_TIME_KERNELS -- each pairwise stage launch (with a replica per
+ * cluster the one launch of the run, its r(t) samples included, counted as
+ * its stages: two per SRK2 step, one per Euler step), each GEMM launch of
  * every 8th step, or (SDE_FLAG_FUSED) the run's GEMMs as one block (mean_ms
  * per timed launch, total_ms summed over the timed events, launches = the
  * launches they bracket).  Without that flag the

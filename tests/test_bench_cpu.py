@@ -43,3 +43,10 @@ def test_reference_config_names_the_kuramoto_workloads():
                      "kuramoto-general-fp32": "kuramoto_general_fp32_cudacore_N8192_R256"}
     assert bench.reference_config(_args("--workload", "kuramoto-pairwise", "--euler"), "s")["workload"] == \
         "kuramoto_pairwise_N4096_R64_euler_prog2"
+
+
+def test_pairwise_launch_counts():
+    assert bench.pairwise_launches((512, 1, 16), 100, 100) == 4
+    assert bench.pairwise_launches((128, 8, 1), 10, 100) == 4 + 20 + 2
+    assert bench.pairwise_launches((512, 2, 1), 200, 100) == 4 + 400 + 3
+    assert bench.pairwise_launches((32, 1, 1), 5, 2) == 4 + 10 + 4
