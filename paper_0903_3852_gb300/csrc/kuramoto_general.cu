@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__
   }
   // the other planes of the FP32 GEMM's K shares; a loop among the loads above would
   // keep them apart (BF16, 1024 x 64: 0.5 us per stage)
-  if (std::is_same<T, float>::value)
+  if (std::is_same<T, float>::value) {
+#pragma unroll 4
     for (int p = 1; p < planes; ++p) {
       const float *D = Dt + p * 2 * a.NR;
 #pragma unroll
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(256) kg_stage_kernel(const float *__restrict__
         pc[u] += D[(2 * r + 1) * N + ii];
       }
     }
+  }
 #pragma unroll
   for (int u = 0; u < kStageIlp; ++u) {
     if (!ok[u]) continue;
