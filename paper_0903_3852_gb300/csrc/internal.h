@@ -81,8 +81,12 @@ struct JJLaunchArgs {
 // drawn by a second warp).
 constexpr int kJJWarpPairs = 21;
 // Up to this many units of 32 paths per SM that kernel is taken.  Fig. 2's
-// point, 4000 steps, against the fastest other kernel: 166 vs 430 us at 2 units
-// per SM and below, 214 vs 431 at 4, 370 vs 432 at 8, 615 vs 592 at 12.
+// point, 4000 steps, against the fastest kernel that the autotuner tries: 166 vs
+// 430 us at 2 units per SM and below, 214 vs 431 at 4, 370 vs 432 at 8, 615 vs 592
+// at 12.  Euler-Maruyama, whose chain is shorter for the same noise, 2000 steps,
+// against the fastest kernel of all: 68 vs 118 us at 2, 90 vs 119 at 4, 113 vs 148
+// at 6, 139 vs 146 at 8 (SRK2: 88 vs 151, 112 vs 152, 150 vs 187, 191 vs 185).  P =
+// 1020, with 8 KB of tables per CTA: the same within 3 %.
 constexpr int kWsUnitsPerSm = 8;
 
 // Kernel launchers (josephson.cu).

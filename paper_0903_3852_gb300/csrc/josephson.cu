@@ -496,14 +496,15 @@ __global__ void __maxnreg__(96) jj_kernel_packed4_cap96(const JJLaunchArgs A) {
 // better drawn elsewhere: a CTA holds kPairs pairs of warps, one stepping 32
 // paths, the other drawing their Gaussians ahead into a ring of two blocks of
 // 64 steps (named barriers hand the blocks over; blocks of 32 steps: 197 us
-// where 64 take 164).  Four warps per CTA, so that
-// each has a scheduler to itself.  The chain of a step is 13 FP32 operations
-// (x -> force -> v~ -> x'), 52 cycles; rint(x) on it is taken as (x + 1.5
-// 2^23) - 1.5 2^23, the same value for |x| < 2^22 in two additions where the
-// conversion unit takes longer, and a group's floor(x) from two comparisons.  The steps' values and roundings are those of
-// the one-path kernel: bit-identical.
-// 1024 paths, 20,000 steps: 0.82 ms (85 cycles per step, 73 of them the chain)
-// against 2.19 ms for the fastest kernel that draws and steps in one warp.
+// where 64 take 164).  Four warps per CTA, so that each has a scheduler to
+// itself.  The chain of a step is 13 FP32 operations (x -> force -> v~ -> x'), 52
+// cycles at 4 each; rint(x) on it is taken as (x + 1.5 2^23) - 1.5 2^23, the same
+// value for |x| < 2^22 in two additions where the conversion unit takes longer,
+// and a group's floor(x) from two comparisons.  The steps' values and roundings
+// are those of the one-path kernel: bit-identical.
+// 1024 paths, 20,000 steps: 0.80 ms (83 cycles per step: the chain, x's fold after
+// every fourth step, and the step's other operations issued in between) against
+// 2.19 ms for the fastest kernel that draws and steps in one warp.
 constexpr int kPairs = 2;               // stepping warps per CTA
 constexpr int kWsBlock = 64 * kPairs;
 constexpr uint32_t kRingGroups = 16;    // groups of 4 steps per ring block (aligned to 64 steps)

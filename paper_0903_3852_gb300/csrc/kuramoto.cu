@@ -1549,9 +1549,8 @@ cudaError_t launch_meanfield(const KurArgs &a, int block, int opt, int cs, bool 
   }
 }
 
-// Blocks per replica of the grid-wide mean field: enough oscillators per
-// thread to amortise the reduction, about eight blocks per SM in total.
-// One full wave of each kernel (resident blocks per SM from the occupancy
+// Blocks per replica of the grid-wide mean field, enough oscillators per
+// thread to amortise the reduction: one full wave of each kernel (resident blocks per SM from the occupancy
 // calculator x SMs, shared among the replicas), at most one block per
 // kMfgThreads x kMfgIlp oscillators.
 void mfg_grid_for(int64_t N, int64_t R, int sm_count, int grid[4]) {

@@ -23,12 +23,13 @@
 //   warp 17, one thread: MMA issuer, M = 128, N = 256, K = 16 per
 //     instruction, for the groups in turn, each group's accumulator (256 FP32
 //     columns) in its half of tensor memory, which warp 17 allocates and frees.
-// What bounds it: the epilogues' instruction issue (about ten instructions per
-// SiLU).  With one tile per CTA they and the MMAs alternated (issue 48 %); with
-// two a group's MMAs run during the other group's epilogue (issue 63 %, two
-// warps per scheduler while one group waits).  100,000 points of 4 members: 178
-// us against 269.  Measured beside it: 16 accumulator columns at a time with
-// the next in flight instead of 32 (215 us: half the independent work per warp).
+// What bounds it: the epilogues' instruction issue (13 instructions per
+// activation).  With one tile per CTA they and the MMAs alternated (issue 48 %);
+// with two a group's MMAs run during the other group's epilogue (issue 62 %, two
+// warps per scheduler while one group waits).  100,000 points of 4 members: 191
+// us per call against 287.  Measured beside it: 16 accumulator columns at a time
+// with the next in flight instead of 32 (a fifth slower: half the independent
+// work per warp).
 // Layer handoffs go through mbarriers per group: `abuf` (256 arrivals: the A
 // operand of the next square layer is in shared memory) and `acc`
 // (tcgen05.commit: the accumulator is complete).  Every wait is bounded by one
